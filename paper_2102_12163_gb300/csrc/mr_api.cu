@@ -71,13 +71,17 @@ void dq_inverse(int eq, double lambda, double inv[5][5]) {
         for (int j = 0; j < q; ++j) inv[i][j] = A[i][q + j];
 }
 
-int nwords_h(int l) { return l >= 5 ? (1 << (l - 5)) : 1; }
+// level and index of a cell in heap numbering
+void cell_of(uint32_t h, int &l, long long &k) {
+    l = 31 - __builtin_clz(h);
+    k = (long long)h - (1LL << l);
+}
 // compiled scheme variant of the kernels: D1Q2^n by field count, D1Q3, D1Q5
 int variant_of(int eq) { return eq == MR_EQ_SW_D1Q3 ? 4 : eq == MR_EQ_SW_D1Q5 ? 5 : nfields_of(eq); }
 // Group of the queue order an instance belongs to, most work per instance
 // first: gamma = 2, 3 (general kernel); gamma = 1 with the reconstructed
 // collision; gamma = 1 with the leaves collision and at least CW_MIN_WORDS
-// mask words per bitmask (the fast code with candidate words); the other
+// words per bit array (the fast code with candidate words); the other
 // gamma = 1 instances with the leaves collision (fast kernel, or the scalar
 // kernel when every instance of the group has one field).
 constexpr int NGROUP = 4;
@@ -242,11 +246,7 @@ static void layout(mr_ctx *c) {
         InstDesc &h = c->hdesc[i];
         int nf = nfields_of(d.eq), q = npop_of(d.eq);
         long long S = (1LL << (d.Jmax + 1)) - (1LL << d.Jmin), N = 1LL << d.Jmax;
-        int W = 0, OW = 0;
-        for (int l = d.Jmin; l <= d.Jmax; ++l) {
-            W += nwords_h(l);
-            OW += occ_words_of(l);
-        }
+        const int W = mask_words_of(d.Jmax), OW = occ_words_of(d.Jmax);
         h.Jmin = d.Jmin;
         h.Jmax = d.Jmax;
         h.bc = d.bc;
@@ -278,12 +278,12 @@ static void layout(mr_ctx *c) {
         size_t vb = c->vbytes();
         size_t oV = 0, oPhi = align_up(oV + vb * q * S), oM = align_up(oPhi + vb * q * (N + 1));
         size_t oL = align_up(oM + sizeof(uint32_t) * (size_t)mask_region_words(W, OW));
-        // every list holds distinct cells of the instance, so S entries always suffice
-        long long caps[NLIST] = {S, S, S, S};
+        // every list holds distinct leaves or distinct cells of the levels below
+        // Jmax, so N entries always suffice
         long long lo = 0;
         for (int L = 0; L < NLIST; ++L) {
             h.list_off[L] = lo;
-            lo += (caps[L] + 63) / 64 * 64;
+            lo += (N + 63) / 64 * 64;
         }
         size_t end = align_up(oL + sizeof(uint32_t) * lo);
         // pointers are filled at bind time; keep relative offsets for now
@@ -792,12 +792,13 @@ mr_status mr_get_leaves(mr_ctx *c, int inst, int *level, long *index, double *f,
     const InstDesc &h = c->hdesc[inst];
     int q = npop_of(h.eq);
     for (int i = 0; i < st.nleaf; ++i) {
-        int l = (int)(ent[i] >> KBITS);
-        long k = (long)(ent[i] & KMASK);
+        int l;
+        long long k;
+        cell_of(ent[i], l, k);
         if (level) level[i] = l;
-        if (index) index[i] = k;
+        if (index) index[i] = (long)k;
         if (f) {
-            long long cell = ((1LL << l) - (1LL << h.Jmin)) + k;
+            const long long cell = (long long)ent[i] - (1LL << h.Jmin);
             for (int hh = 0; hh < q; ++hh) f[(long)hh * cap + i] = vals[(size_t)cell * q + hh];
         }
     }
@@ -817,8 +818,7 @@ mr_status mr_get_moments(mr_ctx *c, int inst, double *m, long cap, long *count) 
     const InstDesc &h = c->hdesc[inst];
     if (m)
         for (int i = 0; i < st.nleaf; ++i) {
-            int l = (int)(ent[i] >> KBITS);
-            long long cell = ((1LL << l) - (1LL << h.Jmin)) + (ent[i] & KMASK);
+            const long long cell = (long long)ent[i] - (1LL << h.Jmin);
             if (h.eq == MR_EQ_SW_D1Q3 || h.eq == MR_EQ_SW_D1Q5) {
                 const double w[5] = {0.0, 1.0, -1.0, 2.0, -2.0};
                 double m0 = 0.0, m1 = 0.0;
@@ -862,11 +862,11 @@ mr_status mr_get_tree(mr_ctx *c, int inst, unsigned char *R) {
     std::vector<uint32_t> w(h.Wtot);
     if ((rc = c->cuda(cudaMemcpy(w.data(), h.masks + (size_t)st.cur * h.Wtot, sizeof(uint32_t) * h.Wtot, cudaMemcpyDeviceToHost), "copy")))
         return (mr_status)rc;
-    int g = 0;
-    for (int l = h.Jmin; l <= h.Jmax; ++l) {
-        long long n = 1LL << l, base = (1LL << l) - (1LL << h.Jmin);
-        for (long long k = 0; k < n; ++k) R[base + k] = (w[g + (k >> 5)] >> (k & 31)) & 1u;
-        g += nwords_h(l);
+    // cell c is in the tree when its parent c / 2 is internal; the coarsest level always is
+    const uint32_t first = 1u << h.Jmin, end = 2u << h.Jmax;
+    for (uint32_t c = first; c < end; ++c) {
+        const uint32_t p = c >> 1;
+        R[c - first] = c < 2u * first ? 1 : (unsigned char)((w[p >> 5] >> (p & 31u)) & 1u);
     }
     return MR_OK;
 }

@@ -1,19 +1,19 @@
 // mr_common.h -- data layout shared by the CUDA kernels and the host side of
 // the C ABI (include/mrlbm.h).  Internal to the library.
 //
-// Per instance the device workspace holds (all 256-byte aligned):
+// Cells are numbered as in a heap: cell k of level l is h = 2^l + k.  Per
+// instance the device workspace holds (all 256-byte aligned):
 //   V      S x q values, cell-major (the q populations of a cell contiguous),
-//          level l at cells [2^l - 2^Jmin, ...) (dense level-wise arrays:
-//          every cell of every level has a slot)
+//          cell h at (h - 2^Jmin) q (dense level-wise arrays: every cell of
+//          every level has a slot)
 //   Phi    (2^Jmax + 1) x q reconstructed boundary values, interface-major,
 //          indexed by the finest-lattice interface they belong to
-//   masks  NMASK bitmasks over all cells of all levels, 32 cells per word,
-//          level l at words [woff_l, woff_l + max(1, 2^l / 32)); then the
-//          candidate-word list of the step (Wtot entries at most) and two
-//          occupancy bitmaps (one per tree buffer) with one bit per mask
-//          word, level l at occupancy words [ooff_l, ooff_l + max(1, W_l / 32))
-//   lists  compacted cell lists (entry = level << KBITS | index), sorted by
-//          level then index; per-level segments in InstState::seg
+//   masks  NMASK bit arrays over the cells of the levels below Jmax (bit h,
+//          Wtot words each); then the candidate-word list of the step (Wtot
+//          entries) and two occupancy bit arrays (one per tree buffer) with
+//          one bit per mask word
+//   lists  compacted cell lists (entries h), sorted; per-level segments in
+//          InstState::seg
 //   state  InstState
 #pragma once
 #include <cstddef>
@@ -23,19 +23,17 @@ namespace mrg {
 
 constexpr int MAXLEV = 24;  // Jmax <= 24
 constexpr int MAXDJ = MAXLEV;
-constexpr int KBITS = 27;
-constexpr uint32_t KMASK = (1u << KBITS) - 1u;
 
 constexpr int NOT_POW2 = 1 << 20;  // InstDesc::lam_log2 of a lattice velocity that is no power of two
 
-// bitmasks; KEEP / REF (written by the details, read by the enlargement) share
-// storage with PRED / GH (written by the grading sweep, read by the list
-// compaction, which clears them for the next step)
-enum { M_R0 = 0, M_R1 = 1, M_LEAF = 2, M_PRED = 3, M_GH = 4, NMASK = 5, M_KEEP = M_PRED, M_REF = M_GH };
-// lists: internal cells of the tree, leaves, cells to predict in the transfer (A6)
-// and ghosts (S3); the even cells of the tree, whose details A2 tests, are the
-// first children of the internal cells
-enum { L_INT = 0, L_LEAF = 1, L_PRED = 2, L_GH = 3, NLIST = 4 };
+// bit arrays: the internal cells of the tree (two buffers: old and new; the
+// cells above Jmin are marked too) and the internal cells whose children the
+// details keep (KEEP) and refine (REF), clear between two adaptations
+enum { M_I0 = 0, M_I1 = 1, M_KEEP = 2, M_REF = 3, NMASK = 4 };
+// lists: internal cells of the tree, parents of the pairs to predict in the
+// transfer (A6) and of the ghost pairs (S3), leaves; the first three come with
+// segments by level
+enum { L_INT = 0, L_PRED = 1, L_GH = 2, L_LEAF = 3, NLIST = 4, NSEG = 3 };
 // phases of the persistent kernel
 enum { PH_INIT_FULL = 1, PH_INIT_STATE = 2, PH_ADAPT = 4, PH_STEP = 8, PH_FINEST = 16 };
 // device status bits
@@ -51,12 +49,12 @@ enum {
 };
 
 struct InstState {
-    int cur;                      // mask (M_R0 or M_R1) holding the current tree
+    int cur;                      // bit array (M_I0 or M_I1) holding the current tree
     int nleaf;                    // #S(Lambda) of the current tree
-    int seg[NLIST][MAXLEV + 2];   // list segments: level l at [seg[l], seg[l+1])
+    int seg[NSEG][MAXLEV + 2];    // list segments: level l >= 5 at [seg[l], seg[l+1]), the levels below it at [0, seg[5])
     int status;                   // ST_* bits
     int near_ties;                // threshold decisions within 1e-12 relative of the threshold
-    unsigned deplev[2];           // levels holding transfer / ghost cells that wait on the same list
+    unsigned deplev[2];           // levels holding transfer / ghost pairs that wait on the same list
     unsigned long long updates;   // sum over steps of #S(Lambda^{n+1})
     unsigned long long steps;
     unsigned long long passes;    // team barriers since the initial state (dependent passes)
@@ -70,8 +68,8 @@ struct InstDesc {
     int gamma;             // prediction stencil half-width (1, 2 or 3)
     int collision;         // 0: leaves collision, 1: reconstructed collision (Section 4.5)
     int lam_log2;          // k when lambda = 2^k exactly (|k| <= 16), else NOT_POW2
-    int Wtot;              // mask words over all levels
-    int OW;                // occupancy words over all levels (one bit per mask word)
+    int Wtot;              // words of a bit array over the cells of levels below Jmax
+    int OW;                // words of an occupancy array (one bit per word of a bit array)
     double eps, a, b, lam, eqp;
     double s[3];
     long long S;           // cells over all levels
@@ -96,26 +94,29 @@ struct InstDesc {
     double oms[3], eu_a, eu_b, eu_c, sw_g2;
 };
 
-// words of the mask region of an instance: NMASK bitmasks, the candidate-word
-// list and two occupancy bitmaps
+// words of a bit array over the cells h < 2^Jmax, and of its occupancy array
+#ifdef __CUDACC__
+#define MRG_HD __host__ __device__
+#else
+#define MRG_HD
+#endif
+MRG_HD inline int mask_words_of(int Jmax) { return Jmax >= 5 ? (1 << (Jmax - 5)) : 1; }
+MRG_HD inline int occ_words_of(int Jmax) { return Jmax >= 10 ? (1 << (Jmax - 10)) : 1; }
+// words of the mask region of an instance: NMASK bit arrays, the candidate-word
+// list and two occupancy arrays
 inline long long mask_region_words(int Wtot, int OW) { return (long long)(NMASK + 1) * Wtot + 2LL * OW; }
-// gamma = 1 instances with the leaves collision and at least this many mask
-// words per bitmask run their word passes over the step's candidate words
+// gamma = 1 instances with the leaves collision and at least this many words
+// per bit array run their word passes over the step's candidate words
 // (K_LARGE); smaller ones visit every word, which costs less than building the
 // candidate list (measured on the Jmax 8..14 batch and the single instances).
 // The wide-stencil and reconstructed-collision variants visit every word at
 // any size.
-constexpr int CW_MIN_WORDS = 2048;
+constexpr int CW_MIN_WORDS = 1024;
 // words of the mask region a block keeps in shared memory: without candidate
-// words the list and the occupancy bitmaps are not used
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline long long smem_region_words(int Wtot, int OW) {
+// words the list and the occupancy arrays are not used
+MRG_HD inline long long smem_region_words(int Wtot, int OW) {
     return Wtot >= CW_MIN_WORDS ? (long long)(NMASK + 1) * Wtot + 2LL * OW : (long long)NMASK * Wtot;
 }
-// occupancy words of one level: one bit per mask word of the level
-inline int occ_words_of(int l) { return l >= 10 ? (1 << (l - 10)) : 1; }
 
 // fills InstDesc's float copies of lam, eqp, s and minv (host side, after those are set)
 inline void fill_float_constants(InstDesc &h) {
@@ -173,7 +174,7 @@ struct LaunchArgs {
 // residency; K_RECOLL: gamma = 1 with the reconstructed collision, the code of
 // K_GENERAL compiled for a residency of its own (its dense reconstruction gains
 // from blocks in flight, the wide stencils from registers); K_LARGE: the code of
-// K_FAST for the instances with at least CW_MIN_WORDS mask words per bitmask,
+// K_FAST for the instances with at least CW_MIN_WORDS words per bit array,
 // whose word passes visit the step's candidate words (the code that builds
 // them stays out of the other variants, which it slowed down).
 constexpr int K_FAST = 0, K_GENERAL = 1, K_SCALAR = 2, K_RECOLL = 3, K_LARGE = 4, NKIND = 5;

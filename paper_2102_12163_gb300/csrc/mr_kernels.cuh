@@ -11,10 +11,11 @@
 //     A2  details of the pairs of the tree, threshold T, Harten flags (Sections
 //         3.2, 3.4, 4.2) -> KEEP / REF bitmasks
 //     A3  enlargement H: same-level dilation and children of REF pairs
-//     A4  grading G, sweeping fine to coarse over bitmask words (Def. Graded
-//         tree), fused with the leaf / transfer / ghost marking
-//     A5  list compaction: popcount + prefix scan over the mask words
-//     A6  data transfer: prediction of the new cells, coarse to fine
+//     A4  grading G, sweeping fine to coarse over the words of the tree (Def.
+//         Graded tree)
+//     A5  list compaction (internal cells, leaves, pairs to transfer, ghost
+//         pairs): word operations, popcount and prefix scan
+//     A6  data transfer: prediction of the new pairs, coarse to fine
 //   step (Sections 4.3, 4.5)
 //     S1  leaves collision (eq. LeavesCollision)
 //     S2  projection of the collided values up the new tree
@@ -24,8 +25,11 @@
 //     S5  compact stream (eq. AdaptiveStreamPhase) + mass audit (FP64 totals)
 //
 // The cell arrays are dense per level (every cell of every level has a slot),
-// the tree is a set of bitmasks with 32 cells per word, and every per-cell
-// phase walks a compacted list so its work is proportional to the tree.
+// the tree is a bit array over the cells, and every per-cell phase walks a
+// compacted list so its work is proportional to the tree.  A block spends most
+// of a step on the dependent instructions of its busiest warp (it issues in a
+// quarter of the cycles, its loads hit L1): fewer instructions on that path are
+// what shortens a step.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -72,20 +76,30 @@ struct V2<float> {
 };
 
 // ---------------------------------------------------------------------------
-// level geometry and bit helpers
+// cells and bitmasks in heap numbering
+//
+// Cell k of level l is h = 2^l + k: its level is 31 - clz(h), its parent h / 2,
+// its children 2h and 2h + 1, its neighbours h +- 1 (wrapped or clamped inside
+// [2^l, 2^(l+1))).  A set of cells is one bit array over h, word h / 32, so word
+// w >= 1 holds 32 cells of level 5 + log2(w), word 0 the levels 0..4, the words
+// of a level follow one another, and the children of word w's cells are words
+// 2w and 2w + 1: the same numbering again, on words.
+//
+// The tree is the set I of its internal cells (a pair of siblings is in the
+// tree exactly when its parent is internal), with the cells above Jmin marked
+// too, so that cell h is in the tree exactly when I holds h / 2.  That is half
+// the words of a set of cells, and siblings need no closing.
 
-__device__ __forceinline__ long long cell_off(int l, int Jmin) { return (1LL << l) - (1LL << Jmin); }
-__device__ __forceinline__ int nwords(int l) { return l >= 5 ? (1 << (l - 5)) : 1; }
-__device__ __forceinline__ uint32_t valid_bits(int l) {
-    return l >= 5 ? 0xFFFFFFFFu : ((1u << (1 << l)) - 1u);
+__device__ __forceinline__ int level_of(uint32_t h) { return 31 - __clz(h); }
+__device__ __forceinline__ uint32_t level_first(uint32_t h) { return 0x80000000u >> __clz(h); }
+__device__ __forceinline__ bool bit_of(const uint32_t *a, uint32_t h) { return (a[h >> 5] >> (h & 31u)) & 1u; }
+// the cell a places to the right of h on its level, whose first cell is lo
+// (bc 0 periodic: wrapped, 1 copy: the boundary cell)
+__device__ __forceinline__ uint32_t neighbour(uint32_t h, int a, uint32_t lo, int bc) {
+    if (bc == 0) return lo | ((h + (uint32_t)a) & (lo - 1u));
+    const int x = (int)h + a;
+    return (uint32_t)min(max(x, (int)lo), (int)(2u * lo - 1u));
 }
-// cell index at level l under the boundary condition (0 periodic: wrap, 1 copy: clamp)
-__device__ __forceinline__ long long wrapc(long long k, int l, int bc) {
-    long long n = 1LL << l;
-    if (bc == 0) return k & (n - 1);
-    return k < 0 ? 0 : (k >= n ? n - 1 : k);
-}
-__device__ __forceinline__ uint32_t pack(int l, long long k) { return ((uint32_t)l << KBITS) | (uint32_t)k; }
 
 // bits 0, 2, ..., 30 of x -> bits 0..15
 __device__ __forceinline__ uint32_t compact_even(uint32_t x) {
@@ -93,75 +107,63 @@ __device__ __forceinline__ uint32_t compact_even(uint32_t x) {
     x = (x | (x >> 1)) & 0x33333333u;
     x = (x | (x >> 2)) & 0x0F0F0F0Fu;
     x = (x | (x >> 4)) & 0x00FF00FFu;
-    x = (x | (x >> 8)) & 0x0000FFFFu;
-    return x;
-}
-// parent bits of two child words (a: cells 0..31, b: cells 32..63)
-__device__ __forceinline__ uint32_t fold2(uint32_t a, uint32_t b) {
-    return compact_even(a | (a >> 1)) | (compact_even(b | (b >> 1)) << 16);
+    return __byte_perm(x, 0u, 0x4420);
 }
 // 16 parent bits -> 32 child bits (both children of every parent)
 __device__ __forceinline__ uint32_t spread16(uint32_t x) {
-    x &= 0xFFFFu;
-    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = __byte_perm(x, 0u, 0x4140);
     x = (x | (x << 4)) & 0x0F0F0F0Fu;
     x = (x | (x << 2)) & 0x33333333u;
     x = (x | (x << 1)) & 0x55555555u;
     return x | (x << 1);
 }
-// close a set of cells under siblings (pairs 2p, 2p+1 never straddle a word)
-__device__ __forceinline__ uint32_t pairexpand(uint32_t x) {
-    return x | ((x & 0x55555555u) << 1) | ((x & 0xAAAAAAAAu) >> 1);
-}
-// word wp of level l-1 holding the parents of the cells set in level l (words `child`)
-__device__ __forceinline__ uint32_t fold_at(const uint32_t *child, int l, int wp) {
-    return l >= 6 ? fold2(child[2 * wp], child[2 * wp + 1]) : fold2(child[0], 0u);
-}
+// the 32 cells of word w whose parents are in p: p's word w / 2 spread
+__device__ __forceinline__ uint32_t children_word(const uint32_t *p, uint32_t w) { return spread16(p[w >> 1] >> (16u * (w & 1u))); }
 
-// Dilation by r cells of the set held in word wi of level l; get(j) returns word j
-// of that level.  Periodic: wrap; copy: cells beyond the domain are dropped.
+// word 0 of a bit array (levels 2, 3, 4 at bits 4..7, 8..15, 16..31) dilated by
+// one cell on each of its levels
+__device__ __forceinline__ uint32_t dilate_word0(uint32_t x, int bc) {
+    // the shifts, without what crosses from one level into the next
+    uint32_t d = x | ((x << 1) & ~0x00010116u) | ((x >> 1) & ~0x8000808Bu);
+    if (bc == 0)
+        d |= ((x & 0x10u) << 3) | ((x & 0x80u) >> 3) | ((x & 0x100u) << 7) | ((x & 0x8000u) >> 7) | ((x & 0x10000u) << 15) |
+             ((x & 0x80000000u) >> 15);
+    return d;
+}
+// the words beside word w >= 1 on its level (get(j): word j); 0 beyond a copy boundary
 template <class Get>
-__device__ __forceinline__ uint32_t dilate(Get get, int l, int wi, int r, int bc) {
-    uint32_t x = get(wi);
-    uint32_t out = x;
-    if (l < 5) {
-        int n = 1 << l;
-        uint32_t vb = (1u << n) - 1u;
-        for (int s = 1; s <= r; ++s) {
-            if (bc == 0)
-                out |= (((x << s) | (x >> (n - s))) & vb) | (((x >> s) | (x << (n - s))) & vb);
-            else
-                out |= ((x << s) & vb) | (x >> s);
-        }
-        return out;
-    }
-    int W = 1 << (l - 5);
-    uint32_t xl, xr;
-    if (W == 1) {
-        xl = xr = (bc == 0) ? x : 0u;
-    } else if (bc == 0) {
-        xl = get((wi - 1) & (W - 1));
-        xr = get((wi + 1) & (W - 1));
+__device__ __forceinline__ void words_beside(Get get, uint32_t w, int bc, uint32_t &xl, uint32_t &xr) {
+    const uint32_t lo = level_first(w);
+    if (bc == 0) {
+        xl = get(lo | ((w - 1u) & (lo - 1u)));
+        xr = get(lo | ((w + 1u) & (lo - 1u)));
     } else {
-        xl = wi > 0 ? get(wi - 1) : 0u;
-        xr = wi + 1 < W ? get(wi + 1) : 0u;
+        xl = w == lo ? 0u : get(w - 1u);
+        xr = w + 1u == 2u * lo ? 0u : get(w + 1u);
     }
-    for (int s = 1; s <= r; ++s) out |= (x << s) | (xl >> (32 - s)) | (x >> s) | (xr << (32 - s));
-    return out;
 }
-
-// word j of a level of W words under the boundary rule: wrapped (periodic) or
-// empty beyond the domain (copy)
-__device__ __forceinline__ uint32_t word_bc(const uint32_t *a, int j, int W, int bc) {
-    if (j < 0) return bc == 0 ? a[j + W] : 0u;
-    if (j >= W) return bc == 0 ? a[j - W] : 0u;
-    return a[j];
+// x dilated by r <= 3 cells, given the words on its left and right
+__device__ __forceinline__ uint32_t dilate_edges(uint32_t x, uint32_t xl, uint32_t xr, int r) {
+    uint32_t d = x;
+    for (int s = 1; s <= r; ++s) d |= __funnelshift_l(xl, x, s) | __funnelshift_r(x, xr, s);
+    return d;
 }
-// 4 child bits -> 2 parent bits
-__device__ __forceinline__ uint32_t fold_low2(uint32_t x) { return ((x | (x >> 1)) & 1u) | (((x >> 2) | (x >> 3)) & 1u) << 1; }
-// dilation by one cell of a word, given the neighbouring cells just outside it
-__device__ __forceinline__ uint32_t dilate1_edges(uint32_t x, bool left, bool right) {
-    return x | (x << 1) | (x >> 1) | (left ? 1u : 0u) | (right ? 0x80000000u : 0u);
+// word w of the bit array a dilated by r cells on its level
+__device__ __forceinline__ uint32_t dilate_word(const uint32_t *a, uint32_t w, int r, int bc) {
+    uint32_t x = a[w];
+    if (w == 0u) {
+        for (int s = 0; s < r; ++s) x = dilate_word0(x, bc);
+        return x;
+    }
+    uint32_t xl, xr;
+    words_beside([&](uint32_t j) { return a[j]; }, w, bc, xl, xr);
+    return dilate_edges(x, xl, xr, r);
+}
+// Grading, one word: the 16 parents of word x's cells that must be internal,
+// those of every cell within r of a marked one
+__device__ __forceinline__ uint32_t graded_parents(uint32_t x, uint32_t xl, uint32_t xr, int r) {
+    const uint32_t d = dilate_edges(x, xl, xr, r);
+    return compact_even(d | (d >> 1));
 }
 
 // ---------------------------------------------------------------------------
@@ -170,20 +172,15 @@ __device__ __forceinline__ uint32_t dilate1_edges(uint32_t x, bool left, bool ri
 template <typename T>
 struct TeamSmem {
     InstDesc d;
-    int woff[MAXLEV + 2];
-    int ooff[MAXLEV + 2];    // occupancy words of level l start at ooff[l]
-    int cw_seg[MAXLEV + 2];  // candidate words of level l: entries [cw_seg[l], cw_seg[l+1]) of the list
-    int sparse;              // word passes over candidate words (else over every word)
-    int seg[NLIST][MAXLEV + 2];
+    int cw_seg[MAXLEV + 2];  // candidate words of level l >= 5: entries [cw_seg[l], cw_seg[l+1]) of their list
+    int seg[NSEG][MAXLEV + 2];
     double eps_l[MAXLEV + 1], big_l[MAXLEV + 1], dx_l[MAXLEV + 1];  // per level
     float eps_f[MAXLEV + 1], big_f[MAXLEV + 1];
     double mass[3];
     double audit;
     unsigned long long updates, steps, passes;
-    int cur, nleaf, status, near_ties;
-    uint32_t deplev[2];  // levels holding transfer (0) / ghost (1) cells that wait on the same list
-    int idx;
-    int g0s, gbase;  // level_of_word constants
+    int cur, nleaf, status, near_ties, ncw;
+    uint32_t deplev[2];  // levels holding transfer (0) / ghost (1) pairs that wait on the same list
 #ifdef MRG_PHASE_TIMERS
     long long tlast;
     unsigned long long ptime[NPHASE];
@@ -192,7 +189,7 @@ struct TeamSmem {
 
 // block-team scratch (scan partials and reduction slots of the warps)
 struct BlockScratch {
-    int scan_w[2][NLIST][32];
+    uint32_t scan_w[2][2][32];
     double red[3][64];
 };
 
@@ -203,18 +200,6 @@ struct BlockSmem {
     TeamSmem<T> team;
     int idx;
 };
-
-template <typename T>
-__device__ __forceinline__ void level_of_word(const TeamSmem<T> &sm, int g, int &l, int &wi) {
-    if (g < sm.g0s) {
-        l = sm.d.Jmin + g;
-        wi = 0;
-    } else {
-        int x = g - sm.g0s + sm.gbase;
-        l = 5 + (31 - __clz(x));
-        wi = x - (1 << (l - 5));
-    }
-}
 
 // ---------------------------------------------------------------------------
 // scheme: vectorial D1Q2^n (Section 2.1, equilibria of Sections 5.1 and 5.3)
@@ -450,102 +435,6 @@ __device__ __forceinline__ void dq_equilibrium_populations(const InstDesc &d, co
     }
 }
 
-// prediction of child `odd` of cell p of a row at level lp (Section 3.1, gamma = 1)
-template <typename T, typename R>
-__device__ __forceinline__ T predict(const R &row, long long p, int odd, int lp, int bc) {
-    T vl = row[wrapc(p - 1, lp, bc)], vp = row[p], vr = row[wrapc(p + 1, lp, bc)];
-    T t = T(C1) * (vr - vl);  // exact: c_1 is a power of two
-    return odd ? vp - t : vp + t;
-}
-
-// the same for a stencil of half-width gamma = 2 or 3 (coefficients c[0..gamma-1]):
-// f_p +- sum_a c_a (f_{p+a} - f_{p-a}), the sum accumulated in increasing a
-template <typename T, typename R>
-__device__ __forceinline__ T predict_g(const R &row, long long p, int odd, int lp, int bc, int gamma, const T *c) {
-    T t = c[0] * (row[wrapc(p + 1, lp, bc)] - row[wrapc(p - 1, lp, bc)]);
-#pragma unroll
-    for (int a = 2; a <= 3; ++a)
-        if (a <= gamma) t = t + c[a - 1] * (row[wrapc(p + a, lp, bc)] - row[wrapc(p - a, lp, bc)]);
-    const T vp = row[p];
-    return odd ? vp - t : vp + t;
-}
-
-// dilation by r <= 16 cells of the word x, given the words on its left (xl) and
-// right (xr) (only their r cells nearest to x are read)
-__device__ __forceinline__ uint32_t dilate_edges(uint32_t x, uint32_t xl, uint32_t xr, int r) {
-    uint32_t out = x;
-    for (int s = 1; s <= r; ++s) out |= (x << s) | (xl >> (32 - s)) | (x >> s) | (xr << (32 - s));
-    return out;
-}
-// parent bits of 6 child bits (3 parents)
-__device__ __forceinline__ uint32_t fold3(uint32_t t) {
-    t |= t >> 1;
-    return (t & 1u) | ((t >> 1) & 2u) | ((t >> 2) & 4u);
-}
-
-// First (last = false) or last finest value of one population row of the leaf
-// (l, k), by the reconstruction operator of Section 3.3 (Definition V): the
-// level-l window k - 2G .. k + 2G (tree and ghost values) is predicted level by
-// level down to Jmax around the leaf's first (last) finest cell, and wherever a
-// finer level holds a cell of the tree (the children of refined neighbours)
-// its value is used instead.  Out-of-domain cells take the value of the nearest
-// domain cell (copy boundary) or wrap (periodic), as in the prediction.
-template <typename T, int G, bool LAST>
-__device__ __noinline__ T edge_walk(const T *rowbase, int qs, int Jmin, int Jmax, int bc, const uint32_t *R,
-                                    const int *woff, const T *c, int l, long long k) {
-    constexpr int W = 4 * G + 1, C = 2 * G, E = LAST ? 1 : 0;
-    T w[W], nw[W];
-    {
-        const T *row = rowbase + cell_off(l, Jmin) * qs;
-#pragma unroll
-        for (int t = 0; t < W; ++t) w[t] = row[wrapc(k + t - C, l, bc) * qs];
-    }
-    long long i = k;
-    for (int m = l; m < Jmax; ++m) {
-        const long long nn = 1LL << (m + 1), inext = 2 * i + E;
-        const T *row = rowbase + cell_off(m + 1, Jmin) * qs;
-        const uint32_t *Rm = R + woff[m + 1];
-        T lo = T(0), hi = T(0);  // values of the first and last cells of the level (copy boundary)
-#pragma unroll
-        for (int t = 0; t < W; ++t) {
-            // window position t is cell inext + t - C; its parent is window position pp of level m
-            const long long pos = inext + t - C;
-            const int pp = C + ((E + t - C) >> 1);
-            const bool odd = ((E + t - C) & 1) != 0;
-            long long cp = pos;
-            bool inside = true;
-            if (bc == 0)
-                cp = pos & (nn - 1);
-            else
-                inside = pos >= 0 && pos < nn;
-            T v;
-            if (inside && ((Rm[(int)(cp >> 5)] >> (cp & 31)) & 1u)) {
-                v = row[cp * qs];
-            } else {
-                T sum = c[0] * (w[pp + 1] - w[pp - 1]);
-#pragma unroll
-                for (int a = 2; a <= G; ++a) sum = sum + c[a - 1] * (w[pp + a] - w[pp - a]);
-                v = odd ? w[pp] - sum : w[pp] + sum;
-            }
-            nw[t] = v;
-            if (pos == 0) lo = v;
-            if (pos == nn - 1) hi = v;
-        }
-        if (bc != 0) {
-#pragma unroll
-            for (int t = 0; t < W; ++t) {
-                const long long pos = inext + t - C;
-                if (pos < 0) nw[t] = lo;
-                if (pos >= nn) nw[t] = hi;
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < W; ++t) w[t] = nw[t];
-        i = inext;
-    }
-    return w[C];
-}
-
 // NaN or infinity, from the exponent field (integer units)
 __device__ __forceinline__ bool nonfinite(double x) { return (__double2hiint(x) & 0x7FF00000) == 0x7FF00000; }
 __device__ __forceinline__ bool nonfinite(float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; }
@@ -579,17 +468,9 @@ __device__ __forceinline__ void decide_bits(unsigned long long Db, double el, do
 }
 
 // ---------------------------------------------------------------------------
-// the instance worker; TS threads (a warp or the whole block) form the team
+// the instance worker; the TS threads of the block form the team
 
 constexpr int QMAX = 6;  // populations of the largest scheme (vectorial D1Q2^3)
-
-// One population of the cell-major value layout: the Q values of a cell are
-// contiguous, so element k of the population starting at p sits at p[k * Q].
-template <typename T, int Q>
-struct SRow {
-    T *p;
-    __device__ __forceinline__ T &operator[](long long k) const { return p[k * Q]; }
-};
 
 // WIDE: prediction stencils gamma = 2, 3 (the gamma = 1 code is a separate instantiation)
 // SPM: word passes over every word (0) or over candidate words (1, the
@@ -597,28 +478,24 @@ struct SRow {
 // even where it does not run)
 template <typename T, int NF, int TS, bool WIDE, int SPM>
 struct Worker {
-    static constexpr bool WARP = TS == 32;
     // NF = 1, 2, 3: vectorial D1Q2^NF; NF = 4: D1Q3, NF = 5: D1Q5 shallow water
     static constexpr bool DQ = NF >= 4;
-    static constexpr int nf = DQ ? 2 : NF;                          // conserved moments
-    static constexpr int q = DQ ? (NF == 4 ? 3 : 5) : 2 * NF;       // populations
-    static constexpr int SIGMA = NF == 5 ? 2 : 1;                   // enlargement width max |w^h|
+    static constexpr int nf = DQ ? 2 : NF;                     // conserved moments
+    static constexpr int q = DQ ? (NF == 4 ? 3 : 5) : 2 * NF;  // populations
+    static_assert(TS >= 64 && TS % 64 == 0, "team width");
     TeamSmem<T> &sm;
     const Tables<T> &tab;
     BlockScratch &bx;
     const InstDesc &d;
-    T *V;
-    T *Phi;
-    uint32_t *M;     // mask base (shared memory when the masks fit, else global)
-    int tid;         // rank in the team
-    long long voff;  // -2^Jmin q: level l's values start at V + 2^l q + voff
+    T *V;         // cell h at V + h q
+    uint32_t *M;  // bit arrays (shared memory when they fit, else global)
+    const int tid;
+    const int bc, Jmin, Jmax;
 
     __device__ Worker(TeamSmem<T> &s, const Tables<T> &tb, BlockScratch &x, int rank, uint32_t *masks)
-        : sm(s), tab(tb), bx(x), d(s.d), tid(rank) {
-        V = (T *)d.V;
-        Phi = (T *)d.Phi;
+        : sm(s), tab(tb), bx(x), d(s.d), tid(rank), bc(s.d.bc), Jmin(s.d.Jmin), Jmax(s.d.Jmax) {
+        V = (T *)d.V - (1LL << d.Jmin) * q;
         M = masks;
-        voff = -(1LL << d.Jmin) * q;
     }
 
     // leaves collision of the q populations of one cell
@@ -635,10 +512,7 @@ struct Worker {
     // thread after the barrier; the batch variants do not: the count cost them
     // 7 % (measured), most of their passes being short.
     __device__ __forceinline__ void sync() const {
-        if constexpr (WARP)
-            __syncwarp();
-        else
-            __syncthreads();
+        __syncthreads();
         if constexpr (SPM != 0)
             if (tid == TS - 1) ++sm.passes;
     }
@@ -657,66 +531,93 @@ struct Worker {
 #endif
     }
 
-    __device__ __forceinline__ uint32_t *mask(int m) { return M + (long long)m * d.Wtot; }
-    // candidate-word list of the step (global mask word indices, sorted by level then word)
-    __device__ __forceinline__ uint32_t *cwl() { return M + (long long)NMASK * d.Wtot; }
-    // i-th word of the step's word passes: a candidate word, or word i itself
-    __device__ __forceinline__ int cw_at(int i) { return sparse_on() ? (int)cwl()[i] : i; }
-    __device__ __forceinline__ bool sparse_on() const { return SPM != 0; }
-    // occupancy bitmap of tree buffer b (M_R0 or M_R1): bit wi & 31 of word ooff[l] + (wi >> 5) is set
-    // when word wi of level l of that tree holds a cell
-    __device__ __forceinline__ uint32_t *occ(int b) { return M + (long long)(NMASK + 1) * d.Wtot + (long long)b * d.OW; }
-    __device__ __forceinline__ uint32_t *list(int L) { return d.lists + d.list_off[L]; }
-    // population h on level l, and population h of the interface array
-    // population h of level l, at cell_off(l, Jmin) q + h.  The FP64 kernels hold
-    // Jmin in voff: the descriptor field, reloaded from shared memory after every
-    // store, would sit on the dependent chain of each population loop (measured:
-    // +1.5 % FP64); the FP32 kernels keep the reload, whose register is dearer
-    // to them (the offset cost them spills and 3.6 %)
-    __device__ __forceinline__ SRow<T, q> row(int h, int l) const {
-        if constexpr (sizeof(T) == 8)
-            return SRow<T, q>{V + ((1LL << l) * q + voff + h)};
-        else
-            return SRow<T, q>{V + cell_off(l, d.Jmin) * q + h};
+    __device__ __forceinline__ uint32_t *mask(int m) const { return M + m * d.Wtot; }
+    // candidate-word list of the step (word indices, sorted)
+    __device__ __forceinline__ uint32_t *cwl() const { return M + NMASK * d.Wtot; }
+    // occupancy array of tree buffer b (M_I0 or M_I1): bit w is set when word w of that tree is not empty
+    __device__ __forceinline__ uint32_t *occ(int b) const { return M + (long long)(NMASK + 1) * d.Wtot + b * d.OW; }
+    __device__ __forceinline__ uint32_t *list(int L) const { return d.lists + d.list_off[L]; }
+    // first word of the word passes (it holds the cells of level Jmin - 1) and
+    // their number; i-th word of a pass: a candidate word, or the words in turn
+    __device__ __forceinline__ uint32_t first_word() const { return (1u << (Jmin - 1)) >> 5; }
+    __device__ __forceinline__ int nwords() const {
+        if constexpr (SPM != 0) return sm.ncw;
+        return d.Wtot - (int)first_word();
     }
-    __device__ __forceinline__ SRow<T, q> phi(int h) const { return SRow<T, q>{Phi + h}; }
+    __device__ __forceinline__ uint32_t word_at(int i) const {
+        if constexpr (SPM != 0) return cwl()[i];
+        return first_word() + (uint32_t)i;
+    }
+    // index of the segment end of a whole list (levels below 5 share one segment)
+    __device__ __forceinline__ int top() const { return Jmax > 5 ? Jmax : 5; }
+    // the cells above Jmin among the bits of word w
+    __device__ __forceinline__ uint32_t above(uint32_t w) const {
+        if (w == 0u) return Jmin >= 5 ? 0xFFFFFFFEu : (1u << (1 << Jmin)) - 2u;
+        return Jmin > 5 && w < (1u << (Jmin - 5)) ? FULL : 0u;
+    }
+    __device__ __forceinline__ T *cell(uint32_t h) const { return V + h * (uint32_t)q; }
+    __device__ __forceinline__ T *phi(uint32_t x) const { return (T *)d.Phi + x * (uint32_t)q; }
+    __device__ __forceinline__ uint32_t nb(uint32_t h, int a, uint32_t lo) const { return neighbour(h, a, lo, bc); }
 
-    // sums over the team of nf per-thread doubles, valid in thread 0 (one barrier)
-    // The team's sum of x[j], in thread 0.  GB300's FP64 units take a warp-wide
-    // instruction whole whatever its active lanes, so the additions are kept
-    // off most warps: a few shuffle rounds in each warp leave 64 partial sums
-    // per field (groups of TS / 64 lanes) in shared memory, and warp 0 folds
-    // them (two per lane, then a shuffle tree).  A fixed order: deterministic.
-    __device__ __forceinline__ void team_sum(double (&x)[3]) {
-        if constexpr (WARP) {
+    // the q populations of cell h in registers; two a load where the cells are
+    // aligned for it (even q: a cell starts at a multiple of two values)
+    __device__ __forceinline__ void load_cell(uint32_t h, T *f) const { load_pops(cell(h), f); }
+    __device__ __forceinline__ void load_pops(const T *p, T *f) const {
+        if constexpr (q % 2 == 0) {
 #pragma unroll
-            for (int j = 0; j < 3; ++j)
-                if (j < nf)
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) x[j] += __shfl_down_sync(FULL, x[j], o);
+            for (int j = 0; j < q / 2; ++j) {
+                const auto v = reinterpret_cast<const typename V2<T>::type *>(p)[j];
+                f[2 * j] = v.x;
+                f[2 * j + 1] = v.y;
+            }
         } else {
-            static_assert(TS >= 64 && TS % 64 == 0, "team width");
-            constexpr int G = TS / 64;  // lanes per partial sum: 1, 2, 4, 8 or 16
+#pragma unroll
+            for (int j = 0; j < q; ++j) f[j] = p[j];
+        }
+    }
+    __device__ __forceinline__ void store_cell(uint32_t h, const T *f) const {
+        T *p = cell(h);
+        if constexpr (q % 2 == 0) {
+#pragma unroll
+            for (int j = 0; j < q / 2; ++j) {
+                typename V2<T>::type v;
+                v.x = f[2 * j];
+                v.y = f[2 * j + 1];
+                reinterpret_cast<typename V2<T>::type *>(p)[j] = v;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < q; ++j) p[j] = f[j];
+        }
+    }
+
+    // The team's sum of x[j], in thread 0 (one barrier).  GB300's FP64 units
+    // take a warp-wide instruction whole whatever its active lanes, so the
+    // additions are kept off most warps: a few shuffle rounds in each warp leave
+    // 64 partial sums per field (groups of TS / 64 lanes) in shared memory, and
+    // warp 0 folds them (two per lane, then a shuffle tree).  A fixed order:
+    // deterministic.
+    __device__ __forceinline__ void team_sum(double (&x)[3]) {
+        constexpr int G = TS / 64;  // lanes per partial sum: 1, 2, 4, 8 or 16
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            if (j < nf)
+#pragma unroll
+                for (int o = G / 2; o > 0; o >>= 1) x[j] += __shfl_down_sync(FULL, x[j], o);
+        if ((tid & (G - 1)) == 0)
 #pragma unroll
             for (int j = 0; j < 3; ++j)
-                if (j < nf)
+                if (j < nf) bx.red[j][tid / G] = x[j];
+        sync();
+        if (tid < 32)
 #pragma unroll
-                    for (int o = G / 2; o > 0; o >>= 1) x[j] += __shfl_down_sync(FULL, x[j], o);
-            if ((tid & (G - 1)) == 0)
+            for (int j = 0; j < 3; ++j)
+                if (j < nf) {
+                    double v = bx.red[j][tid] + bx.red[j][tid + 32];
 #pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (j < nf) bx.red[j][tid / G] = x[j];
-            sync();
-            if (tid < 32)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (j < nf) {
-                        double v = bx.red[j][tid] + bx.red[j][tid + 32];
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-                        x[j] = v;
-                    }
-        }
+                    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
+                    x[j] = v;
+                }
     }
 
     // float-float accumulation (hi + lo, error-free transformation TwoSum of
@@ -742,65 +643,35 @@ struct Worker {
                     const float h2 = __shfl_down_sync(FULL, hi[j], o), l2 = __shfl_down_sync(FULL, lo[j], o);
                     ff_add(hi[j], lo[j], h2, l2);
                 }
-        if constexpr (!WARP) {
-            float2 *red = reinterpret_cast<float2 *>(&bx.red[0][0]);
-            if ((tid & 31) == 0)
+        float2 *red = reinterpret_cast<float2 *>(&bx.red[0][0]);
+        if ((tid & 31) == 0)
 #pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (j < nf) red[j * 32 + (tid >> 5)] = make_float2(hi[j], lo[j]);
-            sync();
-            if (tid == 0)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (j < nf) {
-                        float h = 0.0f, l = 0.0f;
-                        for (int w = 0; w < TS / 32; ++w) ff_add(h, l, red[j * 32 + w].x, red[j * 32 + w].y);
-                        hi[j] = h;
-                        lo[j] = l;
-                    }
-        }
+            for (int j = 0; j < 3; ++j)
+                if (j < nf) red[j * 32 + (tid >> 5)] = make_float2(hi[j], lo[j]);
+        sync();
         // only thread 0 holds the sums: the other threads keep off the FP64 pipe
         if (tid == 0)
 #pragma unroll
             for (int j = 0; j < 3; ++j)
-                if (j < nf) out[j] = (double)hi[j] + (double)lo[j];
-    }
-
-    // ---- projection of the internal cells of level l (Def. Projection operator)
-    __device__ __forceinline__ void project_level(const uint32_t *lst, int l) {
-        int b = sm.seg[L_INT][l], e = sm.seg[L_INT][l + 1];
-        for (int i = b + tid; i < e; i += TS) {
-            long long k = lst[i] & KMASK;
-            // the two children are adjacent cells: 2q contiguous values
-            T ce[QMAX], co[QMAX];
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) {
-                    const auto rc = row(h, l + 1);
-                    ce[h] = rc[2 * k];
-                    co[h] = rc[2 * k + 1];
+                if (j < nf) {
+                    float h = 0.0f, l = 0.0f;
+#pragma unroll 1
+                    for (int w = 0; w < TS / 32; ++w) ff_add(h, l, red[j * 32 + w].x, red[j * 32 + w].y);
+                    out[j] = (double)h + (double)l;
                 }
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) row(h, l)[k] = half_of<T>(ce[h] + co[h]);
-        }
     }
 
     // ---- S1: leaves collision (eq. LeavesCollision) ---------------------------
     __device__ void collide_all() {
         const uint32_t *lst = list(L_LEAF);
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            uint32_t ent = lst[i];
-            int l = ent >> KBITS;
-            long long k = ent & KMASK;
-            T f[QMAX];
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) f[h] = row(h, l)[k];
+        const int n = sm.nleaf;
+#pragma unroll 1
+        for (int i = tid; i < n; i += TS) {
+            const uint32_t h = lst[i];
+            T f[q];
+            load_cell(h, f);
             collide_cell(f);
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) row(h, l)[k] = f[h];
+            store_cell(h, f);
         }
     }
 
@@ -830,43 +701,46 @@ struct Worker {
         }
     }
 
+    // the populations of every finest cell by the reconstruction operator
+    // (Definition V): internal cells projected, then every cell outside the
+    // tree predicted, level by level
+    __device__ void fill_finest() {
+        upsweep();
+        const uint32_t *I = mask(sm.cur);
+#pragma unroll 1
+        for (int l = Jmin; l < Jmax; ++l) {
+            const uint32_t lo = 1u << l;
+#pragma unroll 1
+            for (uint32_t p = lo + tid; p < 2u * lo; p += TS)
+                if (!bit_of(I, p)) predict_pair(p, lo);
+            sync();
+        }
+    }
+
     // S1 with the reconstructed collision (Section 4.5, eq. reconstructedCollision):
-    // the pre-collision populations are reconstructed on every finest cell
-    // (projection up the tree, prediction of every other cell level by level);
+    // the pre-collision populations are reconstructed on every finest cell;
     // each warp averages, one leaf at a time, the equilibria of the relaxed
     // moments over the leaf's 2^dj finest cells (into the interface array, free
     // until S4); then every leaf relaxes towards those averages.
     __device__ __noinline__ void collide_reconstructed() {
-        upsweep();
-        sync();
-        const uint32_t *R = mask(sm.cur);
-        for (int l = d.Jmin + 1; l <= d.Jmax; ++l) {
-            const long long n = 1LL << l;
-            const uint32_t *rl = R + sm.woff[l];
-            for (long long k = tid; k < n; k += TS)
-                if (!((rl[k >> 5] >> (k & 31)) & 1u))
-                    for (int h = 0; h < q; ++h)
-                        row(h, l)[k] = predict_g<T>(row(h, l - 1), k >> 1, (int)(k & 1), l - 1, d.bc, d.gamma,
-                                                    tab.pc[d.gamma]);
-            sync();
-        }
+        fill_finest();
         constexpr int NR = DQ ? q - 2 : nf;  // relaxed moments
         constexpr int NWARP = TS / 32;
         const int lane = tid & 31, warp = tid >> 5;
         const uint32_t *leaves = list(L_LEAF);
+        T *Phi = (T *)d.Phi;
         const long long stride = d.N + 1;
-        for (int i = warp; i < sm.nleaf; i += NWARP) {
-            const uint32_t ent = leaves[i];
-            const int l = ent >> KBITS;
-            const long long k = ent & KMASK;
-            const int dj = d.Jmax - l;
-            const long long first = k << dj, ncell = 1LL << dj;
+        const int nl = sm.nleaf;
+#pragma unroll 1
+        for (int i = warp; i < nl; i += NWARP) {
+            const uint32_t hl = leaves[i];
+            const int dj = Jmax - level_of(hl);
+            const uint32_t first = hl << dj, end = first + (1u << dj);
             T acc[3] = {T(0), T(0), T(0)};
-            for (long long c = first + lane; c < first + ncell; c += 32) {
-                T g[QMAX], meq[3];
-#pragma unroll
-                for (int h = 0; h < QMAX; ++h)
-                    if (h < q) g[h] = row(h, d.Jmax)[c];
+#pragma unroll 1
+            for (uint32_t c = first + lane; c < end; c += 32) {
+                T g[q], meq[3];
+                load_cell(c, g);
                 relaxed_equilibria(g, meq);
 #pragma unroll
                 for (int r = 0; r < NR; ++r) acc[r] = acc[r] + meq[r];
@@ -880,14 +754,11 @@ struct Worker {
                 for (int r = 0; r < NR; ++r) Phi[r * stride + i] = acc[r] * pow2m<T>(dj);
         }
         sync();
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            const uint32_t ent = leaves[i];
-            const int l = ent >> KBITS;
-            const long long k = ent & KMASK;
-            T f[QMAX], mavg[3];
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) f[h] = row(h, l)[k];
+#pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            const uint32_t hc = leaves[i];
+            T f[q], mavg[3];
+            load_cell(hc, f);
 #pragma unroll
             for (int r = 0; r < NR; ++r) mavg[r] = Phi[r * stride + i];
             if constexpr (DQ) {
@@ -928,19 +799,44 @@ struct Worker {
                     f[2 * j + 1] = half_of<T>(A::sub(mc, g));
                 }
             }
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) row(h, l)[k] = f[h];
+            store_cell(hc, f);
         }
         sync();
     }
 
-    // ---- A1 / S2: projection sweep, fine to coarse ---------------------------
+    // ---- A1 / S2: projection sweep, fine to coarse (Def. Projection operator) -
+    // projection of cell h: the mean of its two children, 2q adjacent values
+    __device__ __forceinline__ void project_cell(uint32_t h) const {
+        T a[q], b[q];
+        load_cell(2u * h, a);
+        load_cell(2u * h + 1u, b);
+#pragma unroll
+        for (int j = 0; j < q; ++j) a[j] = half_of<T>(a[j] + b[j]);
+        store_cell(h, a);
+    }
+    // one level per barrier; the levels of at most 32 cells by one warp, cell by
+    // lane, without block barriers.  Ends with a barrier.
     __device__ void upsweep() {
         const uint32_t *li = list(L_INT);
-        for (int l = d.Jmax - 1; l >= d.Jmin; --l) {
-            if (sm.seg[L_INT][l] == sm.seg[L_INT][l + 1]) continue;
-            project_level(li, l);
+        const int ls = Jmin > 6 ? Jmin : 6;
+#pragma unroll 1
+        for (int l = Jmax - 1; l >= ls; --l) {
+            const int b = sm.seg[L_INT][l], e = sm.seg[L_INT][l + 1];
+            if (b == e) continue;
+#pragma unroll 1
+            for (int i = b + tid; i < e; i += TS) project_cell(li[i]);
+            sync();
+        }
+        if (Jmin < 6) {
+            if (tid < 32) {
+                const uint32_t *I = mask(sm.cur);
+#pragma unroll 1
+                for (int l = Jmax - 1 < 5 ? Jmax - 1 : 5; l >= Jmin; --l) {
+                    const uint32_t h = (1u << l) + tid;
+                    if (tid < (1 << l) && bit_of(I, h)) project_cell(h);
+                    __syncwarp();
+                }
+            }
             sync();
         }
     }
@@ -959,24 +855,28 @@ struct Worker {
     // adaptation then starts from projected internal cells (status ST_FLUXED).
     __device__ __forceinline__ void project_by_flux_pass() {
         const uint32_t *li = list(L_INT);
-        const int b = sm.seg[L_INT][d.Jmin], e = sm.seg[L_INT][d.Jmax];
-        for (int i = b + tid; i < e; i += TS) {
-            const uint32_t ent = li[i];
-            const int l = ent >> KBITS;
-            const long long k = ent & KMASK;
-            const int dj = d.Jmax - l;
-            long long first = k << dj, next = (k + 1) << dj;
-            if (d.bc == 0) next &= d.N - 1;
-            const T w = pow2m<T>(dj);
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) {
-                    const auto ph = phi(h);
-                    const T coef = (h & 1) ? -w : w;
-                    const auto r = row(h, l);
-                    r[k] = r[k] + coef * (ph[first] - ph[next]);
-                }
+        const int e = sm.seg[L_INT][top()];
+#pragma unroll 1
+        for (int i = tid; i < e; i += TS) {
+            const uint32_t h = li[i];
+            T f[q];
+            stream_cell(h, f);
+            store_cell(h, f);
         }
+    }
+    // the D1Q2^n stream of cell h (leaf or internal): f + w (Phi[first] - Phi[next])
+    __device__ __forceinline__ void stream_cell(uint32_t h, T *f) const {
+        const int dj = Jmax - level_of(h);
+        const uint32_t first = (h << dj) & ((1u << Jmax) - 1u);
+        uint32_t next = first + (1u << dj);
+        if (bc == 0) next &= (1u << Jmax) - 1u;
+        const T w = pow2m<T>(dj);
+        load_cell(h, f);
+        T x[q], y[q];
+        load_pops(phi(first), x);
+        load_pops(phi(next), y);
+#pragma unroll
+        for (int j = 0; j < q; ++j) f[j] = f[j] + ((j & 1) ? -w : w) * (x[j] - y[j]);
     }
 
     // ---- A2: details of the pairs of the tree, threshold T, Harten flags ----
@@ -984,56 +884,62 @@ struct Worker {
     // a rigorous bound on its rounding error; only when a threshold lies within
     // that bound is the detail recomputed in FP64 from the stored values, so
     // every decision equals the one the exact detail of the stored state gives.
+    // KEEP / REF bits go to the pair's parent p (both children of a kept pair
+    // are kept).  The prediction sums c_a (f_{p+a} - f_{p-a}) in increasing a.
     __device__ void details() {
-        if constexpr (WIDE) {
-            details_wide();
-            return;
-        }
-        // the even cells of the tree above Jmin: first children 2p of the internal cells p
         const uint32_t *lst = list(L_INT);
-        int b = sm.seg[L_INT][d.Jmin], e = sm.seg[L_INT][d.Jmax];
+        const int e = sm.seg[L_INT][top()];
+        const int g = WIDE ? d.gamma : 1;
         uint32_t *keep = mask(M_KEEP), *ref = mask(M_REF);
-        for (int i = b + tid; i < e; i += TS) {
-            uint32_t ent = lst[i];
-            int l = (int)(ent >> KBITS) + 1;
-            const bool hasref = l < d.Jmax;
-            long long p = ent & KMASK, k = 2 * p;
-            long long pl = wrapc(p - 1, l - 1, d.bc), pr = wrapc(p + 1, l - 1, d.bc);
+#pragma unroll 1
+        for (int i = tid; i < e; i += TS) {
+            const uint32_t p = lst[i];
+            const uint32_t lo = level_first(p);
+            const int l = level_of(p) + 1;
+            const bool hasref = l < Jmax;
             bool keepit, refit, tie = false;
+            const T *vk = cell(2u * p), *vp = cell(p), *vl = cell(nb(p, -1, lo)), *vr = cell(nb(p, 1, lo));
             if constexpr (sizeof(T) == 8) {
                 unsigned long long Db = 0ull;
 #pragma unroll
-                for (int h = 0; h < QMAX; ++h)
-                    if (h < q) {
-                        const auto rc = row(h, l - 1);
-                        const double dv = row(h, l)[k] - (rc[p] + C1 * (rc[pr] - rc[pl]));
-                        const unsigned long long b = abs_bits(dv);
-                        Db = b > Db ? b : Db;
-                    }
+                for (int h = 0; h < q; ++h) {
+                    double sum = C1 * (vr[h] - vl[h]);
+                    if constexpr (WIDE) sum = wide_sum(p, lo, h, sum);
+                    const unsigned long long b = abs_bits(vk[h] - (vp[h] + sum));
+                    Db = b > Db ? b : Db;
+                }
                 decide_bits(Db, sm.eps_l[l], sm.big_l[l], hasref, keepit, refit, tie);
             } else {
                 float D = 0.0f, B = 0.0f;
 #pragma unroll
-                for (int h = 0; h < QMAX; ++h)
-                    if (h < q) {
-                        const auto rc = row(h, l - 1);
-                        float vk = row(h, l)[k], vl = rc[pl], vp = rc[p], vr = rc[pr];
-                        float dv = vk - (vp + float(C1) * (vr - vl));
-                        D = fmaxf(D, fabsf(dv));
-                        B = fmaxf(B, fabsf(vk) + fabsf(vp) + fabsf(vl) + fabsf(vr));
+                for (int h = 0; h < q; ++h) {
+                    const float xk = vk[h], xp = vp[h], xl = vl[h], xr = vr[h];
+                    float sum = float(C1) * (xr - xl), mag = fabsf(xl) + fabsf(xr);
+                    if constexpr (WIDE) {
+                        sum = wide_sum(p, lo, h, sum);
+                        mag += wide_mag(p, lo, h);
                     }
-                B *= 0x1p-21f;  // 4 times the rounding bound of the detail evaluation
-                float el = sm.eps_f[l], bl = sm.big_f[l];
+                    D = fmaxf(D, fabsf(xk - (xp + sum)));
+                    B = fmaxf(B, fabsf(xk) + fabsf(xp) + mag);
+                }
+                // the rounding of the detail: for gamma = 1 4 times the bound of its
+                // evaluation; (6 gamma + 2) u times the sum of |inputs| else (3 gamma + 1
+                // roundings, each at most u times that sum, with a factor 2 margin)
+                B *= WIDE && g > 1 ? (float)(6 * g + 2) * 0x1p-24f : 0x1p-21f;
+                const float el = sm.eps_f[l], bl = sm.big_f[l];
                 // the band also covers the rounding of the thresholds to float
-                bool amb = fabsf(D - el) <= B + el * 0x1p-22f || (hasref && fabsf(D - bl) <= B + bl * 0x1p-22f);
+                const bool amb = fabsf(D - el) <= B + el * 0x1p-22f || (hasref && fabsf(D - bl) <= B + bl * 0x1p-22f);
                 if (amb) {
                     double Dd = 0.0;
+#pragma unroll 1
                     for (int h = 0; h < q; ++h) {
-                        const auto rc = row(h, l - 1);
-                        double dv = (double)row(h, l)[k] - ((double)rc[p] + C1 * ((double)rc[pr] - (double)rc[pl]));
-                        Dd = fmax(Dd, fabs(dv));
+                        double sum = (WIDE ? (double)tab.pc[g][0] : C1) * ((double)vr[h] - (double)vl[h]);
+                        if constexpr (WIDE)
+                            for (int a = 2; a <= g; ++a)
+                                sum = sum + (double)tab.pc[g][a - 1] * ((double)cell(nb(p, a, lo))[h] - (double)cell(nb(p, -a, lo))[h]);
+                        Dd = fmax(Dd, fabs((double)vk[h] - ((double)vp[h] + sum)));
                     }
-                    double e64 = sm.eps_l[l], b64 = sm.big_l[l];
+                    const double e64 = sm.eps_l[l], b64 = sm.big_l[l];
                     keepit = Dd >= e64;
                     refit = hasref && Dd >= b64;
                     tie = fabs(Dd - e64) <= 1e-12 * e64 || (hasref && fabs(Dd - b64) <= 1e-12 * b64);
@@ -1044,128 +950,48 @@ struct Worker {
             }
             if (tie) atomicAdd(&sm.near_ties, 1);
             if (keepit) {
-                int w = (int)(k >> 5);
-                uint32_t bits = 3u << (k & 31);
-                atomicOr(&keep[sm.woff[l] + w], bits);
-                if (refit) atomicOr(&ref[sm.woff[l] + w], bits);
+                const uint32_t bit = 1u << (p & 31u);
+                atomicOr(&keep[p >> 5], bit);
+                if (refit) atomicOr(&ref[p >> 5], bit);
             }
         }
     }
-
-    // A2 with the stencil of half-width gamma = 2 or 3: the prediction sums
-    // c_a (f_{p+a} - f_{p-a}) in increasing a; the FP32 rounding band grows with
-    // the number of operations, (6 gamma + 2) u times the sum of |inputs|
-    // (3 gamma + 1 roundings, each at most u times that sum, with a factor 2 margin)
-    __device__ __noinline__ void details_wide() {
-        const uint32_t *lst = list(L_INT);  // first children 2p of the internal cells p
-        const int b = sm.seg[L_INT][d.Jmin], e = sm.seg[L_INT][d.Jmax], g = d.gamma;
+    // sum_a c_a (f_{p+a} - f_{p-a}) of population h with the instance's stencil,
+    // given the gamma = 1 sum first (used as it is when gamma = 1)
+    __device__ __forceinline__ T wide_sum(uint32_t p, uint32_t lo, int h, T first) const {
+        const int g = d.gamma;
+        if (g == 1) return first;
         const T *c = tab.pc[g];
-        uint32_t *keep = mask(M_KEEP), *ref = mask(M_REF);
-        for (int i = b + tid; i < e; i += TS) {
-            const uint32_t ent = lst[i];
-            const int l = (int)(ent >> KBITS) + 1;
-            const bool hasref = l < d.Jmax;
-            const long long p = ent & KMASK, k = 2 * p;
-            bool keepit, refit, tie = false;
-            double Dd = 0.0;
-            unsigned long long Db = 0ull;
-            float Df = 0.0f, B = 0.0f;
-            for (int h = 0; h < q; ++h) {
-                const auto rc = row(h, l - 1);
-                T sum = T(0);
-                float mag = 0.0f;
-                for (int a = 1; a <= g; ++a) {
-                    const T vr = rc[wrapc(p + a, l - 1, d.bc)], vl = rc[wrapc(p - a, l - 1, d.bc)];
-                    sum = a == 1 ? c[0] * (vr - vl) : sum + c[a - 1] * (vr - vl);
-                    if constexpr (sizeof(T) == 4) mag = mag + fabsf(vr) + fabsf(vl);
-                }
-                const T vk = row(h, l)[k], vp = rc[p];
-                if constexpr (sizeof(T) == 8) {
-                    const unsigned long long b = abs_bits(vk - (vp + sum));
-                    Db = b > Db ? b : Db;
-                } else {
-                    Df = fmaxf(Df, fabsf(vk - (vp + sum)));
-                    B = fmaxf(B, fabsf(vk) + fabsf(vp) + mag);
-                }
-            }
-            if constexpr (sizeof(T) == 8) {
-                decide_bits(Db, sm.eps_l[l], sm.big_l[l], hasref, keepit, refit, tie);
-            } else {
-                B *= (float)(6 * g + 2) * 0x1p-24f;
-                const float el = sm.eps_f[l], bl = sm.big_f[l];
-                const bool amb = fabsf(Df - el) <= B + el * 0x1p-22f || (hasref && fabsf(Df - bl) <= B + bl * 0x1p-22f);
-                if (amb) {
-                    for (int h = 0; h < q; ++h) {
-                        const auto rc = row(h, l - 1);
-                        double sum = 0.0;
-                        for (int a = 1; a <= g; ++a)
-                            sum = a == 1 ? (double)c[0] * ((double)rc[wrapc(p + 1, l - 1, d.bc)] - (double)rc[wrapc(p - 1, l - 1, d.bc)])
-                                         : sum + (double)c[a - 1] * ((double)rc[wrapc(p + a, l - 1, d.bc)] -
-                                                                     (double)rc[wrapc(p - a, l - 1, d.bc)]);
-                        Dd = fmax(Dd, fabs((double)row(h, l)[k] - ((double)rc[p] + sum)));
-                    }
-                    const double e64 = sm.eps_l[l], b64 = sm.big_l[l];
-                    keepit = Dd >= e64;
-                    refit = hasref && Dd >= b64;
-                    tie = fabs(Dd - e64) <= 1e-12 * e64 || (hasref && fabs(Dd - b64) <= 1e-12 * b64);
-                } else {
-                    keepit = Df >= el;
-                    refit = hasref && Df >= bl;
-                }
-            }
-            if (tie) atomicAdd(&sm.near_ties, 1);
-            if (keepit) {
-                const int w = (int)(k >> 5);
-                const uint32_t bits = 3u << (k & 31);
-                atomicOr(&keep[sm.woff[l] + w], bits);
-                if (refit) atomicOr(&ref[sm.woff[l] + w], bits);
-            }
-        }
+        T sum = c[0] * (cell(nb(p, 1, lo))[h] - cell(nb(p, -1, lo))[h]);
+#pragma unroll 1
+        for (int a = 2; a <= g; ++a) sum = sum + c[a - 1] * (cell(nb(p, a, lo))[h] - cell(nb(p, -a, lo))[h]);
+        return sum;
+    }
+    __device__ __forceinline__ float wide_mag(uint32_t p, uint32_t lo, int h) const {
+        float m = 0.0f;
+#pragma unroll 1
+        for (int a = 2; a <= d.gamma; ++a) m += fabsf((float)cell(nb(p, a, lo))[h]) + fabsf((float)cell(nb(p, -a, lo))[h]);
+        return m;
     }
 
     // ---- candidate words of the step -----------------------------------------
-    // Every cell of the new tree lies within 2 gamma + 4 cells of a cell of the
-    // old tree on its level or of a child of one (the enlargement moves at most
-    // sigma + 1 <= 3 cells from a kept cell and adds children of kept pairs;
-    // grading from level l + 1 reaches gamma + 2 cells beyond half of that
-    // level's distance), and every transfer or ghost mark lies within
-    // 2 gamma + 10 <= 16 cells of one: inside the mask words next to (+-1 word)
-    // a word that holds an old cell, or a child word of one.  Those words are
-    // the step's candidates.  The word passes (enlargement, grading and
-    // marking, list compaction, clearing) visit them only; every other word of
-    // every mask stays zero.  The list is built from the occupancy bitmap of
-    // the old tree (one bit per mask word) by a block scan.
-
-    // level l and index j within the level of occupancy word og (levels up to 9
-    // have one occupancy word, level l >= 10 has 2^(l - 10))
-    __device__ __forceinline__ void level_of_occ(int og, int &l, int &j) const {
-        const int nsmall = max(0, min(d.Jmax, 9) - d.Jmin + 1);
-        if (og < nsmall) {
-            l = d.Jmin + og;
-            j = 0;
-            return;
-        }
-        const int L0 = d.Jmin > 10 ? d.Jmin : 10;
-        const int x = og - nsmall + (1 << (L0 - 10));
-        l = 10 + (31 - __clz(x));
-        j = x - (1 << (l - 10));
+    // (gamma = 1.)  A cell that becomes internal is within one cell of a kept
+    // one, a child of a refined one, or an ancestor that grading requires, and
+    // those lie within three cells of an internal cell of the old tree on their
+    // level, or of a child of one; ghost parents lie one cell further.  All of
+    // them are in the words next to (+-1 word) a word that holds an old internal
+    // cell or a child word of one.  Those words, and the first 32 words, are
+    // the step's candidates.  The word passes (enlargement, grading, list
+    // compaction, clearing) visit them only; every other word of every bit array
+    // stays zero.  The list is built from the occupancy array of the old tree,
+    // a heap of words, by a block scan.
+    __device__ __forceinline__ uint32_t cand_bits(const uint32_t *oc, uint32_t j) const {
+        if (j == 0u) return FULL;
+        auto near = [&](uint32_t i) { return oc[i] | children_word(oc, i); };
+        uint32_t xl, xr;
+        words_beside(near, j, bc, xl, xr);
+        return dilate_edges(near(j), xl, xr, 1);
     }
-    // candidate bits of occupancy word j of level l, from the old tree's occupancy oc
-    __device__ __forceinline__ uint32_t cand_bits(const uint32_t *oc, int l, int j) const {
-        const int Lo = l >= 5 ? l - 5 : 0;  // the level's mask words: 2^Lo
-        const uint32_t vb = Lo >= 5 ? FULL : ((1u << (1 << Lo)) - 1u);
-        if (l <= 6) return vb;  // levels of at most two words: every word
-        const uint32_t *ol = oc + sm.ooff[l];
-        uint32_t x = dilate([&](int q) { return ol[q]; }, Lo, j, 1, d.bc);
-        if (l > d.Jmin) {
-            // child words of the occupied words of level l - 1
-            const uint32_t *op = oc + sm.ooff[l - 1];
-            x |= dilate([&](int q) { return Lo > 5 ? spread16(op[q >> 1] >> (16 * (q & 1))) : (spread16(op[0]) & vb); },
-                        Lo, j, 1, d.bc);
-        }
-        return x & vb;
-    }
-
     __device__ void build_cw() {
         constexpr int NW = TS / 32;
         const int lane = tid & 31, warp = tid >> 5;
@@ -1173,545 +999,193 @@ struct Worker {
         uint32_t *cw = cwl();
         const int OW = d.OW;
         int run = 0;
+        if (tid >= 5 && tid < 10) sm.cw_seg[tid] = 1 << (tid - 5);  // words 0..31 are all candidates
+#pragma unroll 1
         for (int r = 0, base = 0; base < OW; ++r, base += TS) {
-            const int og = base + tid;
-            int l = d.Jmin, j = 0;
-            uint32_t c = 0u;
-            if (og < OW) {
-                level_of_occ(og, l, j);
-                c = cand_bits(oc, l, j);
-            }
-            const int cnt = __popc(c);
-            int x = cnt;
+            const uint32_t j = base + tid;
+            uint32_t c = j < (uint32_t)OW ? cand_bits(oc, j) : 0u;
+            const uint32_t cnt = __popc(c);
+            uint32_t x = cnt;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(FULL, x, o);
+                const uint32_t y = __shfl_up_sync(FULL, x, o);
                 if (lane >= o) x += y;
             }
-            int *sw = bx.scan_w[r & 1][0];  // alternate buffers: one barrier per round
+            uint32_t *sw = bx.scan_w[r & 1][0];  // alternate buffers: one barrier per round
             if (lane == 31) sw[warp] = x;
             sync();
-            const int v = lane < NW ? sw[lane] : 0;
-            const int before = __reduce_add_sync(FULL, lane < warp ? v : 0);
-            const int tot = __reduce_add_sync(FULL, v);
-            int off = run + before + x - cnt;
-            if (og < OW && j == 0) sm.cw_seg[l] = off;
-            const uint32_t g0 = (uint32_t)(sm.woff[l] + 32 * j);
+            const uint32_t v = lane < NW ? sw[lane] : 0u;
+            const uint32_t before = __reduce_add_sync(FULL, lane < warp ? v : 0u);
+            const uint32_t tot = __reduce_add_sync(FULL, v);
+            uint32_t off = run + before + x - cnt;
+            // the words of level l >= 10 start with occupancy word 2^(l - 10)
+            if (j > 0u && j < (uint32_t)OW && (j & (j - 1u)) == 0u) sm.cw_seg[10 + level_of(j)] = off;
+#pragma unroll 1
             while (c) {
                 const int b = __ffs(c) - 1;
                 c &= c - 1u;
-                cw[off++] = g0 + (uint32_t)b;
+                cw[off++] = 32u * j + (uint32_t)b;
             }
             run += tot;
         }
-        if (tid == 0) sm.cw_seg[d.Jmax + 1] = run;
+        if (tid == 0) {
+            sm.cw_seg[Jmax] = run;
+            sm.ncw = run;
+        }
         sync();
     }
 
-    // ---- A3: R(H(T)) per candidate word --------------------------------------
-    __device__ void enlarge(uint32_t *Rn) {
+    // ---- A3: H(T) per word: kept pairs dilated by sigma (one pair for sigma = 1
+    // and 2), children of refined pairs
+    __device__ void enlarge(uint32_t *In) {
         const uint32_t *keep = mask(M_KEEP), *ref = mask(M_REF);
-        const int ncw = sm.cw_seg[d.Jmax + 1];
-        for (int i = tid; i < ncw; i += TS) {
-            const int g = cw_at(i);
-            int l, wi;
-            level_of_word(sm, g, l, wi);
-            uint32_t vb = valid_bits(l), rh;
-            if (l == d.Jmin) {
-                rh = vb;
-            } else {
-                const uint32_t *kl = keep + sm.woff[l];
-                uint32_t rt = kl[wi];
-                rh = rt | pairexpand(dilate([&](int j) { return kl[j]; }, l, wi, SIGMA, d.bc));
-                if (l >= d.Jmin + 2) rh |= spread16(ref[sm.woff[l - 1] + (wi >> 1)] >> (16 * (wi & 1)));
-            }
-            Rn[g] = rh & vb;
+        const int n = nwords();
+#pragma unroll 1
+        for (int i = tid; i < n; i += TS) {
+            const uint32_t w = word_at(i);
+            In[w] = dilate_word(keep, w, 1, bc) | children_word(ref, w) | above(w);
         }
     }
 
-    // ---- A4: grading sweep + leaf / transfer / ghost marking -----------------
-    // Fine to coarse: the cells of level l require (l-1, floor(k/2) + delta),
-    // |delta| <= gamma = 1, with siblings (Def. Graded tree); once level l is
-    // final its leaves (no child in the tree), its transfer marks (new leaves
-    // outside the old tree and the parent stencils of finer marks) and its ghost
-    // marks (reconstruction windows k-2..k+2 of its leaves and the parent
-    // stencils of finer ghosts, outside the tree) are written.  Levels of 64
-    // cells or more work on whole words, with the neighbouring words' edge bits;
-    // the smaller levels are done by one thread without barriers.
-    // grade = false only re-derives the marks of a tree known to be graded.
-    __device__ void grade_and_mark(uint32_t *Rn, const uint32_t *Ro, bool grade) {
-        uint32_t *LF = mask(M_LEAF), *PR = mask(M_PRED), *GH = mask(M_GH);
-        const int g = d.gamma;
-        const int lbig = d.Jmin > 6 ? d.Jmin : 6;
-        for (int l = d.Jmax; l >= lbig; --l) {
-            const int Wl = 1 << (l - 5);
-            const uint32_t *rl = Rn + sm.woff[l];
-            if (grade && l > d.Jmin + 1) {
-                uint32_t *rp = Rn + sm.woff[l - 1];
-                if constexpr (!WIDE) {
-                    for (int i = sm.cw_seg[l - 1] + tid; i < sm.cw_seg[l]; i += TS) {
-                        const int wp = cw_at(i) - sm.woff[l - 1];
-                        uint32_t x = fold2(rl[2 * wp], rl[2 * wp + 1]);
-                        bool eL = (word_bc(rl, 2 * wp - 1, Wl, d.bc) >> 30) != 0u;  // children of parent 32 wp - 1
-                        bool eR = (word_bc(rl, 2 * wp + 2, Wl, d.bc) & 3u) != 0u;   // children of parent 32 wp + 32
-                        rp[wp] |= pairexpand(dilate1_edges(x, eL, eR));
-                    }
-                } else {
-                    for (int i = sm.cw_seg[l - 1] + tid; i < sm.cw_seg[l]; i += TS) {
-                        const int wp = cw_at(i) - sm.woff[l - 1];
-                        const uint32_t x = fold2(rl[2 * wp], rl[2 * wp + 1]);
-                        // parents 29..31 of the word on the left, 0..2 of the word on the right
-                        const uint32_t xl = fold3(word_bc(rl, 2 * wp - 1, Wl, d.bc) >> 26) << 29;
-                        const uint32_t xr = fold3(word_bc(rl, 2 * wp + 2, Wl, d.bc) & 63u);
-                        rp[wp] |= pairexpand(dilate_edges(x, xl, xr, g));
-                    }
-                }
+    // ---- A4: grading (Def. Graded tree), fine to coarse -----------------------
+    // An internal cell p of level l needs the cells p + delta, |delta| <= gamma,
+    // in the tree: their parents must be internal.  The levels of more than 32
+    // words take one block pass each; the others go to one warp: lane i holds
+    // word i of the current level in a register, the words beside it and the
+    // folded halves arrive by shuffles, and no block barrier separates them.
+    __device__ void grade(uint32_t *In) {
+        const int g = WIDE ? d.gamma : 1;
+        const int lwarp = Jmax - 1 < 10 ? Jmax - 1 : 10;
+#pragma unroll 1
+        for (int l = Jmax - 1; l > lwarp && l > Jmin; --l) {
+            // words of level l - 1 from level l
+            int b = 1 << (l - 6), e = 2 * b;
+            if constexpr (SPM != 0) {
+                b = sm.cw_seg[l - 1];
+                e = sm.cw_seg[l];
             }
-            const uint32_t *rol = Ro + sm.woff[l];
-            uint32_t *lfl = LF + sm.woff[l], *prl = PR + sm.woff[l], *ghl = GH + sm.woff[l];
-            const int cb = sm.cw_seg[l], ce = sm.cw_seg[l + 1], wo = sm.woff[l];
-            if (l == d.Jmax) {
-                for (int i = cb + tid; i < ce; i += TS) {
-                    const int wi = cw_at(i) - wo;
-                    uint32_t r = rl[wi];
-                    lfl[wi] = r;
-                    prl[wi] = r & ~rol[wi];
-                    ghl[wi] = 0u;
+#pragma unroll 1
+            for (int i = b + tid; i < e; i += TS) {
+                const uint32_t w = SPM != 0 ? cwl()[i] : (uint32_t)i;
+                const uint32_t x0 = In[2u * w], x1 = In[2u * w + 1u];
+                const uint32_t lo = level_first(w);
+                const bool first = w == lo, last = w + 1u == 2u * lo;
+                uint32_t xl, xr;
+                if (bc == 0) {
+                    xl = In[first ? 4u * lo - 1u : 2u * w - 1u];
+                    xr = In[last ? 2u * lo : 2u * w + 2u];
+                } else {
+                    xl = first ? 0u : In[2u * w - 1u];
+                    xr = last ? 0u : In[2u * w + 2u];
                 }
-            } else if constexpr (WIDE) {
-                const int Wc = Wl << 1;
-                const uint32_t *rc = Rn + sm.woff[l + 1], *pc = PR + sm.woff[l + 1], *gc = GH + sm.woff[l + 1];
-                for (int i = cb + tid; i < ce; i += TS) {
-                    const int wi = cw_at(i) - wo;
-                    const uint32_t r = rl[wi], ro = rol[wi];
-                    const uint32_t lf = r & ~fold2(rc[2 * wi], rc[2 * wi + 1]);
-                    // leaf bits of the 16 cells of each neighbouring word next to this one
-                    const uint32_t cL = word_bc(rc, 2 * wi - 1, Wc, d.bc), cR = word_bc(rc, 2 * wi + 2, Wc, d.bc);
-                    const uint32_t lfL = word_bc(rl, wi - 1, Wl, d.bc) & ~(compact_even(cL | (cL >> 1)) << 16);
-                    const uint32_t lfR = word_bc(rl, wi + 1, Wl, d.bc) & ~compact_even(cR | (cR >> 1));
-                    const uint32_t gw = dilate_edges(lf, lfL, lfR, 2 * g);  // reconstruction windows
-                    const uint32_t pd = dilate_edges(fold2(pc[2 * wi], pc[2 * wi + 1]),
-                                                     fold3(word_bc(pc, 2 * wi - 1, Wc, d.bc) >> 26) << 29,
-                                                     fold3(word_bc(pc, 2 * wi + 2, Wc, d.bc) & 63u), g);
-                    const uint32_t gd = dilate_edges(fold2(gc[2 * wi], gc[2 * wi + 1]),
-                                                     fold3(word_bc(gc, 2 * wi - 1, Wc, d.bc) >> 26) << 29,
-                                                     fold3(word_bc(gc, 2 * wi + 2, Wc, d.bc) & 63u), g);
-                    lfl[wi] = lf;
-                    prl[wi] = (lf | pd) & ~ro;
-                    ghl[wi] = (gw | gd) & ~r;
-                }
-            } else {
-                const int Wc = Wl << 1;
-                const uint32_t *rc = Rn + sm.woff[l + 1], *pc = PR + sm.woff[l + 1], *gc = GH + sm.woff[l + 1];
-                for (int i = cb + tid; i < ce; i += TS) {
-                    const int wi = cw_at(i) - wo;
-                    uint32_t r = rl[wi], ro = rol[wi];
-                    uint32_t lf = r & ~fold2(rc[2 * wi], rc[2 * wi + 1]);
-                    // leaf bits of cells 30, 31 of the left word and 0, 1 of the right word
-                    uint32_t lfL = (word_bc(rl, wi - 1, Wl, d.bc) >> 30) & ~fold_low2(word_bc(rc, 2 * wi - 1, Wc, d.bc) >> 28);
-                    uint32_t lfR = (word_bc(rl, wi + 1, Wl, d.bc) & 3u) & ~fold_low2(word_bc(rc, 2 * wi + 2, Wc, d.bc) & 15u);
-                    uint32_t gw = lf | (lf << 1) | (lf << 2) | (lf >> 1) | (lf >> 2);
-                    gw |= (lfL ? 1u : 0u) | ((lfL & 2u) ? 2u : 0u);                    // from cells 30, 31 on the left
-                    gw |= (lfR ? 0x80000000u : 0u) | ((lfR & 1u) ? 0x40000000u : 0u);  // from cells 0, 1 on the right
-                    uint32_t p = fold2(pc[2 * wi], pc[2 * wi + 1]);
-                    uint32_t pd = dilate1_edges(p, (word_bc(pc, 2 * wi - 1, Wc, d.bc) >> 30) != 0u,
-                                                (word_bc(pc, 2 * wi + 2, Wc, d.bc) & 3u) != 0u);
-                    uint32_t g = fold2(gc[2 * wi], gc[2 * wi + 1]);
-                    uint32_t gd = dilate1_edges(g, (word_bc(gc, 2 * wi - 1, Wc, d.bc) >> 30) != 0u,
-                                                (word_bc(gc, 2 * wi + 2, Wc, d.bc) & 3u) != 0u);
-                    lfl[wi] = lf;
-                    prl[wi] = (lf | pd) & ~ro;
-                    ghl[wi] = (gw | gd) & ~r;
-                }
+                In[w] |= graded_parents(x0, xl, x1, g) | (graded_parents(x1, x0, xr, g) << 16);
             }
             sync();
         }
-        tick(T_GRADE);
-        if (tid == 0 && d.Jmin <= 5) small_levels(Rn, Ro, grade);
+        if (tid < 32) {
+            const int lane = tid;
+            int l = lwarp;
+            uint32_t x0 = 0u;  // the level's 32 cells when l = 5
+            if (l >= 5) {
+                const uint32_t W = 1u << (l - 5);
+                uint32_t x = lane < (int)W ? In[W + lane] : 0u;
+#pragma unroll 1
+                for (; l > 5 && l > Jmin; --l) {
+                    const int n = 1 << (l - 5);
+                    const uint32_t up = lane < n / 2 ? In[n / 2 + lane] : 0u;
+                    uint32_t xl = __shfl_sync(FULL, x, (lane - 1) & (n - 1)), xr = __shfl_sync(FULL, x, (lane + 1) & (n - 1));
+                    if (bc != 0) {
+                        if (lane == 0) xl = 0u;
+                        if (lane == n - 1) xr = 0u;
+                    }
+                    const uint32_t z = graded_parents(x, xl, xr, g);
+                    const uint32_t z0 = __shfl_sync(FULL, z, (2 * lane) & 31), z1 = __shfl_sync(FULL, z, (2 * lane + 1) & 31);
+                    x = up | z0 | (z1 << 16);
+                    if (lane < n / 2) In[n / 2 + lane] = x;
+                }
+                x0 = x;
+            }
+            // level 5 (one word) and the levels of word 0, by lane 0
+            if (lane == 0 && Jmin < 5) {
+                uint32_t y = In[0];
+                if (l == 5) {
+                    const uint32_t e = bc == 0 ? x0 : 0u;
+                    y |= graded_parents(x0, e, e, g) << 16;
+                    l = 4;
+                }
+#pragma unroll 1
+                for (; l > Jmin; --l) {
+                    uint32_t z = y;
+                    for (int s = 0; s < g; ++s) z = dilate_word0(z, bc);
+                    z &= (2u << (2 * (1 << l) - 1)) - (1u << (1 << l));  // the cells of level l
+                    z = (z | (z >> 1)) & 0x55555555u;                    // bit 2p: parent p
+                    y |= compact_even(z);
+                }
+                In[0] = y;
+            }
+        }
         sync();
-    }
-
-    // The levels of at most 32 cells (one word each), coarsest last, by one
-    // thread: grading of level l-1 and the marks of level l as in the word-wise
-    // sweep, with the words of the level below kept in registers rather than
-    // reloaded after the previous level wrote them.
-    __device__ void small_levels(uint32_t *Rn, const uint32_t *Ro, bool grade) {
-        const int gam = WIDE ? d.gamma : 1;
-        // the descriptor fields in registers: a store through a mask pointer
-        // could otherwise force their reload from shared memory at every level
-        const int Jmin = d.Jmin, Jmax = d.Jmax, bc = d.bc;
-        uint32_t *LF = mask(M_LEAF), *PR = mask(M_PRED), *GH = mask(M_GH);
-        const int ltop = Jmax < 5 ? Jmax : 5;
-        // words of level ltop + 1 (two words when it has 64 cells, one when fewer)
-        uint32_t rc0 = 0u, rc1 = 0u, pc0 = 0u, pc1 = 0u, gc0 = 0u, gc1 = 0u;
-        if (ltop < Jmax) {
-            const int oc = sm.woff[ltop + 1];
-            rc0 = Rn[oc];
-            pc0 = PR[oc];
-            gc0 = GH[oc];
-            if (ltop + 1 >= 6) {
-                rc1 = Rn[oc + 1];
-                pc1 = PR[oc + 1];
-                gc1 = GH[oc + 1];
-            }
-        }
-        uint32_t r = Rn[sm.woff[ltop]];
-        int o = sm.woff[ltop];
-        for (int l = ltop; l >= Jmin; --l) {
-            const int n = 1 << l;
-            const int op = l > Jmin ? sm.woff[l - 1] : 0;
-            const uint32_t vb = n == 32 ? 0xFFFFFFFFu : ((1u << n) - 1u);
-            const uint32_t ro = Ro[o];
-            uint32_t rp = l > Jmin ? Rn[op] : 0u;
-            if (grade && l > Jmin + 1) {
-                const int np = n >> 1;
-                const uint32_t vbp = (1u << np) - 1u;
-                rp |= pairexpand(dil_small(fold2(r, 0u), np, gam, bc)) & vbp;
-            }
-            uint32_t lf = r, pr, gh = 0u;
-            if (l < Jmax) {
-                lf = r & ~fold2(rc0, rc1);
-                pr = (lf | dil_small(fold2(pc0, pc1), n, gam, bc)) & ~ro;
-                gh = (dil_small(lf, n, 2 * gam, bc) | dil_small(fold2(gc0, gc1), n, gam, bc)) & ~r;
-            } else {
-                pr = lf & ~ro;
-            }
-            lf &= vb;
-            pr &= vb;
-            gh &= vb;
-            LF[o] = lf;
-            PR[o] = pr;
-            GH[o] = gh;
-            if (l > Jmin) Rn[op] = rp;
-            rc0 = r;
-            rc1 = 0u;
-            pc0 = pr;
-            pc1 = 0u;
-            gc0 = gh;
-            gc1 = 0u;
-            r = rp;
-            o = op;
-        }
-    }
-
-    // dilation by r cells inside a level of n <= 32 cells held in one word
-    __device__ __forceinline__ uint32_t dil_small(uint32_t x, int n, int r, int bc) const {
-        const uint32_t vb = n == 32 ? 0xFFFFFFFFu : ((1u << n) - 1u);
-        uint32_t out = x;
-        for (int s = 1; s <= r; ++s) {
-            if (bc == 0) {
-                // rotations within the level (a wide stencil's reach may exceed n)
-                const int sm_ = WIDE ? s % n : s;
-                if (sm_) out |= ((x << sm_) | (x >> (n - sm_)) | (x >> sm_) | (x << (n - sm_))) & vb;
-            } else {
-                out |= ((x << s) & vb) | (x >> s);
-            }
-        }
-        return out;
-    }
-    // parent bits (n of them) of the child level l+1 of a level of n <= 32 cells
-    __device__ __forceinline__ uint32_t fold_small(const uint32_t *child, int l) const {
-        return l + 1 >= 6 ? fold2(child[0], child[1]) : fold2(child[0], 0u);
     }
 
     // ---- A5: list compaction -------------------------------------------------
-    __device__ __forceinline__ void word_lists(const uint32_t *Rn, int g, int l, uint32_t (&m)[NLIST]) {
-        uint32_t r = Rn[g], lf = mask(M_LEAF)[g];
-        m[L_INT] = r & ~lf;
-        m[L_LEAF] = lf;
-        m[L_PRED] = mask(M_PRED)[g];
-        m[L_GH] = mask(M_GH)[g];
-    }
-
-    // Rounds of TS consecutive candidate words, one word per thread; a block
-    // scan of the per-word counts places each word's entries (the lists stay
-    // sorted by level, then cell).  A dense word costs its owner at most 32
-    // stores per list, and dense levels are spread over as many threads as they
-    // have words.  The occupancy bitmap occn of the listed tree is set on the
-    // way (it must start cleared).
-    __device__ void build_lists(const uint32_t *Rn, uint32_t *occn) {
+    // With the tree graded every list is a word operation: internal cells I,
+    // leaves (children of I outside I), pairs new to the tree I \ I_old, whose
+    // values the transfer predicts (an internal cell among them is its
+    // children's projection at once), and ghost pairs.  The reconstruction
+    // window of a leaf reaches 2 gamma cells, gamma pairs, and so does the
+    // closure of the ghosts under prediction stencils: a ghost within 2 gamma
+    // cells of a tree cell has its parent within gamma of a tree cell and its
+    // stencil within 2 gamma of it; and beyond an internal cell's gamma
+    // neighbours (in the tree) the next cells are within reach of a leaf.  The
+    // ghost pairs are therefore the gamma-dilation of I without I, at every
+    // level but the finest.  (A sweep with its own marks per level, from fine to
+    // coarse, gave the same sets; the marks were a third of the step's bit work.)
+    //
+    // Rounds of TS units; a unit is a word or, when there are fewer words than
+    // threads, a part of one, so that the threads share the entries of dense
+    // words.  A block scan of the units' counts, two counts per 32-bit value,
+    // places the entries (the lists stay sorted).  KEEP and REF, read for the
+    // last time by A3, are cleared on the way.
+    __device__ void build_lists(const uint32_t *In, const uint32_t *Io, uint32_t *occn) {
         constexpr int NW = TS / 32;
         const int lane = tid & 31, warp = tid >> 5;
-        const int ncw = sm.cw_seg[d.Jmax + 1];
-        const bool sparse = sparse_on();
-        int run[NLIST] = {0, 0, 0, 0};
+        const int g = WIDE ? d.gamma : 1;
+        const int nw = nwords();
+        uint32_t *keep = mask(M_KEEP), *ref = mask(M_REF);
+        int s = 0;
+        while (s < 3 && (nw << (s + 1)) <= TS) ++s;
+        const int nu = nw << s, width = 32 >> s;
+        const uint32_t wend = d.Wtot;
+        uint32_t run[NLIST] = {0u, 0u, 0u, 0u};
         if (tid == 0) sm.deplev[0] = sm.deplev[1] = 0u;  // new lists: gathered again by predict_fill
-        for (int r = 0, base = 0; base < ncw; ++r, base += TS) {
-            const int i = base + tid;
-            const bool valid = i < ncw;
-            int l = 0, wi = 0;
-            uint32_t m[NLIST] = {0u, 0u, 0u, 0u};
-            if (valid) {
-                const int g = cw_at(i);
-                level_of_word(sm, g, l, wi);
-                word_lists(Rn, g, l, m);
-                if (sparse && (m[L_INT] | m[L_LEAF])) atomicOr(&occn[sm.ooff[l] + (wi >> 5)], 1u << (wi & 31));
-            }
-            int inc[NLIST];
-#pragma unroll
-            for (int L = 0; L < NLIST; ++L) {
-                int x = __popc(m[L]);
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(FULL, x, o);
-                    if (lane >= o) x += y;
-                }
-                inc[L] = x;
-            }
-            int(*sw)[32] = bx.scan_w[r & 1];  // alternate buffers: one barrier per round
-            if (lane == 31)
-#pragma unroll
-                for (int L = 0; L < NLIST; ++L) sw[L][warp] = inc[L];
-            sync();
-            const uint32_t pk = pack(l, 32LL * wi);
-#pragma unroll
-            for (int L = 0; L < NLIST; ++L) {
-                const int v = lane < NW ? sw[L][lane] : 0;
-                const int before = __reduce_add_sync(FULL, lane < warp ? v : 0);
-                const int tot = __reduce_add_sync(FULL, v);
-                uint32_t x = m[L];
-                int off = run[L] + before + inc[L] - __popc(x);
-                if (valid && i == sm.cw_seg[l]) {
-                    // first candidate word of level l; levels just below without
-                    // candidate words hold no cell and start at the same place
-                    sm.seg[L][l] = off;
-                    for (int k = l - 1; k >= d.Jmin && sm.cw_seg[k] == sm.cw_seg[l]; --k) sm.seg[L][k] = off;
-                }
-                uint32_t *dst = list(L);
-                while (x) {
-                    const int bit = __ffs(x) - 1;
-                    x &= x - 1u;
-                    dst[off++] = pk + (uint32_t)bit;
-                }
-                run[L] += tot;
-            }
-        }
-        if (tid == 0) {
-#pragma unroll
-            for (int L = 0; L < NLIST; ++L) sm.seg[L][d.Jmax + 1] = run[L];
-            // the finest levels without candidate words are empty
-            for (int k = d.Jmax; k >= d.Jmin && sm.cw_seg[k] == ncw; --k)
-#pragma unroll
-                for (int L = 0; L < NLIST; ++L) sm.seg[L][k] = run[L];
-            sm.nleaf = run[L_LEAF];
-        }
-        sync();
-    }
-
-    // ---- the word passes over every word (instances without candidate words) ----
-    __device__ void enlarge_dense(uint32_t *Rn) {
-        const uint32_t *keep = mask(M_KEEP), *ref = mask(M_REF);
-        for (int g = tid; g < d.Wtot; g += TS) {
-            int l, wi;
-            level_of_word(sm, g, l, wi);
-            uint32_t vb = valid_bits(l), rh;
-            if (l == d.Jmin) {
-                rh = vb;
-            } else {
-                const uint32_t *kl = keep + sm.woff[l];
-                uint32_t rt = kl[wi];
-                rh = rt | pairexpand(dilate([&](int j) { return kl[j]; }, l, wi, SIGMA, d.bc));
-                if (l >= d.Jmin + 2) rh |= spread16(ref[sm.woff[l - 1] + (wi >> 1)] >> (16 * (wi & 1)));
-            }
-            Rn[g] = rh & vb;
-        }
-    }
-
-    __device__ void grade_and_mark_dense(uint32_t *Rn, const uint32_t *Ro, bool grade) {
-        uint32_t *LF = mask(M_LEAF), *PR = mask(M_PRED), *GH = mask(M_GH);
-        const int g = d.gamma;
-        const int lbig = d.Jmin > 6 ? d.Jmin : 6;
-        // gamma = 1: the levels of at most 32 words go to one warp (grade_warp)
-        const int lwarp = WIDE ? lbig - 1 : (d.Jmax < 10 ? d.Jmax : 10);
-        for (int l = d.Jmax; l >= lbig && l > lwarp; --l) {
-            const int Wl = 1 << (l - 5);
-            const uint32_t *rl = Rn + sm.woff[l];
-            if (grade && l > d.Jmin + 1) {
-                uint32_t *rp = Rn + sm.woff[l - 1];
-                if constexpr (!WIDE) {
-                    for (int wp = tid; wp < (Wl >> 1); wp += TS) {
-                        uint32_t x = fold2(rl[2 * wp], rl[2 * wp + 1]);
-                        bool eL = (word_bc(rl, 2 * wp - 1, Wl, d.bc) >> 30) != 0u;  // children of parent 32 wp - 1
-                        bool eR = (word_bc(rl, 2 * wp + 2, Wl, d.bc) & 3u) != 0u;   // children of parent 32 wp + 32
-                        rp[wp] |= pairexpand(dilate1_edges(x, eL, eR));
-                    }
-                } else {
-                    for (int wp = tid; wp < (Wl >> 1); wp += TS) {
-                        const uint32_t x = fold2(rl[2 * wp], rl[2 * wp + 1]);
-                        // parents 29..31 of the word on the left, 0..2 of the word on the right
-                        const uint32_t xl = fold3(word_bc(rl, 2 * wp - 1, Wl, d.bc) >> 26) << 29;
-                        const uint32_t xr = fold3(word_bc(rl, 2 * wp + 2, Wl, d.bc) & 63u);
-                        rp[wp] |= pairexpand(dilate_edges(x, xl, xr, g));
-                    }
+#pragma unroll 1
+        for (int r = 0, base = 0; base < nu; ++r, base += TS) {
+            const int u = base + tid;
+            uint32_t m[3] = {0u, 0u, 0u}, lf0 = 0u, lf1 = 0u, w = 0u;
+            const bool whole = u < nu && (u & ((1 << s) - 1)) == 0;  // the first unit of its word
+            if (u < nu) {
+                w = word_at(u >> s);
+                const uint32_t x = In[w], pm = (FULL >> (32 - width)) << ((u & ((1 << s) - 1)) * width);
+                const uint32_t c0 = 2u * w < wend ? In[2u * w] : 0u, c1 = 2u * w + 1u < wend ? In[2u * w + 1u] : 0u;
+                const uint32_t xp = x & pm;
+                m[L_INT] = xp & ~above(w);
+                m[L_PRED] = xp & ~Io[w];
+                if (2u * w < wend || w == 0u) m[L_GH] = dilate_word(In, w, g, bc) & ~x & pm;
+                if (w == 0u) m[L_GH] &= (1u << (Jmax - 1 < 5 ? 1 << (Jmax - 1) : 31)) * (Jmax - 1 < 5 ? 1u : 2u) - 1u;
+                lf0 = spread16(xp) & ~c0;
+                lf1 = spread16(xp >> 16) & ~c1;
+                if (whole) {
+                    keep[w] = 0u;
+                    ref[w] = 0u;
+                    if constexpr (SPM != 0)
+                        if (x) atomicOr(&occn[w >> 5], 1u << (w & 31u));
                 }
             }
-            const uint32_t *rol = Ro + sm.woff[l];
-            uint32_t *lfl = LF + sm.woff[l], *prl = PR + sm.woff[l], *ghl = GH + sm.woff[l];
-            if (l == d.Jmax) {
-                for (int wi = tid; wi < Wl; wi += TS) {
-                    uint32_t r = rl[wi];
-                    lfl[wi] = r;
-                    prl[wi] = r & ~rol[wi];
-                    ghl[wi] = 0u;
-                }
-            } else if constexpr (WIDE) {
-                const int Wc = Wl << 1;
-                const uint32_t *rc = Rn + sm.woff[l + 1], *pc = PR + sm.woff[l + 1], *gc = GH + sm.woff[l + 1];
-                for (int wi = tid; wi < Wl; wi += TS) {
-                    const uint32_t r = rl[wi], ro = rol[wi];
-                    const uint32_t lf = r & ~fold2(rc[2 * wi], rc[2 * wi + 1]);
-                    // leaf bits of the 16 cells of each neighbouring word next to this one
-                    const uint32_t cL = word_bc(rc, 2 * wi - 1, Wc, d.bc), cR = word_bc(rc, 2 * wi + 2, Wc, d.bc);
-                    const uint32_t lfL = word_bc(rl, wi - 1, Wl, d.bc) & ~(compact_even(cL | (cL >> 1)) << 16);
-                    const uint32_t lfR = word_bc(rl, wi + 1, Wl, d.bc) & ~compact_even(cR | (cR >> 1));
-                    const uint32_t gw = dilate_edges(lf, lfL, lfR, 2 * g);  // reconstruction windows
-                    const uint32_t pd = dilate_edges(fold2(pc[2 * wi], pc[2 * wi + 1]),
-                                                     fold3(word_bc(pc, 2 * wi - 1, Wc, d.bc) >> 26) << 29,
-                                                     fold3(word_bc(pc, 2 * wi + 2, Wc, d.bc) & 63u), g);
-                    const uint32_t gd = dilate_edges(fold2(gc[2 * wi], gc[2 * wi + 1]),
-                                                     fold3(word_bc(gc, 2 * wi - 1, Wc, d.bc) >> 26) << 29,
-                                                     fold3(word_bc(gc, 2 * wi + 2, Wc, d.bc) & 63u), g);
-                    lfl[wi] = lf;
-                    prl[wi] = (lf | pd) & ~ro;
-                    ghl[wi] = (gw | gd) & ~r;
-                }
-            } else {
-                const int Wc = Wl << 1;
-                const uint32_t *rc = Rn + sm.woff[l + 1], *pc = PR + sm.woff[l + 1], *gc = GH + sm.woff[l + 1];
-                for (int wi = tid; wi < Wl; wi += TS) {
-                    uint32_t r = rl[wi], ro = rol[wi];
-                    uint32_t lf = r & ~fold2(rc[2 * wi], rc[2 * wi + 1]);
-                    // leaf bits of cells 30, 31 of the left word and 0, 1 of the right word
-                    uint32_t lfL = (word_bc(rl, wi - 1, Wl, d.bc) >> 30) & ~fold_low2(word_bc(rc, 2 * wi - 1, Wc, d.bc) >> 28);
-                    uint32_t lfR = (word_bc(rl, wi + 1, Wl, d.bc) & 3u) & ~fold_low2(word_bc(rc, 2 * wi + 2, Wc, d.bc) & 15u);
-                    uint32_t gw = lf | (lf << 1) | (lf << 2) | (lf >> 1) | (lf >> 2);
-                    gw |= (lfL ? 1u : 0u) | ((lfL & 2u) ? 2u : 0u);                    // from cells 30, 31 on the left
-                    gw |= (lfR ? 0x80000000u : 0u) | ((lfR & 1u) ? 0x40000000u : 0u);  // from cells 0, 1 on the right
-                    uint32_t p = fold2(pc[2 * wi], pc[2 * wi + 1]);
-                    uint32_t pd = dilate1_edges(p, (word_bc(pc, 2 * wi - 1, Wc, d.bc) >> 30) != 0u,
-                                                (word_bc(pc, 2 * wi + 2, Wc, d.bc) & 3u) != 0u);
-                    uint32_t g = fold2(gc[2 * wi], gc[2 * wi + 1]);
-                    uint32_t gd = dilate1_edges(g, (word_bc(gc, 2 * wi - 1, Wc, d.bc) >> 30) != 0u,
-                                                (word_bc(gc, 2 * wi + 2, Wc, d.bc) & 3u) != 0u);
-                    lfl[wi] = lf;
-                    prl[wi] = (lf | pd) & ~ro;
-                    ghl[wi] = (gw | gd) & ~r;
-                }
-            }
-            sync();
-        }
-        if constexpr (!WIDE)
-            if (tid < 32 && lwarp >= lbig) grade_warp(Rn, Ro, grade, lwarp, lbig);
-        tick(T_GRADE);
-        if (tid == 0 && d.Jmin <= 5) small_levels(Rn, Ro, grade);
-        sync();
-    }
-
-    // Grading and marking of the levels ltop .. lbot of at most 32 words each
-    // (gamma = 1) by one warp, without block barriers: lane i holds word i of
-    // the current level and words 2i, 2i + 1 of the level below it (R, PR, GH)
-    // in registers, neighbouring and child words arrive by shuffles (wrapped
-    // or empty beyond the domain, as word_bc), and the results are stored for
-    // the list compaction and the small levels.  The same operations as the
-    // block-wide sweep, level for level.
-    __device__ __noinline__ void grade_warp(uint32_t *Rn, const uint32_t *Ro, bool grade, int ltop, int lbot) {
-        uint32_t *LF = mask(M_LEAF), *PR = mask(M_PRED), *GH = mask(M_GH);
-        const int lane = tid;  // tid < 32
-        const int bc = d.bc;
-        const int Wt = 1 << (ltop - 5);
-        // words 2 lane, 2 lane + 1 of level ltop + 1 (final: graded and marked by the block)
-        uint32_t rc0 = 0u, rc1 = 0u, pc0 = 0u, pc1 = 0u, gc0 = 0u, gc1 = 0u;
-        if (ltop < d.Jmax && lane < Wt) {
-            const int o = sm.woff[ltop + 1] + 2 * lane;
-            rc0 = Rn[o];
-            rc1 = Rn[o + 1];
-            pc0 = PR[o];
-            pc1 = PR[o + 1];
-            gc0 = GH[o];
-            gc1 = GH[o + 1];
-        }
-        uint32_t r = lane < Wt ? Rn[sm.woff[ltop] + lane] : 0u;  // level ltop, graded from ltop + 1
-        for (int l = ltop; l >= lbot; --l) {
-            const int Wl = 1 << (l - 5);  // 2 .. 32 words
-            const bool act = lane < Wl;
-            const uint32_t ro = act ? Ro[sm.woff[l] + lane] : 0u;
-            // word j of a level of Wl words whose word q lane q holds in v
-            auto word = [&](uint32_t v, int j) -> uint32_t {
-                const bool out = j < 0 || j >= Wl;
-                const int src = bc == 0 ? ((j + Wl) & (Wl - 1)) : (out ? 0 : j);
-                const uint32_t x = __shfl_sync(FULL, v, src);
-                return (bc != 0 && out) ? 0u : x;
-            };
-            // grading of level l - 1: parent word wp = lane from words 2wp - 1 .. 2wp + 2 of level l
-            const uint32_t c0 = word(r, 2 * lane), c1 = word(r, 2 * lane + 1);
-            const uint32_t cL = word(r, 2 * lane - 1), cR = word(r, 2 * lane + 2);
-            uint32_t rpn = 0u;
-            if (l > d.Jmin) {
-                const int Wp = Wl >> 1;
-                uint32_t hp = lane < Wp ? Rn[sm.woff[l - 1] + lane] : 0u;  // enlarged set of level l - 1
-                if (grade && l > d.Jmin + 1 && lane < Wp)
-                    hp |= pairexpand(dilate1_edges(fold2(c0, c1), (cL >> 30) != 0u, (cR & 3u) != 0u));
-                if (lane < Wp) Rn[sm.woff[l - 1] + lane] = hp;
-                rpn = lane < Wp ? hp : 0u;
-            }
-            // leaf, transfer and ghost marks of level l
-            uint32_t lf, pr, gh = 0u;
-            if (l == d.Jmax) {
-                lf = r;
-                pr = r & ~ro;
-            } else {
-                const uint32_t rl0 = word(r, lane - 1), rl1 = word(r, lane + 1);
-                const uint32_t rcL = word(rc1, lane - 1), rcR = word(rc0, lane + 1);  // words 2 lane - 1, 2 lane + 2 below
-                const uint32_t pcL = word(pc1, lane - 1), pcR = word(pc0, lane + 1);
-                const uint32_t gcL = word(gc1, lane - 1), gcR = word(gc0, lane + 1);
-                lf = r & ~fold2(rc0, rc1);
-                const uint32_t lfL = (rl0 >> 30) & ~fold_low2(rcL >> 28);
-                const uint32_t lfR = (rl1 & 3u) & ~fold_low2(rcR & 15u);
-                uint32_t gw = lf | (lf << 1) | (lf << 2) | (lf >> 1) | (lf >> 2);
-                gw |= (lfL ? 1u : 0u) | ((lfL & 2u) ? 2u : 0u);
-                gw |= (lfR ? 0x80000000u : 0u) | ((lfR & 1u) ? 0x40000000u : 0u);
-                const uint32_t pd = dilate1_edges(fold2(pc0, pc1), (pcL >> 30) != 0u, (pcR & 3u) != 0u);
-                const uint32_t gd = dilate1_edges(fold2(gc0, gc1), (gcL >> 30) != 0u, (gcR & 3u) != 0u);
-                pr = (lf | pd) & ~ro;
-                gh = (gw | gd) & ~r;
-            }
-            if (act) {
-                const int o = sm.woff[l] + lane;
-                LF[o] = lf;
-                PR[o] = pr;
-                GH[o] = gh;
-            }
-            // the next level (l - 1): its lane i holds words 2i, 2i + 1 of level l
-            rc0 = c0;
-            rc1 = c1;
-            pc0 = __shfl_sync(FULL, pr, (2 * lane) & 31);
-            pc1 = __shfl_sync(FULL, pr, (2 * lane + 1) & 31);
-            gc0 = __shfl_sync(FULL, gh, (2 * lane) & 31);
-            gc1 = __shfl_sync(FULL, gh, (2 * lane + 1) & 31);
-            r = rpn;
-        }
-        __syncwarp();
-    }
-
-    __device__ void build_lists_dense(const uint32_t *Rn) {
-        constexpr int NW = TS / 32;
-        const int lane = tid & 31, warp = tid >> 5;
-        const int Wtot = d.Wtot;
-        int run[NLIST] = {0, 0, 0, 0};
-        if (tid == 0) sm.deplev[0] = sm.deplev[1] = 0u;  // new lists: gathered again by predict_fill
-        for (int r = 0, base = 0; base < Wtot; ++r, base += TS) {
-            const int g = base + tid;
-            const bool valid = g < Wtot;
-            int l = 0, wi = 0;
-            uint32_t m[NLIST] = {0u, 0u, 0u, 0u};
-            if (valid) {
-                level_of_word(sm, g, l, wi);
-                word_lists(Rn, g, l, m);
-            }
-            // the four lists' counts two per value, in 16-bit fields (a round's
-            // totals are at most 1024 x 32 < 2^16): half the scan steps and reductions
+            // per round at most 1024 x 32 internal cells and new pairs (16 bits
+            // each), 1024 x 64 leaves (17 bits), 1024 x 16 ghost pairs (15 bits)
             uint32_t x01 = (uint32_t)__popc(m[0]) | ((uint32_t)__popc(m[1]) << 16);
-            uint32_t x23 = (uint32_t)__popc(m[2]) | ((uint32_t)__popc(m[3]) << 16);
+            uint32_t x23 = (uint32_t)(__popc(lf0) + __popc(lf1)) | ((uint32_t)__popc(m[2]) << 17);
+            const uint32_t c01 = x01, c23 = x23;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y01 = __shfl_up_sync(FULL, x01, o), y23 = __shfl_up_sync(FULL, x23, o);
@@ -1720,104 +1194,121 @@ struct Worker {
                     x23 += y23;
                 }
             }
-            int(*sw)[32] = bx.scan_w[r & 1];  // alternate buffers: one barrier per round
+            uint32_t(*sw)[32] = bx.scan_w[r & 1];  // alternate buffers: one barrier per round
             if (lane == 31) {
-                sw[0][warp] = (int)x01;
-                sw[1][warp] = (int)x23;
+                sw[0][warp] = x01;
+                sw[1][warp] = x23;
             }
             sync();
-            const uint32_t v01 = lane < NW ? (uint32_t)sw[0][lane] : 0u, v23 = lane < NW ? (uint32_t)sw[1][lane] : 0u;
-            const uint32_t b01 = __reduce_add_sync(FULL, lane < warp ? v01 : 0u);
-            const uint32_t b23 = __reduce_add_sync(FULL, lane < warp ? v23 : 0u);
+            const uint32_t v01 = lane < NW ? sw[0][lane] : 0u, v23 = lane < NW ? sw[1][lane] : 0u;
+            x01 += __reduce_add_sync(FULL, lane < warp ? v01 : 0u) - c01;
+            x23 += __reduce_add_sync(FULL, lane < warp ? v23 : 0u) - c23;
             const uint32_t t01 = __reduce_add_sync(FULL, v01), t23 = __reduce_add_sync(FULL, v23);
-            const int inc[NLIST] = {(int)(x01 & 0xFFFFu), (int)(x01 >> 16), (int)(x23 & 0xFFFFu), (int)(x23 >> 16)};
-            const int before[NLIST] = {(int)(b01 & 0xFFFFu), (int)(b01 >> 16), (int)(b23 & 0xFFFFu), (int)(b23 >> 16)};
-            const int tot[NLIST] = {(int)(t01 & 0xFFFFu), (int)(t01 >> 16), (int)(t23 & 0xFFFFu), (int)(t23 >> 16)};
-            const uint32_t pk = pack(l, 32LL * wi);
+            const uint32_t at[3] = {run[0] + (x01 & 0xFFFFu), run[1] + (x01 >> 16), run[2] + (x23 >> 17)};
+            if (whole && w > 0u) {
+                // the first word of a level; a candidate list may leave whole levels out
+                const int l = 5 + level_of(w);
+                int k = l;
+                if constexpr (SPM != 0) {
+                    const uint32_t before = word_at((u >> s) - 1);  // a list starts with words 0, 1, ...
+                    k = before == 0u ? 5 : 6 + level_of(before);
+                } else if ((w & (w - 1u)) != 0u)
+                    k = l + 1;
+                for (; k <= l; ++k)
 #pragma unroll
-            for (int L = 0; L < NLIST; ++L) {
-                uint32_t x = m[L];
-                int off = run[L] + before[L] + inc[L] - __popc(x);
-                if (valid && wi == 0) sm.seg[L][l] = off;
-                uint32_t *dst = list(L);
-                while (x) {
-                    const int bit = __ffs(x) - 1;
-                    x &= x - 1u;
-                    dst[off++] = pk + (uint32_t)bit;
-                }
-                run[L] += tot[L];
+                    for (int L = 0; L < NSEG; ++L) sm.seg[L][k] = at[L];
             }
+            const uint32_t h0 = 32u * w;
+#pragma unroll
+            for (int L = 0; L < NSEG; ++L) {
+                uint32_t *dst = list(L) + at[L];
+                uint32_t x = m[L];
+#pragma unroll 1
+                while (x) {
+                    *dst++ = h0 + (uint32_t)__ffs(x) - 1u;
+                    x &= x - 1u;
+                }
+            }
+            {
+                uint32_t *dst = list(L_LEAF) + run[3] + (x23 & 0x1FFFFu);
+#pragma unroll 1
+                while (lf0) {
+                    *dst++ = 2u * h0 + (uint32_t)__ffs(lf0) - 1u;
+                    lf0 &= lf0 - 1u;
+                }
+#pragma unroll 1
+                while (lf1) {
+                    *dst++ = 2u * h0 + 31u + (uint32_t)__ffs(lf1);
+                    lf1 &= lf1 - 1u;
+                }
+            }
+            run[0] += t01 & 0xFFFFu;
+            run[1] += t01 >> 16;
+            run[2] += t23 >> 17;
+            run[3] += t23 & 0x1FFFFu;
         }
         if (tid == 0) {
+            // the end of the finest level (and of the levels that no candidate word reached)
+            int k = top();
+            if constexpr (SPM != 0) k = 6 + level_of(word_at(nw - 1));
+            for (; k <= top(); ++k)
 #pragma unroll
-            for (int L = 0; L < NLIST; ++L) sm.seg[L][d.Jmax + 1] = run[L];
-            sm.nleaf = run[L_LEAF];
+                for (int L = 0; L < NSEG; ++L) sm.seg[L][k] = run[L];
+            sm.nleaf = run[3];
         }
         sync();
     }
 
-    // ---- A6 / S3: prediction of listed cells, coarse to fine -----------------
-    // predicts the listed cell ent (level l) from level l - 1
-    __device__ __forceinline__ void predict_entry(uint32_t ent, int l) {
-        {
-            const long long k = ent & KMASK;
-            T v[QMAX];
-            if constexpr (!WIDE) {
+    // ---- A6 / S3: prediction of listed pairs ----------------------------------
+    // the children of p from p's level, whose first cell is lo (Section 3.1)
+    __device__ __forceinline__ void predict_pair(uint32_t p, uint32_t lo) const {
+        T a[2 * q];
+        const T *vp = cell(p), *vl = cell(nb(p, -1, lo)), *vr = cell(nb(p, 1, lo));
 #pragma unroll
-                for (int h = 0; h < QMAX; ++h)
-                    if (h < q) v[h] = predict<T>(row(h, l - 1), k >> 1, (int)(k & 1), l - 1, d.bc);
-            } else {
-#pragma unroll
-                for (int h = 0; h < QMAX; ++h)
-                    if (h < q)
-                        v[h] = predict_g<T>(row(h, l - 1), k >> 1, (int)(k & 1), l - 1, d.bc, d.gamma, tab.pc[d.gamma]);
-            }
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) row(h, l)[k] = v[h];
+        for (int h = 0; h < q; ++h) {
+            T t = T(C1) * (vr[h] - vl[h]);  // exact: c_1 is a power of two
+            if constexpr (WIDE) t = wide_sum(p, lo, h, t);
+            a[h] = vp[h] + t;
+            a[q + h] = vp[h] - t;
         }
+        store_cell(2u * p, a);
+        store_cell(2u * p + 1u, a + q);
     }
-
-    // whether the prediction stencil of cell (l, k) at level l - 1 (parent +-
-    // gamma, wrapped or clamped as the prediction does) holds a cell marked in P
-    __device__ __forceinline__ bool stencil_marked(const uint32_t *P, int l, long long k) const {
-        const int gg = WIDE ? d.gamma : 1, lp = l - 1;
-        const uint32_t *pl = P + sm.woff[lp];
-        const long long p = k >> 1;
-        bool hit = false;
-        for (int a = -gg; a <= gg; ++a) {
-            const long long c = wrapc(p + a, lp, d.bc);
-            hit |= ((pl[c >> 5] >> (c & 31)) & 1u) != 0u;
-        }
-        return hit;
+    // whether the stencil of the pair's prediction holds a cell outside the tree I
+    __device__ __forceinline__ bool stencil_outside(const uint32_t *I, uint32_t p, uint32_t lo) const {
+        const int g = WIDE ? d.gamma : 1;
+        bool all = true;
+        for (int a = -g; a <= g; ++a) all = all && bit_of(I, nb(p, a, lo) >> 1);
+        return !all;
     }
-
-    // A6 / S3.  A listed cell whose stencil holds no cell of the same list reads
-    // only tree values (the old tree for the transfer, the current tree for the
-    // ghosts: the marking closes both lists under prediction stencils), so those
-    // cells go in one pass over all levels; the rest follow level by level,
-    // coarse to fine, on the levels that have any.  The marks of both lists stay
-    // in their masks until the next step's A2 clears them.
-    __device__ void predict_fill(int L) {
+    // A listed pair whose stencil lies in the tree I (the old tree for the
+    // transfer, the current one for the ghosts) reads only tree values, so those
+    // pairs go in one pass over all levels; the others, whose stencils hold
+    // pairs of the same list, follow level by level, coarse to fine, on the
+    // levels that have any.
+    __device__ void predict_fill(int L, const uint32_t *I) {
         const uint32_t *lst = list(L);
-        const uint32_t *P = mask(L == L_GH ? M_GH : M_PRED);
-        const int slot = L == L_GH ? 1 : 0;
-        const int b = sm.seg[L][d.Jmin + 1], e = sm.seg[L][d.Jmax + 1];
-        for (int i = b + tid; i < e; i += TS) {
-            const uint32_t ent = lst[i];
-            const int l = (int)(ent >> KBITS);
-            if (stencil_marked(P, l, ent & KMASK))
-                atomicOr(&sm.deplev[slot], 1u << l);
+        uint32_t *dep = &sm.deplev[L == L_GH ? 1 : 0];
+        const int n = sm.seg[L][top()];
+#pragma unroll 1
+        for (int i = tid; i < n; i += TS) {
+            const uint32_t p = lst[i], lo = level_first(p);
+            if (stencil_outside(I, p, lo))
+                atomicOr(dep, lo);
             else
-                predict_entry(ent, l);
+                predict_pair(p, lo);
         }
         sync();
-        const uint32_t lv = sm.deplev[slot];
-        for (int l = d.Jmin + 1; l <= d.Jmax; ++l) {
-            if (!((lv >> l) & 1u)) continue;
-            for (int i = sm.seg[L][l] + tid; i < sm.seg[L][l + 1]; i += TS) {
-                const uint32_t ent = lst[i];
-                if (stencil_marked(P, l, ent & KMASK)) predict_entry(ent, l);
+        uint32_t lv = *dep;
+#pragma unroll 1
+        while (lv) {
+            const int l = __ffs(lv) - 1;
+            lv &= lv - 1u;
+            const int b = l >= 5 ? sm.seg[L][l] : 0, e = sm.seg[L][l >= 5 ? l + 1 : 5];
+#pragma unroll 1
+            for (int i = b + tid; i < e; i += TS) {
+                const uint32_t p = lst[i], lo = 1u << l;
+                if (level_of(p) == l && stencil_outside(I, p, lo)) predict_pair(p, lo);
             }
             sync();
         }
@@ -1825,49 +1316,37 @@ struct Worker {
 
     // ---- mesh adaptation ----------------------------------------------------
     __device__ void adapt() {
-        uint32_t *Ro = mask(sm.cur), *Rn = mask(sm.cur ^ 1);
+        uint32_t *Io = mask(sm.cur), *In = mask(sm.cur ^ 1);
         tick(NPHASE);
-        if (sparse_on()) build_cw();
-        {
-            // the transfer / ghost marks of the last list compaction share storage
-            // with KEEP / REF, which A2 accumulates into: clear them (all of them
-            // lie in candidate words; the barrier of A1 orders this before A2),
-            // and the occupancy bitmap the list compaction will fill
-            uint32_t *pr = mask(M_PRED), *gh = mask(M_GH);
-            const int ncw = sm.cw_seg[d.Jmax + 1];
-            for (int i = tid; i < ncw; i += TS) {
-                const int g = cw_at(i);
-                pr[g] = 0u;
-                gh[g] = 0u;
-            }
-            if (sparse_on()) {
-                uint32_t *on = occ(sm.cur ^ 1);
-                for (int g = tid; g < d.OW; g += TS) on[g] = 0u;
-            }
+        if constexpr (SPM != 0) {
+            build_cw();
+            uint32_t *on = occ(sm.cur ^ 1);  // the occupancy array the list compaction will fill
+#pragma unroll 1
+            for (int j = tid; j < d.OW; j += TS) on[j] = 0u;
         }
         tick(T_CANDIDATES);
         // internal cells: already projected by the last stream (D1Q2^n), else level by level
         if (DQ || !(sm.status & ST_FLUXED)) upsweep();
-        sync();
         tick(T_UPSWEEP_A);
         details();
         sync();
         tick(T_DETAILS);
-        if (sparse_on()) enlarge(Rn); else enlarge_dense(Rn);
+        enlarge(In);
         sync();
         tick(T_ENLARGE);
-        if (sparse_on()) grade_and_mark(Rn, Ro, true); else grade_and_mark_dense(Rn, Ro, true);
-        tick(T_GRADE_SMALL);
-        if (sparse_on()) build_lists(Rn, occ(sm.cur ^ 1)); else build_lists_dense(Rn);
+        grade(In);
+        tick(T_GRADE);
+        build_lists(In, Io, SPM != 0 ? occ(sm.cur ^ 1) : nullptr);
         tick(T_LISTS);
-        predict_fill(L_PRED);
-        if (sparse_on()) {
+        predict_fill(L_PRED, Io);
+        if constexpr (SPM != 0) {
             // the old tree's buffer holds the next step's new tree: clear it (its
-            // cells lie in candidate words; nothing reads it after the grading);
-            // without candidate words the enlargement writes every word
+            // cells lie in candidate words); without candidate words the
+            // enlargement writes every word
             const uint32_t *cw = cwl();
-            const int ncw = sm.cw_seg[d.Jmax + 1];
-            for (int i = tid; i < ncw; i += TS) Ro[cw[i]] = 0u;
+            const int ncw = sm.ncw;
+#pragma unroll 1
+            for (int i = tid; i < ncw; i += TS) Io[cw[i]] = 0u;
         }
         tick(T_TRANSFER);
         if (tid == 0) {
@@ -1887,172 +1366,195 @@ struct Worker {
             else
                 collide_all();
         } else {
-            collide_all();      // S1
+            collide_all();  // S1
         }
         sync();
         tick(T_COLLIDE);
-        upsweep();              // S2
+        upsweep();  // S2
         tick(T_UPSWEEP_S);
-        predict_fill(L_GH);     // S3
+        predict_fill(L_GH, mask(sm.cur));  // S3
         tick(T_GHOSTS);
-        reconstruct_edges();    // S4
+        if constexpr (DQ)
+            reconstruct_dq();  // S4 (gamma = 1)
+        else if (WIDE && d.gamma > 1)
+            reconstruct_wide();
+        else
+            reconstruct_edges();
         sync();
         tick(T_RECON);
-        stream_and_audit();     // S5
+        if constexpr (DQ)
+            stream_dq();  // S5
+        else
+            stream_and_audit();
         tick(T_STREAM);
     }
 
-    // S4: first / last finest-cell values of every leaf -> Phi
-    __device__ void reconstruct_edges() {
-        if constexpr (DQ) {
-            reconstruct_dq();  // gamma = 1 (the tables)
-            return;
-        }
-        if constexpr (WIDE) {
-            if (d.gamma > 1) {
-                reconstruct_wide();
-                return;
-            }
-        }
-        const uint32_t *R = mask(sm.cur);
-        const uint32_t *leaves = list(L_LEAF);
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            uint32_t ent = leaves[i];
-            int l = ent >> KBITS;
-            long long k = ent & KMASK;
-            const int dj = d.Jmax - l;
-            const long long nl = 1LL << l;
-            bool at_left = d.bc == 1 && k == 0, at_right = d.bc == 1 && k == nl - 1;
-            bool fin_l = false, fin_r = false;
-            if (dj > 0) {
-                const uint32_t *rf = R + sm.woff[l + 1];
-                if (!at_left) {
-                    long long c = 2 * wrapc(k - 1, l, d.bc);
-                    fin_l = (rf[c >> 5] >> (c & 31)) & 1u;
-                }
-                if (!at_right) {
-                    long long c = 2 * wrapc(k + 1, l, d.bc);
-                    fin_r = (rf[c >> 5] >> (c & 31)) & 1u;
-                }
-            }
-            const T *cf = tab.cf[dj], *t1 = tab.t1[dj], *bf = tab.bf[dj];
+    // sum of four products; FP32: compensated (Kahan) accumulation
+    static __device__ __forceinline__ T dot4(const T *w, T x0, T x1, T x2, T x3) {
+        if constexpr (sizeof(T) == 8) {
+            return fma(w[3], x3, fma(w[2], x2, fma(w[1], x1, w[0] * x0)));
+        } else {
+            T p[4] = {w[0] * x0, w[1] * x1, w[2] * x2, w[3] * x3};
+            T s = T(0), comp = T(0);
 #pragma unroll
-            for (int h = 0; h < QMAX; ++h) {
-                if (h >= q) break;
-                const auto r = row(h, l);
-                const bool plus = (h & 1) == 0;  // velocity +lambda
-                bool need_first = !plus || at_left, need_last = plus || at_right;
-                T rfirst = T(0), rlast = T(0);
-                if (dj == 0) {
-                    rfirst = rlast = r[k];
-                } else {
-                    T vm1 = r[wrapc(k - 1, l, d.bc)], v0 = r[k], vp1 = r[wrapc(k + 1, l, d.bc)];
-                    const auto rf = row(h, l + 1);
-                    // one sum of four products for both stencils, so that a warp whose
-                    // leaves mix them evaluates it once: next to a finer neighbour the
-                    // leaf's own children (predicted) enter with the weights t1, else
-                    // the cells of level l with the weights cf
-                    if (need_first) {
-                        if (at_left) {
-                            rfirst = bf[0] * v0 + bf[1] * vp1;
-                        } else {
-                            T x0, x1, x2, x3;
-                            const T *wt;
-                            if (fin_l) {
-                                const T tt = T(C1) * (vp1 - vm1);
-                                const long long c = 2 * wrapc(k - 1, l, d.bc);
-                                x0 = rf[c];
-                                x1 = rf[c + 1];
-                                x2 = v0 + tt;
-                                x3 = v0 - tt;
-                                wt = t1;
-                            } else {
-                                x0 = r[wrapc(k - 2, l, d.bc)];
-                                x1 = vm1;
-                                x2 = v0;
-                                x3 = vp1;
-                                wt = cf;
-                            }
-                            rfirst = dot4(wt[0], x0, wt[1], x1, wt[2], x2, wt[3], x3);
-                        }
-                    }
-                    if (need_last) {
-                        if (at_right) {
-                            rlast = bf[0] * v0 + bf[1] * vm1;
-                        } else {
-                            T x0, x1, x2, x3;
-                            const T *wt;
-                            if (fin_r) {
-                                const T tt = T(C1) * (vp1 - vm1);
-                                const long long c = 2 * wrapc(k + 1, l, d.bc);
-                                x0 = v0 + tt;
-                                x1 = v0 - tt;
-                                x2 = rf[c];
-                                x3 = rf[c + 1];
-                                wt = t1;
-                            } else {
-                                x0 = vm1;
-                                x1 = v0;
-                                x2 = vp1;
-                                x3 = r[wrapc(k + 2, l, d.bc)];
-                                wt = cf;
-                            }
-                            rlast = dot4(wt[3], x0, wt[2], x1, wt[1], x2, wt[0], x3);
-                        }
-                    }
+            for (int j = 0; j < 4; ++j) {
+                T y = p[j] - comp;
+                T t = s + y;
+                comp = (t - s) - y;
+                s = t;
+            }
+            return s;
+        }
+    }
+
+    // S4: first / last finest-cell values of every leaf -> Phi, from the
+    // per-level-gap tables.  One sum of four products for both stencils, so that
+    // a warp whose leaves mix them evaluates it once: next to a finer neighbour
+    // the leaf's own children (predicted) enter with the weights t1, else the
+    // cells of the leaf's level with the weights cf; the mirrored sum for the
+    // last value.
+    __device__ void reconstruct_edges() {
+        const uint32_t *I = mask(sm.cur);
+        const uint32_t *leaves = list(L_LEAF);
+        const int nl = sm.nleaf;
+        const uint32_t N = 1u << Jmax;
+#pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            const uint32_t h = leaves[i], lo = level_first(h);
+            const int dj = Jmax - level_of(h);
+            const uint32_t hl = nb(h, -1, lo), hr = nb(h, 1, lo);
+            const bool at_left = bc == 1 && h == lo, at_right = bc == 1 && h + 1u == 2u * lo;
+            const uint32_t first = (h << dj) & (N - 1u);
+            uint32_t next = first + (1u << dj);
+            if (bc == 0) next &= N - 1u;
+            T *pf = phi(first), *pn = phi(next);
+            if (dj == 0) {
+                const T *v = cell(h);
+#pragma unroll
+                for (int j = 0; j < NF; ++j) {
+                    const T vp = v[2 * j], vm = v[2 * j + 1];
+                    pn[2 * j] = vp;
+                    pf[2 * j + 1] = vm;
+                    if (at_left) pf[2 * j] = vp;
+                    if (at_right) pn[2 * j + 1] = vm;
                 }
-                const auto ph = phi(h);
-                if (plus) {
-                    long long ix = (k + 1) << dj;
-                    if (d.bc == 0) ix &= d.N - 1;
-                    ph[ix] = rlast;
-                    if (at_left) ph[0] = rfirst;
-                } else {
-                    ph[k << dj] = rfirst;
-                    if (at_right) ph[d.N] = rlast;
+                continue;
+            }
+            const bool fin_l = !at_left && bit_of(I, hl), fin_r = !at_right && bit_of(I, hr);
+            // where the two outer values of each sum come from
+            const T *l0 = fin_l ? cell(2u * hl) : cell(nb(h, -2, lo)), *l1 = fin_l ? cell(2u * hl + 1u) : cell(hl);
+            const T *r0 = fin_r ? cell(2u * hr) : cell(hr), *r1 = fin_r ? cell(2u * hr + 1u) : cell(nb(h, 2, lo));
+            const T *vm1 = cell(hl), *v0 = cell(h), *vp1 = cell(hr);
+            const T *wl = fin_l ? tab.t1[dj] : tab.cf[dj], *wr = fin_r ? tab.t1[dj] : tab.cf[dj], *bf = tab.bf[dj];
+            const T wm[4] = {wr[3], wr[2], wr[1], wr[0]};
+#pragma unroll
+            for (int j = 0; j < NF; ++j) {
+                {  // velocity +lambda: the last value (and the first at the left boundary)
+                    const int c = 2 * j;
+                    const T a = vm1[c], b = v0[c], e = vp1[c];
+                    T x0 = a, x1 = b;
+                    if (fin_r) {
+                        const T tt = T(C1) * (e - a);
+                        x0 = b + tt;
+                        x1 = b - tt;
+                    }
+                    pn[c] = at_right ? bf[0] * b + bf[1] * a : dot4(wm, x0, x1, r0[c], r1[c]);
+                    if (at_left) pf[c] = bf[0] * b + bf[1] * e;
+                }
+                {  // velocity -lambda: the first value (and the last at the right boundary)
+                    const int c = 2 * j + 1;
+                    const T a = vm1[c], b = v0[c], e = vp1[c];
+                    T x2 = b, x3 = e;
+                    if (fin_l) {
+                        const T tt = T(C1) * (e - a);
+                        x2 = b + tt;
+                        x3 = b - tt;
+                    }
+                    pf[c] = at_left ? bf[0] * b + bf[1] * e : dot4(wl, l0[c], l1[c], x2, x3);
+                    if (at_right) pn[c] = bf[0] * b + bf[1] * a;
                 }
             }
         }
+    }
+
+    // First (LAST = false) or last finest value of population c of the leaf h,
+    // by the reconstruction operator of Section 3.3 (Definition V): the window
+    // h - 2G .. h + 2G (tree and ghost values) is predicted level by level down
+    // to Jmax around the leaf's first (last) finest cell, and wherever a finer
+    // level holds a cell of the tree (the children of refined neighbours) its
+    // value is used instead.  Out-of-domain cells take the value of the nearest
+    // domain cell (copy boundary) or wrap (periodic), as in the prediction.
+    template <int G, bool LAST>
+    __device__ __noinline__ T edge_walk(const uint32_t *I, const T *cf, int c, uint32_t h) const {
+        constexpr int W = 4 * G + 1, C = 2 * G, E = LAST ? 1 : 0;
+        T w[W], nw[W];
+        uint32_t lo = level_first(h);
+#pragma unroll
+        for (int t = 0; t < W; ++t) w[t] = cell(nb(h, t - C, lo))[c];
+#pragma unroll 1
+        for (int m = level_of(h); m < Jmax; ++m) {
+            h = 2u * h + E;
+            lo *= 2u;
+            T vlo = T(0), vhi = T(0);  // values of the first and last cells of the level (copy boundary)
+#pragma unroll
+            for (int t = 0; t < W; ++t) {
+                // window position t is cell h + t - C; its parent is window position pp of the level above
+                const int pp = C + ((E + t - C) >> 1);
+                const bool odd = ((E + t - C) & 1) != 0;
+                const uint32_t x = h + (uint32_t)(t - C);
+                const bool inside = bc == 0 || (x >= lo && x < 2u * lo);
+                const uint32_t xc = lo | (x & (lo - 1u));
+                T v;
+                if (inside && bit_of(I, xc >> 1)) {
+                    v = cell(xc)[c];
+                } else {
+                    T sum = cf[0] * (w[pp + 1] - w[pp - 1]);
+#pragma unroll
+                    for (int a = 2; a <= G; ++a) sum = sum + cf[a - 1] * (w[pp + a] - w[pp - a]);
+                    v = odd ? w[pp] - sum : w[pp] + sum;
+                }
+                nw[t] = v;
+                if (x == lo) vlo = v;
+                if (x == 2u * lo - 1u) vhi = v;
+            }
+            if (bc != 0) {
+#pragma unroll
+                for (int t = 0; t < W; ++t) {
+                    const uint32_t x = h + (uint32_t)(t - C);
+                    if (x < lo) nw[t] = vlo;
+                    if (x >= 2u * lo) nw[t] = vhi;
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < W; ++t) w[t] = nw[t];
+        }
+        return w[C];
     }
 
     // S4 with the stencil of half-width gamma = 2 or 3: the first / last finest
     // values by the level-by-level reconstruction (edge_walk) instead of tables
     __device__ __noinline__ void reconstruct_wide() {
-        const uint32_t *R = mask(sm.cur);
+        const uint32_t *I = mask(sm.cur);
         const uint32_t *leaves = list(L_LEAF);
-        const int g = d.gamma;
-        const T *c = tab.pc[g];
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            const uint32_t ent = leaves[i];
-            const int l = ent >> KBITS;
-            const long long k = ent & KMASK;
-            const int dj = d.Jmax - l;
-            const bool at_left = d.bc == 1 && k == 0, at_right = d.bc == 1 && k == (1LL << l) - 1;
-            for (int h = 0; h < q; ++h) {
-                const T *rb = V + h;
-                const bool plus = (h & 1) == 0;  // velocity +lambda
-                const bool need_first = !plus || at_left, need_last = plus || at_right;
+        const int g = d.gamma, nl = sm.nleaf;
+        const T *cf = tab.pc[g];
+        const uint32_t N = 1u << Jmax;
+#pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            const uint32_t h = leaves[i], lo = level_first(h);
+            const int dj = Jmax - level_of(h);
+            const bool at_left = bc == 1 && h == lo, at_right = bc == 1 && h + 1u == 2u * lo;
+            const uint32_t first = (h << dj) & (N - 1u);
+            uint32_t next = first + (1u << dj);
+            if (bc == 0) next &= N - 1u;
+#pragma unroll 1
+            for (int c = 0; c < q; ++c) {
+                const bool plus = (c & 1) == 0;  // velocity +lambda
                 T rfirst = T(0), rlast = T(0);
-                if (dj == 0) {
-                    rfirst = rlast = row(h, l)[k];
-                } else {
-                    if (need_first)
-                        rfirst = g == 2 ? edge_walk<T, 2, false>(rb, q, d.Jmin, d.Jmax, d.bc, R, sm.woff, c, l, k)
-                                        : edge_walk<T, 3, false>(rb, q, d.Jmin, d.Jmax, d.bc, R, sm.woff, c, l, k);
-                    if (need_last)
-                        rlast = g == 2 ? edge_walk<T, 2, true>(rb, q, d.Jmin, d.Jmax, d.bc, R, sm.woff, c, l, k)
-                                       : edge_walk<T, 3, true>(rb, q, d.Jmin, d.Jmax, d.bc, R, sm.woff, c, l, k);
-                }
-                const auto ph = phi(h);
-                if (plus) {
-                    long long ix = (k + 1) << dj;
-                    if (d.bc == 0) ix &= d.N - 1;
-                    ph[ix] = rlast;
-                    if (at_left) ph[0] = rfirst;
-                } else {
-                    ph[k << dj] = rfirst;
-                    if (at_right) ph[d.N] = rlast;
-                }
+                if (!plus || at_left) rfirst = g == 2 ? edge_walk<2, false>(I, cf, c, h) : edge_walk<3, false>(I, cf, c, h);
+                if (plus || at_right) rlast = g == 2 ? edge_walk<2, true>(I, cf, c, h) : edge_walk<3, true>(I, cf, c, h);
+                if (plus || at_right) phi(next)[c] = rlast;
+                if (!plus || at_left) phi(first)[c] = rfirst;
             }
         }
     }
@@ -2065,34 +1567,27 @@ struct Worker {
     // the clamped out-of-domain cells copy.  Second cells from an edge use the
     // second-cell tables.
     __device__ __noinline__ void reconstruct_dq() {
-        const uint32_t *R = mask(sm.cur);
+        const uint32_t *I = mask(sm.cur);
         const uint32_t *leaves = list(L_LEAF);
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            const uint32_t ent = leaves[i];
-            const int l = ent >> KBITS;
-            const long long k = ent & KMASK;
-            const int dj = d.Jmax - l;
-            const long long first = k << dj, last = ((k + 1) << dj) - 1;
-            const bool at_left = d.bc == 1 && k == 0, at_right = d.bc == 1 && k == (1LL << l) - 1;
-            bool fin_l = false, fin_r = false;
-            long long cl = 0, cr = 0;
-            if (dj > 0) {
-                const uint32_t *rf = R + sm.woff[l + 1];
-                cl = 2 * wrapc(k - 1, l, d.bc);
-                cr = 2 * wrapc(k + 1, l, d.bc);
-                if (!at_left) fin_l = (rf[cl >> 5] >> (cl & 31)) & 1u;
-                if (!at_right) fin_r = (rf[cr >> 5] >> (cr & 31)) & 1u;
-            }
+        const int nl = sm.nleaf;
+#pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            const uint32_t hc = leaves[i], lo = level_first(hc);
+            const int dj = Jmax - level_of(hc);
+            const uint32_t first = (hc << dj) & ((1u << Jmax) - 1u), last = first + (1u << dj) - 1u;
+            const bool at_left = bc == 1 && hc == lo, at_right = bc == 1 && hc + 1u == 2u * lo;
+            const uint32_t hl = nb(hc, -1, lo), hr = nb(hc, 1, lo);
+            const bool fin_l = dj > 0 && !at_left && bit_of(I, hl), fin_r = dj > 0 && !at_right && bit_of(I, hr);
+            const T *v0p = cell(hc), *vm1p = cell(hl), *vp1p = cell(hr), *vm2p = cell(nb(hc, -2, lo)), *vp2p = cell(nb(hc, 2, lo));
+            const T *clp = cell(2u * hl), *crp = cell(2u * hr);
+#pragma unroll 1
             for (int h = 1; h < q; ++h) {
                 const int w = dq_w(h), a = w < 0 ? -w : w;
-                const auto r = row(h, l);
-                const auto ph = phi(h);
                 if (dj == 0) {
-                    ph[first] = r[k];
+                    phi(first)[h] = v0p[h];
                     continue;
                 }
-                const T vm1 = r[wrapc(k - 1, l, d.bc)], v0 = r[k], vp1 = r[wrapc(k + 1, l, d.bc)];
-                const auto rf = row(h, l + 1);
+                const T vm1 = vm1p[h], v0 = v0p[h], vp1 = vp1p[h];
                 // cell `sec` (0: first / last, 1: second from that edge) next to the left or right
                 // edge: one sum of four products for both stencils (as in reconstruct_edges), next
                 // to a finer neighbour with the leaf's own (predicted) children and the weights t1
@@ -2101,144 +1596,111 @@ struct Worker {
                             *cf = sec ? tab.cf2[dj] : tab.cf[dj];
                     if (at_left) return bf[0] * v0 + bf[1] * vp1;
                     T x0, x1, x2, x3;
-                    const T *wt;
                     if (fin_l) {
                         const T tt = T(C1) * (vp1 - vm1);
-                        x0 = rf[cl];
-                        x1 = rf[cl + 1];
+                        x0 = clp[h];
+                        x1 = clp[q + h];
                         x2 = v0 + tt;
                         x3 = v0 - tt;
-                        wt = t1;
                     } else {
-                        x0 = r[wrapc(k - 2, l, d.bc)];
+                        x0 = vm2p[h];
                         x1 = vm1;
                         x2 = v0;
                         x3 = vp1;
-                        wt = cf;
                     }
-                    return dot4(wt[0], x0, wt[1], x1, wt[2], x2, wt[3], x3);
+                    return dot4(fin_l ? t1 : cf, x0, x1, x2, x3);
                 };
                 auto from_right = [&](int sec) -> T {
                     const T *bf = sec ? tab.bf2[dj] : tab.bf[dj], *t1 = sec ? tab.t12[dj] : tab.t1[dj],
                             *cf = sec ? tab.cf2[dj] : tab.cf[dj];
                     if (at_right) return bf[0] * v0 + bf[1] * vm1;
                     T x0, x1, x2, x3;
-                    const T *wt;
                     if (fin_r) {
                         const T tt = T(C1) * (vp1 - vm1);
                         x0 = v0 + tt;
                         x1 = v0 - tt;
-                        x2 = rf[cr];
-                        x3 = rf[cr + 1];
-                        wt = t1;
+                        x2 = crp[h];
+                        x3 = crp[q + h];
                     } else {
                         x0 = vm1;
                         x1 = v0;
                         x2 = vp1;
-                        x3 = r[wrapc(k + 2, l, d.bc)];
-                        wt = cf;
+                        x3 = vp2p[h];
                     }
-                    return dot4(wt[3], x0, wt[2], x1, wt[1], x2, wt[0], x3);
+                    const T *wt = fin_r ? t1 : cf;
+                    const T wm[4] = {wt[3], wt[2], wt[1], wt[0]};
+                    return dot4(wm, x0, x1, x2, x3);
                 };
                 if (w > 0) {
-                    ph[last] = from_right(0);
-                    if (a == 2) ph[last - 1] = from_right(1);
-                    if (at_left) ph[first] = from_left(0);
+                    phi(last)[h] = from_right(0);
+                    if (a == 2) phi(last - 1u)[h] = from_right(1);
+                    if (at_left) phi(first)[h] = from_left(0);
                 } else {
-                    ph[first] = from_left(0);
-                    if (a == 2) ph[first + 1] = from_left(1);
-                    if (at_right) ph[last] = from_right(0);
+                    phi(first)[h] = from_left(0);
+                    if (a == 2) phi(first + 1u)[h] = from_left(1);
+                    if (at_right) phi(last)[h] = from_right(0);
                 }
             }
         }
     }
 
-    // S5 for the D1Q3 / D1Q5 schemes (eq. AdaptiveStreamPhase with |w| <= 2):
-    // f^{n+1} = f* + sigma 2^-dj sum_{delta=1}^{|w|} (V[first + eta] - V[next + eta]),
+    // the D1Q3 / D1Q5 stream of cell h (eq. AdaptiveStreamPhase with |w| <= 2):
+    // f + sigma 2^-dj sum_{delta=1}^{|w|} (V[first + eta] - V[next + eta]),
     // eta = -delta (sigma > 0) or delta - 1 (sigma < 0), V the finest values of
-    // reconstruct_dq (wrapped, or clamped at a copy boundary); audit of (h, hu)
+    // reconstruct_dq (wrapped, or clamped at a copy boundary)
+    __device__ __forceinline__ uint32_t finest_at(int i) const {
+        const int N = 1 << Jmax;
+        return (uint32_t)(bc == 0 ? (i & (N - 1)) : min(max(i, 0), N - 1));
+    }
+    __device__ __forceinline__ void stream_cell_dq(uint32_t hc, T *f) const {
+        const int dj = Jmax - level_of(hc);
+        const int first = (int)((hc << dj) & ((1u << Jmax) - 1u)), next = first + (1 << dj);
+        const T wgt = pow2m<T>(dj);
+        load_cell(hc, f);
+#pragma unroll
+        for (int h = 1; h < q; ++h) {
+            const int w = dq_w(h), a = w < 0 ? -w : w;
+            T acc = T(0);
+#pragma unroll
+            for (int dl = 1; dl <= a; ++dl) {
+                const int eta = w > 0 ? -dl : dl - 1;
+                acc = acc + (phi(finest_at(first + eta))[h] - phi(finest_at(next + eta))[h]);
+            }
+            f[h] = f[h] + (w > 0 ? wgt : -wgt) * acc;
+        }
+    }
+
+    // S5 for the D1Q3 / D1Q5 schemes, with the audit of (h, hu)
     __device__ __noinline__ void stream_dq() {
         const uint32_t *leaves = list(L_LEAF);
-        const long long N = d.N;
-        auto at = [&](long long i) -> long long { return d.bc == 0 ? (i & (N - 1)) : (i < 0 ? 0 : (i >= N ? N - 1 : i)); };
         double macc[3] = {0.0, 0.0, 0.0};
         float fhi[3] = {0.0f, 0.0f, 0.0f}, flo[3] = {0.0f, 0.0f, 0.0f};
         bool bad = false;
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            const uint32_t ent = leaves[i];
-            const int l = ent >> KBITS;
-            const long long k = ent & KMASK;
-            const int dj = d.Jmax - l;
-            const long long first = k << dj, next = (k + 1) << dj;
-            const T wgt = pow2m<T>(dj);
-            T fn[QMAX];
+        const int nl = sm.nleaf;
+#pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            const uint32_t hc = leaves[i];
+            T fn[q];
+            stream_cell_dq(hc, fn);
+            store_cell(hc, fn);
 #pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) {
-                    const int w = dq_w(h);
-                    const auto r = row(h, l);
-                    T v = r[k];
-                    if (w != 0) {
-                        const auto ph = phi(h);
-                        const int a = w < 0 ? -w : w;
-                        T acc = T(0);
-                        for (int dl = 1; dl <= a; ++dl) {
-                            const long long eta = w > 0 ? -dl : dl - 1;
-                            acc = acc + (ph[at(first + eta)] - ph[at(next + eta)]);
-                        }
-                        v = v + (w > 0 ? wgt : -wgt) * acc;
-                    }
-                    bad |= nonfinite(v);
-                    r[k] = v;
-                    fn[h] = v;
-                }
-            if constexpr (sizeof(T) == 8) {
-                double m0 = 0.0, m1 = 0.0;
-#pragma unroll
-                for (int h = 0; h < QMAX; ++h)
-                    if (h < q) {
-                        m0 += (double)fn[h];
-                        m1 += (dq_w(h) * d.lam) * (double)fn[h];
-                    }
-                macc[0] += sm.dx_l[l] * m0;
-                macc[1] += sm.dx_l[l] * m1;
-            } else {
-                // exact per-leaf sums of f and of w f in float-float, scaled by 2^-l
-                const float sc = pow2m<float>(l);
-                float a0 = 0.0f, e0 = 0.0f, a1 = 0.0f, e1 = 0.0f;
-#pragma unroll
-                for (int h = 0; h < QMAX; ++h)
-                    if (h < q) {
-                        ff_add(a0, e0, (float)fn[h], 0.0f);
-                        ff_add(a1, e1, (float)(dq_w(h)) * (float)fn[h], 0.0f);
-                    }
-                ff_add(fhi[0], flo[0], a0 * sc, e0 * sc);
-                ff_add(fhi[1], flo[1], a1 * sc, e1 * sc);
-            }
+            for (int h = 0; h < q; ++h) bad |= nonfinite(fn[h]);
+            audit_cell(hc, fn, macc, fhi, flo);
         }
         if (bad) atomicOr(&sm.status, (int)ST_NONFINITE);
-        if constexpr (sizeof(T) == 8) {
-            team_sum(macc);
-        } else {
-            team_sum_ff(fhi, flo, macc);
-            if (tid == 0) {
-                macc[0] *= d.b - d.a;
-                macc[1] *= (d.b - d.a) * d.lam;
-            }
-        }
+        sum_audit(macc, fhi, flo);
         if (tid == 0) {
             // copy boundary: what leaves through x = a and x = b, sum over the
             // populations of sigma 2^-Jmax-weighted telescoped stream terms
             double flux[2] = {0.0, 0.0};
-            if (d.bc == 1) {
-                const double dxJ = sm.dx_l[d.Jmax];
+            if (bc == 1) {
+                const double dxJ = sm.dx_l[Jmax];
                 for (int h = 1; h < q; ++h) {
                     const int w = dq_w(h), a = w < 0 ? -w : w;
-                    const auto ph = phi(h);
                     double t = 0.0;
                     for (int dl = 1; dl <= a; ++dl) {
-                        const long long eta = w > 0 ? -dl : dl - 1;
-                        t += (double)ph[at(eta)] - (double)ph[at(N + eta)];
+                        const int eta = w > 0 ? -dl : dl - 1;
+                        t += (double)phi(finest_at(eta))[h] - (double)phi(finest_at((1 << Jmax) + eta))[h];
                     }
                     t *= (w > 0 ? dxJ : -dxJ);
                     flux[0] += t;
@@ -2255,91 +1717,91 @@ struct Worker {
         sync();
     }
 
-    // sum of four products; FP32: compensated (Kahan) accumulation
-    static __device__ __forceinline__ T dot4(T c0, T x0, T c1, T x1, T c2, T x2, T c3, T x3) {
+    // the audit's partial sums of one leaf: dx_l m_j in FP64, or, in the FP32
+    // path, 2^-l m_j summed exactly per leaf into float-float partials
+    // (relative error near 2^-44) and scaled by b - a at the end
+    __device__ __forceinline__ void audit_cell(uint32_t h, const T *f, double (&macc)[3], float (&fhi)[3], float (&flo)[3]) const {
+        const int l = level_of(h);
         if constexpr (sizeof(T) == 8) {
-            return fma(c3, x3, fma(c2, x2, fma(c1, x1, c0 * x0)));
-        } else {
-            T p[4] = {c0 * x0, c1 * x1, c2 * x2, c3 * x3};
-            T s = T(0), comp = T(0);
+            const double dx = sm.dx_l[l];
+            if constexpr (DQ) {
+                double m0 = 0.0, m1 = 0.0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                T y = p[j] - comp;
-                T t = s + y;
-                comp = (t - s) - y;
-                s = t;
+                for (int c = 0; c < q; ++c) {
+                    m0 += (double)f[c];
+                    m1 += (dq_w(c) * d.lam) * (double)f[c];
+                }
+                macc[0] += dx * m0;
+                macc[1] += dx * m1;
+            } else {
+#pragma unroll
+                for (int j = 0; j < nf; ++j) macc[j] += dx * ((double)f[2 * j] + (double)f[2 * j + 1]);
             }
-            return s;
+        } else {
+            const float sc = pow2m<float>(l);
+            if constexpr (DQ) {
+                float a0 = 0.0f, e0 = 0.0f, a1 = 0.0f, e1 = 0.0f;
+#pragma unroll
+                for (int c = 0; c < q; ++c) {
+                    ff_add(a0, e0, (float)f[c], 0.0f);
+                    ff_add(a1, e1, (float)(dq_w(c)) * (float)f[c], 0.0f);
+                }
+                ff_add(fhi[0], flo[0], a0 * sc, e0 * sc);
+                ff_add(fhi[1], flo[1], a1 * sc, e1 * sc);
+            } else {
+#pragma unroll
+                for (int j = 0; j < nf; ++j) {
+                    float sj, ej;
+                    two_sum((float)f[2 * j], (float)f[2 * j + 1], sj, ej);
+                    ff_add(fhi[j], flo[j], sj * sc, ej * sc);
+                }
+            }
         }
     }
-
-    // S5: f^{n+1} = f* + sigma 2^-dj (Phi[first] - Phi[next]); mass audit.
-    // The totals sum dx_l (f+ + f-) over the leaves: FP64 in the FP64 path; in
-    // the FP32 path 2^-l (f+ + f-) is summed exactly per leaf into float-float
-    // partials (relative error near 2^-44) and scaled by b - a at the end.
-    __device__ void stream_and_audit() {
-        if constexpr (DQ) {
-            stream_dq();
-            return;
-        }
-        const uint32_t *leaves = list(L_LEAF);
-        double macc[3] = {0.0, 0.0, 0.0};
-        float fhi[3] = {0.0f, 0.0f, 0.0f}, flo[3] = {0.0f, 0.0f, 0.0f};
-        bool bad = false;
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            uint32_t ent = leaves[i];
-            int l = ent >> KBITS;
-            long long k = ent & KMASK;
-            int dj = d.Jmax - l;
-            long long first = k << dj, next = (k + 1) << dj;
-            if (d.bc == 0) next &= d.N - 1;
-            const T w = pow2m<T>(dj);
-            T fn[QMAX];
-#pragma unroll
-            for (int h = 0; h < QMAX; ++h)
-                if (h < q) {
-                    const auto ph = phi(h);
-                    T coef = (h & 1) ? -w : w;
-                    const auto r = row(h, l);
-                    T v = r[k] + coef * (ph[first] - ph[next]);
-                    bad |= nonfinite(v);
-                    r[k] = v;
-                    fn[h] = v;
-                }
-            if constexpr (sizeof(T) == 8) {
-                const double dx = sm.dx_l[l];
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (j < nf) macc[j] += dx * ((double)fn[2 * j] + (double)fn[2 * j + 1]);
-            } else {
-                const float sc = pow2m<float>(l);
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    if (j < nf) {
-                        float sj, ej;
-                        two_sum((float)fn[2 * j], (float)fn[2 * j + 1], sj, ej);
-                        ff_add(fhi[j], flo[j], sj * sc, ej * sc);
-                    }
-            }
-        }
-        if (bad) atomicOr(&sm.status, (int)ST_NONFINITE);
-        project_by_flux_pass();  // A1 of the next adaptation, same pass
+    // the audit's totals, in thread 0 (one barrier)
+    __device__ __forceinline__ void sum_audit(double (&macc)[3], float (&fhi)[3], float (&flo)[3]) {
         if constexpr (sizeof(T) == 8) {
             team_sum(macc);
         } else {
             team_sum_ff(fhi, flo, macc);
-            if (tid == 0)
+            if (tid == 0) {
+#pragma unroll
                 for (int j = 0; j < nf; ++j) macc[j] *= d.b - d.a;
+                if constexpr (DQ) macc[1] *= d.lam;
+            }
         }
+    }
+
+    // S5: f^{n+1} = f* + sigma 2^-dj (Phi[first] - Phi[next]); mass audit
+    // (totals sum dx_l (f+ + f-) over the leaves)
+    __device__ void stream_and_audit() {
+        const uint32_t *leaves = list(L_LEAF);
+        double macc[3] = {0.0, 0.0, 0.0};
+        float fhi[3] = {0.0f, 0.0f, 0.0f}, flo[3] = {0.0f, 0.0f, 0.0f};
+        bool bad = false;
+        const int nl = sm.nleaf;
+#pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            const uint32_t h = leaves[i];
+            T fn[q];
+            stream_cell(h, fn);
+            store_cell(h, fn);
+#pragma unroll
+            for (int j = 0; j < q; ++j) bad |= nonfinite(fn[j]);
+            audit_cell(h, fn, macc, fhi, flo);
+        }
+        if (bad) atomicOr(&sm.status, (int)ST_NONFINITE);
+        project_by_flux_pass();  // A1 of the next adaptation, same pass
+        sum_audit(macc, fhi, flo);
         if (tid == 0) {
-            double dxJ = sm.dx_l[d.Jmax];
+            const double dxJ = sm.dx_l[Jmax];
             for (int j = 0; j < nf; ++j) {
                 double flux = 0.0;
-                if (d.bc == 1) {
-                    const auto pp = phi(2 * j), pm = phi(2 * j + 1);
-                    flux = dxJ * (((double)pp[0] - (double)pp[d.N]) - ((double)pm[0] - (double)pm[d.N]));
+                if (bc == 1) {
+                    const T *p0 = phi(0u), *pN = phi(1u << Jmax);
+                    flux = dxJ * (((double)p0[2 * j] - (double)pN[2 * j]) - ((double)p0[2 * j + 1] - (double)pN[2 * j + 1]));
                 }
-                double res = fabs(macc[j] - sm.mass[j] - flux);
+                const double res = fabs(macc[j] - sm.mass[j] - flux);
                 sm.audit = fmax(sm.audit, res);
                 sm.mass[j] = macc[j];
             }
@@ -2352,90 +1814,96 @@ struct Worker {
     // ---- initial state -------------------------------------------------------
     // full tree, populations at equilibrium of the conserved moments (staged m_cons)
     __device__ __noinline__ void init_full(const double *mcons) {
-        uint32_t *R = mask(M_R0);
-        for (int g = tid; g < d.Wtot; g += TS) {
-            int l, wi;
-            level_of_word(sm, g, l, wi);
-            R[g] = valid_bits(l);
-            mask(M_R1)[g] = 0u;
-            mask(M_KEEP)[g] = 0u;
-            mask(M_REF)[g] = 0u;
-        }
-        for (long long k = tid; k < d.N; k += TS) {
-            double mc[3], f[QMAX];
-            for (int j = 0; j < nf; ++j) mc[j] = mcons[j * d.N + k];
+        clear_masks();
+        uint32_t *I = mask(M_I0);
+#pragma unroll 1
+        for (int w = tid; w < d.Wtot; w += TS) I[w] = w == 0 ? (Jmax >= 5 ? 0xFFFFFFFEu : (1u << (1 << Jmax)) - 2u) : FULL;
+        const int N = 1 << Jmax;
+#pragma unroll 1
+        for (int k = tid; k < N; k += TS) {
+            double mc[3], f[q];
+            T ft[q];
+            for (int j = 0; j < nf; ++j) mc[j] = mcons[(long long)j * N + k];
             if constexpr (DQ)
                 dq_equilibrium_populations<q>(d, mc, f);
             else
                 equilibrium_populations<NF>(d, mc, f);
-            for (int h = 0; h < q; ++h) row(h, d.Jmax)[k] = (T)f[h];
+#pragma unroll
+            for (int h = 0; h < q; ++h) ft[h] = (T)f[h];
+            store_cell((uint32_t)(N + k), ft);
         }
-        if (tid == 0) sm.cur = M_R0;
-        sync();
         finish_init();
+    }
+
+    // the bit arrays but the current tree's (M_I0)
+    __device__ __forceinline__ void clear_masks() {
+#pragma unroll 1
+        for (int w = tid; w < d.Wtot; w += TS) {
+            mask(M_I1)[w] = 0u;
+            mask(M_KEEP)[w] = 0u;
+            mask(M_REF)[w] = 0u;
+        }
     }
 
     // arbitrary graded tree (one byte per cell) and values
     __device__ __noinline__ void init_state(const unsigned char *Rb, const double *vals) {
-        uint32_t *R = mask(M_R0);
-        for (int g = tid; g < d.Wtot; g += TS) {
-            int l, wi;
-            level_of_word(sm, g, l, wi);
-            long long base = cell_off(l, d.Jmin) + 32LL * wi;
-            int nb = l >= 5 ? 32 : (1 << l);
-            uint32_t w = 0;
-            for (int b = 0; b < nb; ++b) w |= (Rb[base + b] ? 1u : 0u) << b;
-            R[g] = w;
-            mask(M_R1)[g] = 0u;
-            mask(M_KEEP)[g] = 0u;
-            mask(M_REF)[g] = 0u;
+        clear_masks();
+        uint32_t *I = mask(M_I0);
+        const uint32_t off = 1u << Jmin;
+#pragma unroll 1
+        for (int w = tid; w < d.Wtot; w += TS) {
+            uint32_t x = above(w);
+            for (uint32_t b = 0; b < 32u; ++b) {
+                const uint32_t h = 32u * w + b;  // internal: its first child is in the tree
+                if (h >= off && h < (1u << Jmax) && Rb[2u * h - off]) x |= 1u << b;
+            }
+            I[w] = x;
         }
         // population-major input to the cell-major layout
+#pragma unroll 1
         for (long long c = tid; c < (long long)q * d.S; c += TS) {
-            const long long hh = c / d.S, cell = c - hh * d.S;
-            V[cell * q + hh] = (T)vals[c];
+            const long long hh = c / d.S, k = c - hh * d.S;
+            cell((uint32_t)(k + off))[hh] = (T)vals[c];
         }
-        if (tid == 0) sm.cur = M_R0;
-        sync();
         finish_init();
     }
 
     __device__ __noinline__ void finish_init() {
-        uint32_t *R = mask(sm.cur);
-        {
-            // every mask word is a candidate of this first marking
-            if (sparse_on()) {
-                uint32_t *cw = cwl();
-                for (int g = tid; g < d.Wtot; g += TS) cw[g] = (uint32_t)g;
-                for (int g = tid; g < d.OW; g += TS) {
-                    occ(M_R0)[g] = 0u;
-                    occ(M_R1)[g] = 0u;
-                }
+        if (tid == 0) sm.cur = M_I0;
+        if constexpr (SPM != 0) {
+            // every word is a candidate of this first listing
+            uint32_t *cw = cwl();
+#pragma unroll 1
+            for (int w = tid; w < d.Wtot; w += TS) cw[w] = (uint32_t)w;
+#pragma unroll 1
+            for (int j = tid; j < d.OW; j += TS) {
+                occ(M_I0)[j] = 0u;
+                occ(M_I1)[j] = 0u;
             }
-            for (int l = d.Jmin + tid; l <= d.Jmax + 1; l += TS) sm.cw_seg[l] = sm.woff[l];
+            if (tid == 0) sm.ncw = d.Wtot;
         }
         sync();
-        grade_and_mark(R, R, false);  // PRED empty: the tree is its own old tree
-        build_lists(R, occ(sm.cur));
+        uint32_t *I = mask(M_I0);
+        build_lists(I, I, SPM != 0 ? occ(M_I0) : nullptr);  // the tree is its own old tree
         // FP64 totals of the initial leaves
         const uint32_t *leaves = list(L_LEAF);
         double macc[3] = {0.0, 0.0, 0.0};
-        for (int i = tid; i < sm.nleaf; i += TS) {
-            uint32_t ent = leaves[i];
-            int l = ent >> KBITS;
-            long long k = ent & KMASK;
-            double dx = sm.dx_l[l];
+        const int nl = sm.nleaf;
+#pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            const uint32_t h = leaves[i];
+            const T *f = cell(h);
+            const double dx = sm.dx_l[level_of(h)];
             if constexpr (DQ) {
                 double m0 = 0.0, m1 = 0.0;
-                for (int h = 0; h < q; ++h) {
-                    const double f = (double)row(h, l)[k];
-                    m0 += f;
-                    m1 += (dq_w(h) * d.lam) * f;
+                for (int c = 0; c < q; ++c) {
+                    m0 += (double)f[c];
+                    m1 += (dq_w(c) * d.lam) * (double)f[c];
                 }
                 macc[0] += dx * m0;
                 macc[1] += dx * m1;
             } else {
-                for (int j = 0; j < nf; ++j) macc[j] += dx * ((double)row(2 * j, l)[k] + (double)row(2 * j + 1, l)[k]);
+                for (int j = 0; j < nf; ++j) macc[j] += dx * ((double)f[2 * j] + (double)f[2 * j + 1]);
             }
         }
         team_sum(macc);
@@ -2453,32 +1921,22 @@ struct Worker {
 
     // ---- multiresolution reconstruction on the finest level (measurement) ----
     __device__ __noinline__ void finest(double *out) {
-        upsweep();
+        fill_finest();
         if (tid == 0) sm.status &= ~(int)ST_FLUXED;  // internal cells now project f, not f*
-        sync();
-        const uint32_t *R = mask(sm.cur);
-        for (int l = d.Jmin + 1; l <= d.Jmax; ++l) {
-            long long n = 1LL << l;
-            const uint32_t *rl = R + sm.woff[l];
-            for (long long k = tid; k < n; k += TS)
-                if (!((rl[k >> 5] >> (k & 31)) & 1u))
-                    for (int h = 0; h < q; ++h)
-                        row(h, l)[k] = predict_g<T>(row(h, l - 1), k >> 1, (int)(k & 1), l - 1, d.bc, d.gamma,
-                                                    tab.pc[d.gamma]);
-            sync();
-        }
-        for (long long k = tid; k < d.N; k += TS) {
+        const int N = 1 << Jmax;
+#pragma unroll 1
+        for (int k = tid; k < N; k += TS) {
+            const T *f = cell((uint32_t)(N + k));
             if constexpr (DQ) {
                 double m0 = 0.0, m1 = 0.0;
                 for (int h = 0; h < q; ++h) {
-                    const double f = (double)row(h, d.Jmax)[k];
-                    m0 += f;
-                    m1 += (dq_w(h) * d.lam) * f;
+                    m0 += (double)f[h];
+                    m1 += (dq_w(h) * d.lam) * (double)f[h];
                 }
                 out[k] = m0;
-                out[d.N + k] = m1;
+                out[(long long)N + k] = m1;
             } else {
-                for (int j = 0; j < nf; ++j) out[j * d.N + k] = (double)row(2 * j, d.Jmax)[k] + (double)row(2 * j + 1, d.Jmax)[k];
+                for (int j = 0; j < nf; ++j) out[(long long)j * N + k] = (double)f[2 * j] + (double)f[2 * j + 1];
             }
         }
         sync();
@@ -2488,11 +1946,12 @@ struct Worker {
 // ---------------------------------------------------------------------------
 // instance state in and out of shared memory (TS threads of the team)
 
-template <typename T, int TS, int SPM>
+template <typename T, int TS>
 __device__ void load_instance(TeamSmem<T> &sm, const InstDesc &dg, int tid) {
+    // the descriptor and the list segments, word by word
+    for (int i = tid; i < (int)(sizeof(InstDesc) / 4); i += TS) ((uint32_t *)&sm.d)[i] = ((const uint32_t *)&dg)[i];
+    const InstState &st = *dg.st;
     if (tid == 0) {
-        sm.d = dg;
-        const InstState &st = *dg.st;
         sm.cur = st.cur;
         sm.nleaf = st.nleaf;
         sm.status = st.status;
@@ -2508,22 +1967,6 @@ __device__ void load_instance(TeamSmem<T> &sm, const InstDesc &dg, int tid) {
         for (int p = 0; p < NPHASE; ++p) sm.ptime[p] = st.ptime[p];
         sm.tlast = clock64();
 #endif
-        int Jmin = dg.Jmin, Jmax = dg.Jmax;
-        int o = 0, oo = 0;
-        for (int l = Jmin; l <= Jmax; ++l) {
-            sm.woff[l] = o;
-            sm.ooff[l] = oo;
-            o += l >= 5 ? (1 << (l - 5)) : 1;
-            oo += l >= 10 ? (1 << (l - 10)) : 1;
-        }
-        sm.woff[Jmax + 1] = o;
-        sm.ooff[Jmax + 1] = oo;
-        sm.sparse = SPM != 0 ? 1 : 0;
-        // without candidate words every word of level l is visited
-        if (!sm.sparse)
-            for (int l = Jmin; l <= Jmax + 1; ++l) sm.cw_seg[l] = sm.woff[l];
-        sm.g0s = Jmin < 5 ? 5 - Jmin : 0;
-        sm.gbase = Jmin < 5 ? 1 : (1 << (Jmin - 5));
     }
     for (int l = tid; l <= MAXLEV; l += TS) {
         // eps_l = 2^{l - Jmax} eps (Prop. ErrorControl), Harten level 2^{mu_bar + 1} eps_l
@@ -2535,20 +1978,14 @@ __device__ void load_instance(TeamSmem<T> &sm, const InstDesc &dg, int tid) {
         sm.big_f[l] = (float)bl;
         sm.dx_l[l] = ldexp(dg.b - dg.a, -l);
     }
-    for (int i = tid; i < NLIST * (MAXLEV + 2); i += TS) (&sm.seg[0][0])[i] = (&dg.st->seg[0][0])[i];
-    if constexpr (TS == 32)
-        __syncwarp();
-    else
-        __syncthreads();
+    for (int i = tid; i < NSEG * (MAXLEV + 2); i += TS) (&sm.seg[0][0])[i] = (&st.seg[0][0])[i];
+    __syncthreads();
 }
 
 template <typename T, int TS>
 __device__ void store_instance(TeamSmem<T> &sm, int tid) {
     // the barrier count of the last pass is written after that pass's barrier
-    if constexpr (TS == 32)
-        __syncwarp();
-    else
-        __syncthreads();
+    __syncthreads();
     InstState &st = *sm.d.st;
     if (tid == 0) {
         st.cur = sm.cur;
@@ -2566,11 +2003,8 @@ __device__ void store_instance(TeamSmem<T> &sm, int tid) {
         for (int p = 0; p < NPHASE; ++p) st.ptime[p] = sm.ptime[p];
 #endif
     }
-    for (int i = tid; i < NLIST * (MAXLEV + 2); i += TS) (&st.seg[0][0])[i] = (&sm.seg[0][0])[i];
-    if constexpr (TS == 32)
-        __syncwarp();
-    else
-        __syncthreads();
+    for (int i = tid; i < NSEG * (MAXLEV + 2); i += TS) (&st.seg[0][0])[i] = (&sm.seg[0][0])[i];
+    __syncthreads();
 }
 
 // one instance for the launch's steps
@@ -2580,6 +2014,7 @@ __device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &t
     Worker<T, NF, TS, WIDE, SPM> w(sm, tab, bx, tid, masks);
     if (a.phases & PH_INIT_FULL) w.init_full((const double *)a.aux0 + sm.d.m_off);
     if (a.phases & PH_INIT_STATE) w.init_state((const unsigned char *)a.aux0, (const double *)a.aux1);
+#pragma unroll 1
     for (int n = 0; n < a.nsteps; ++n) {
         if (a.phases & PH_ADAPT) w.adapt();
         if (a.phases & PH_STEP) w.lbm_step();
@@ -2587,15 +2022,14 @@ __device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &t
     if (a.phases & PH_FINEST) w.finest((double *)a.aux0);
 }
 
-// Bitmasks live in shared memory (smask, room for `cap` words per mask) when the
-// instance fits: the current tree and the transfer / ghost marks (which a later
-// step's predictions read; KEEP / REF share their storage and A2 clears it) are
-// copied in at the start and back at the end; the other masks are rebuilt by
-// every step.
+// The bit arrays live in shared memory (smask, room for `cap` words) when the
+// instance fits: the current tree is copied in at the start and back at the
+// end; KEEP and REF are clear between two adaptations, and every adaptation
+// writes the other tree buffer.
 template <typename T, int TS, bool WIDE, bool SCALAR, int SPM>
 __device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx, const LaunchArgs &a,
                          const InstDesc &dg, int tid, uint32_t *smask, int cap) {
-    load_instance<T, TS, SPM>(sm, dg, tid);
+    load_instance<T, TS>(sm, dg, tid);
     const int W = sm.d.Wtot, OW = sm.d.OW;
     const long long region = smem_region_words(W, OW);
     const bool local = smask != nullptr && region <= cap;
@@ -2607,13 +2041,12 @@ __device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx
         for (int g = tid; g < W; g += TS) other[g] = 0u;
     }
     if (local) {
-        const uint32_t *gr = sm.d.masks + (long long)sm.cur * W;
-        uint32_t *lr = smask + sm.cur * W;
-        const uint32_t *gp = sm.d.masks + (long long)M_PRED * W, *gg = sm.d.masks + (long long)M_GH * W;
+        const uint32_t *gi = sm.d.masks + (long long)sm.cur * W;
+        uint32_t *li = smask + sm.cur * W;
         for (int g = tid; g < W; g += TS) {
-            lr[g] = gr[g];
-            smask[M_PRED * W + g] = gp[g];
-            smask[M_GH * W + g] = gg[g];
+            li[g] = gi[g];
+            smask[M_KEEP * W + g] = 0u;
+            smask[M_REF * W + g] = 0u;
         }
         if constexpr (SPM != 0)
             for (int g = tid; g < OW; g += TS) smask[oo + g] = sm.d.masks[oo + g];
@@ -2633,14 +2066,14 @@ __device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx
         }
     }
     if (local) {
-        uint32_t *gr = sm.d.masks + (long long)sm.cur * W;
-        uint32_t *gp = sm.d.masks + (long long)M_PRED * W, *gg = sm.d.masks + (long long)M_GH * W;
-        const uint32_t *lr = smask + sm.cur * W;
-        for (int g = tid; g < W; g += TS) {
-            gr[g] = lr[g];
-            gp[g] = smask[M_PRED * W + g];
-            gg[g] = smask[M_GH * W + g];
-        }
+        uint32_t *gi = sm.d.masks + (long long)sm.cur * W;
+        const uint32_t *li = smask + sm.cur * W;
+        for (int g = tid; g < W; g += TS) gi[g] = li[g];
+        if (a.phases & (PH_INIT_FULL | PH_INIT_STATE))  // clear there too, for a launch that keeps them there
+            for (int g = tid; g < W; g += TS) {
+                sm.d.masks[(long long)M_KEEP * W + g] = 0u;
+                sm.d.masks[(long long)M_REF * W + g] = 0u;
+            }
         const long long oc = (long long)(NMASK + 1) * W + (long long)sm.cur * OW;
         if constexpr (SPM != 0)
             for (int g = tid; g < OW; g += TS) sm.d.masks[oc + g] = smask[oc + g];

@@ -105,11 +105,7 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     // layout of the scratch area for this instance (same regions as a bound context)
     const int q = mrg_npop(d.eq);
     const long long S = (1LL << (d.Jmax + 1)) - (1LL << d.Jmin), N = 1LL << d.Jmax;
-    int W = 0, OW = 0;
-    for (int l = d.Jmin; l <= d.Jmax; ++l) {
-        W += l >= 5 ? (1 << (l - 5)) : 1;
-        OW += occ_words_of(l);
-    }
+    const int W = mask_words_of(d.Jmax), OW = occ_words_of(d.Jmax);
     const long long region = mask_region_words(W, OW);
     const size_t vb = fp32 ? 4 : 8;
     size_t o = 0;
@@ -131,7 +127,7 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     long long lo = 0, list_off[NLIST];
     for (int L = 0; L < NLIST; ++L) {
         list_off[L] = lo;
-        lo += (S + 63) / 64 * 64;
+        lo += (N + 63) / 64 * 64;
     }
     o = align256(o + sizeof(uint32_t) * lo);
     if (o > (size_t)MR_STATIC_SCRATCH_BYTES)

@@ -37,11 +37,7 @@ enum { L_INT = 0, L_PRED = 1, L_GH = 2, L_LEAF = 3, NLIST = 4, NSEG = 3 };
 // phases of the persistent kernel
 enum { PH_INIT_FULL = 1, PH_INIT_STATE = 2, PH_ADAPT = 4, PH_STEP = 8, PH_FINEST = 16 };
 // device status bits
-// ST_FLUXED: the last step streamed with interface values in Phi (D1Q2^n
-// schemes) and, in the same pass, moved every internal cell by the flux through
-// its own edges, so the internal cells hold the projection of the leaves and the
-// next adaptation skips its projection (see the kernel).
-enum { ST_NONFINITE = 1, ST_FLUXED = 2 };
+enum { ST_NONFINITE = 1 };
 // phases timed by the profiling build (MRG_PHASE_TIMERS)
 enum {
     T_UPSWEEP_A = 0, T_DETAILS, T_ENLARGE, T_GRADE, T_GRADE_SMALL, T_CANDIDATES, T_LISTS, T_TRANSFER,

@@ -6,8 +6,8 @@
 // atomic work queue sorted largest first (persistent launch).  Inside a step:
 //
 //   adapt (Section 4.1)
-//     A1  projection up the current tree (Def. Projection operator); right
-//         after a D1Q2^n step, one conservative update of the internal cells
+//     A1  projection up the current tree (Def. Projection operator): one
+//         conservative update of the internal cells, in the last step's S5
 //     A2  details of the pairs of the tree, threshold T, Harten flags (Sections
 //         3.2, 3.4, 4.2) -> KEEP / REF bitmasks
 //     A3  enlargement H: same-level dilation and children of REF pairs
@@ -841,18 +841,20 @@ struct Worker {
         }
     }
 
-    // A1 right after a step of a D1Q2^n scheme, by conservation.  The stream
-    // (S5) moved every leaf by w (Phi[first] - Phi[next]) with w = +-2^-dj, one
-    // value of Phi per interface shared by the two cells it separates, so the
-    // size-weighted mean of the leaves under an internal cell moved by the same
-    // expression at the cell's own two edges (the inner interfaces cancel), and
-    // the internal cells still hold the projection of f* (S2; ghosts lie outside
-    // the tree).  One update of every internal cell, all levels in one pass,
-    // therefore equals the level-by-level projection of the streamed leaves up
-    // to rounding, and replaces its Jmax - Jmin dependent passes.
-    // The update runs in the stream's own pass (S5): it reads only Phi, which S4
-    // completed, and the internal cells, which S5 does not touch; the next
-    // adaptation then starts from projected internal cells (status ST_FLUXED).
+    // A1 by conservation.  The stream (S5) moves every leaf by sigma 2^-dj times
+    // the difference of what crosses its two edges, one value per interface
+    // shared by the two cells it separates (for |w| = 2 the sum of the two cells
+    // upwind of it), so the size-weighted mean of the leaves under an internal
+    // cell moves by the same expression at the cell's own two edges (the inner
+    // interfaces cancel), and the internal cells hold the projection of f* (S2;
+    // ghosts lie outside the tree).  One update of every internal cell, all
+    // levels in one pass, therefore equals the level-by-level projection of the
+    // streamed leaves up to rounding, and replaces its Jmax - Jmin dependent
+    // passes.  It runs in the stream's own pass: it reads only Phi, which S4
+    // completed, and the internal cells, which the leaves' stream does not touch.
+    // With it the internal cells hold the projection of the leaves between any
+    // two calls: the initial state projects them, the stream moves them, and a
+    // cell that becomes internal is the projection of the pair predicted from it.
     __device__ __forceinline__ void project_by_flux_pass() {
         const uint32_t *li = list(L_INT);
         const int e = sm.seg[L_INT][top()];
@@ -860,7 +862,10 @@ struct Worker {
         for (int i = tid; i < e; i += TS) {
             const uint32_t h = li[i];
             T f[q];
-            stream_cell(h, f);
+            if constexpr (DQ)
+                stream_cell_dq(h, f);
+            else
+                stream_cell(h, f);
             store_cell(h, f);
         }
     }
@@ -1325,9 +1330,6 @@ struct Worker {
             for (int j = tid; j < d.OW; j += TS) on[j] = 0u;
         }
         tick(T_CANDIDATES);
-        // internal cells: already projected by the last stream (D1Q2^n), else level by level
-        if (DQ || !(sm.status & ST_FLUXED)) upsweep();
-        tick(T_UPSWEEP_A);
         details();
         sync();
         tick(T_DETAILS);
@@ -1352,7 +1354,6 @@ struct Worker {
         if (tid == 0) {
             sm.cur ^= 1;
             sm.updates += (unsigned long long)sm.nleaf;
-            sm.status &= ~(int)ST_FLUXED;  // new tree: its internal cells are projections of f
         }
         sync();
     }
@@ -1688,6 +1689,7 @@ struct Worker {
             audit_cell(hc, fn, macc, fhi, flo);
         }
         if (bad) atomicOr(&sm.status, (int)ST_NONFINITE);
+        project_by_flux_pass();  // A1 of the next adaptation, same pass
         sum_audit(macc, fhi, flo);
         if (tid == 0) {
             // copy boundary: what leaves through x = a and x = b, sum over the
@@ -1806,7 +1808,6 @@ struct Worker {
                 sm.mass[j] = macc[j];
             }
             sm.steps += 1ULL;
-            sm.status |= ST_FLUXED;  // before the barrier: every thread of the next adaptation sees it
         }
         sync();
     }
@@ -1885,6 +1886,7 @@ struct Worker {
         sync();
         uint32_t *I = mask(M_I0);
         build_lists(I, I, SPM != 0 ? occ(M_I0) : nullptr);  // the tree is its own old tree
+        upsweep();
         // FP64 totals of the initial leaves
         const uint32_t *leaves = list(L_LEAF);
         double macc[3] = {0.0, 0.0, 0.0};
@@ -1922,7 +1924,6 @@ struct Worker {
     // ---- multiresolution reconstruction on the finest level (measurement) ----
     __device__ __noinline__ void finest(double *out) {
         fill_finest();
-        if (tid == 0) sm.status &= ~(int)ST_FLUXED;  // internal cells now project f, not f*
         const int N = 1 << Jmax;
 #pragma unroll 1
         for (int k = tid; k < N; k += TS) {

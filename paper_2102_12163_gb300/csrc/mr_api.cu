@@ -842,7 +842,12 @@ mr_status mr_get_finest(mr_ctx *c, int inst, double *out) {
     const InstDesc &h = c->hdesc[inst];
     bool dev = is_device_ptr(out);
     void *dst = dev ? (void *)out : (void *)(c->ws + c->off_stage);
-    int rc = launch(c, PH_FINEST, 0, inst, dst, nullptr);
+    if (!c->bound) return (mr_status)c->fail(MR_ERR_STATE, "context not bound to a workspace");
+    int rc = c->cuda((cudaError_t)mrg_finest(c->fp32(), variant_of(h.eq), h.Jmax, (const InstDesc *)(c->ws + c->off_desc) + inst,
+                                             c->ws + c->off_tab + (c->fp32() ? sizeof(Tables<double>) : 0), (double *)dst,
+                                             c->stream),
+                     "kernel launch");
+    ++c->launches;
     if (rc) return (mr_status)rc;
     if (!dev) {
         rc = c->cuda(cudaMemcpyAsync(out, dst, sizeof(double) * h.nf * h.N, cudaMemcpyDeviceToHost, c->stream), "copy");
@@ -1108,6 +1113,7 @@ void mrg_tables(Tables<double> *td, Tables<float> *tf) { make_tables(*td, *tf); 
 int mrg_nfields(int eq) { return nfields_of(eq); }
 int mrg_npop(int eq) { return npop_of(eq); }
 int mrg_nrates(int eq) { return nrates_of(eq); }
+int mrg_variant(int eq) { return variant_of(eq); }
 void mrg_dq_inverse(int eq, double lambda, double inv[5][5]) { dq_inverse(eq, lambda, inv); }
 
 // Message reported by mr_last_error(NULL, ...) for calls without a context.

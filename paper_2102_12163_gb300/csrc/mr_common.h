@@ -35,7 +35,7 @@ enum { M_I0 = 0, M_I1 = 1, M_KEEP = 2, M_REF = 3, NMASK = 4 };
 // segments by level
 enum { L_INT = 0, L_PRED = 1, L_GH = 2, L_LEAF = 3, NLIST = 4, NSEG = 3 };
 // phases of the persistent kernel
-enum { PH_INIT_FULL = 1, PH_INIT_STATE = 2, PH_ADAPT = 4, PH_STEP = 8, PH_FINEST = 16 };
+enum { PH_INIT_FULL = 1, PH_INIT_STATE = 2, PH_ADAPT = 4, PH_STEP = 8 };
 // device status bits
 enum { ST_NONFINITE = 1 };
 // phases timed by the profiling build (MRG_PHASE_TIMERS)
@@ -185,6 +185,9 @@ int mrg_launch(bool fp32, int block, int grid, const mrg::LaunchArgs &a, void *s
 int mrg_occupancy(bool fp32, int block, int kind, int mask_words, int *blocks_per_sm);
 int mrg_min_blocks(bool fp32, int block, int kind);  // residency the variant is compiled for
 size_t mrg_smem_bytes(bool fp32, int block, int mask_words);
+// reconstruction of one instance (scheme variant var: D1Q2^1..3, 4 D1Q3, 5 D1Q5)
+// on its finest level, into device memory (mr_field.cu)
+int mrg_finest(bool fp32, int var, int Jmax, const mrg::InstDesc *desc, const void *tables, double *out, void *stream);
 void mrg_tables(mrg::Tables<double> *td, mrg::Tables<float> *tf);
 void mrg_set_error(const char *msg);
 // scheme shape (mr_api.cu): conserved fields, populations, relaxation rates of
@@ -192,5 +195,6 @@ void mrg_set_error(const char *msg);
 int mrg_nfields(int eq);
 int mrg_npop(int eq);
 int mrg_nrates(int eq);
+int mrg_variant(int eq);  // compiled scheme variant of the kernels
 void mrg_dq_inverse(int eq, double lambda, double inv[5][5]);
 }

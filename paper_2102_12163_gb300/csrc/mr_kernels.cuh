@@ -1920,28 +1920,6 @@ struct Worker {
         if (tid == TS - 1) sm.passes = 0ULL;  // the thread that counts the barriers
         sync();
     }
-
-    // ---- multiresolution reconstruction on the finest level (measurement) ----
-    __device__ __noinline__ void finest(double *out) {
-        fill_finest();
-        const int N = 1 << Jmax;
-#pragma unroll 1
-        for (int k = tid; k < N; k += TS) {
-            const T *f = cell((uint32_t)(N + k));
-            if constexpr (DQ) {
-                double m0 = 0.0, m1 = 0.0;
-                for (int h = 0; h < q; ++h) {
-                    m0 += (double)f[h];
-                    m1 += (dq_w(h) * d.lam) * (double)f[h];
-                }
-                out[k] = m0;
-                out[(long long)N + k] = m1;
-            } else {
-                for (int j = 0; j < nf; ++j) out[(long long)j * N + k] = (double)f[2 * j] + (double)f[2 * j + 1];
-            }
-        }
-        sync();
-    }
 };
 
 // ---------------------------------------------------------------------------
@@ -2020,7 +1998,6 @@ __device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &t
         if (a.phases & PH_ADAPT) w.adapt();
         if (a.phases & PH_STEP) w.lbm_step();
     }
-    if (a.phases & PH_FINEST) w.finest((double *)a.aux0);
 }
 
 // The bit arrays live in shared memory (smask, room for `cap` words) when the

@@ -145,7 +145,8 @@ struct mr_ctx {
     int precision = MR_FP64;
     // layout (bytes from the workspace base)
     size_t off_desc = 0, off_state = 0, off_order = 0, off_ident = 0, off_queue = 0, off_tab = 0,
-           off_stage = 0, total = 0;
+           off_stage = 0, off_chunk = 0, total = 0;
+    int nchunk = 0;                // runs of the initial state over all instances
     std::vector<size_t> inst_off;  // per instance region start
     std::vector<InstDesc> hdesc;   // host copy of the device descriptors
     std::vector<long long> m_off;  // per instance offset in the initial-data array
@@ -239,6 +240,11 @@ static void layout(mr_ctx *c) {
     c->stage_doubles = st;
     c->off_stage = o;
     o = align_up(o + st * sizeof(double));
+    c->nchunk = 0;
+    for (int i = 0; i < n; ++i) c->nchunk += init_chunks_of(c->desc[i].Jmax);
+    c->off_chunk = o;
+    o = align_up(o + sizeof(int) * (size_t)c->nchunk);
+    int chunk0 = 0;
     c->inst_off.assign(n, 0);
     c->hdesc.assign(n, InstDesc{});
     for (int i = 0; i < n; ++i) {
@@ -274,6 +280,8 @@ static void layout(mr_ctx *c) {
         h.S = S;
         h.N = N;
         h.m_off = c->m_off[i];
+        h.chunk0 = chunk0;
+        chunk0 += init_chunks_of(d.Jmax);
         c->inst_off[i] = o;
         size_t vb = c->vbytes();
         size_t oV = 0, oPhi = align_up(oV + vb * q * S), oM = align_up(oPhi + vb * q * (N + 1));
@@ -657,6 +665,10 @@ mr_status mr_bind(mr_ctx *c, void *ws, size_t bytes, void *stream) {
     if ((rc = c->cuda(cudaMemcpyAsync(c->ws + c->off_tab, &td, sizeof td, cudaMemcpyHostToDevice, s), "upload"))) return (mr_status)rc;
     if ((rc = c->cuda(cudaMemcpyAsync(c->ws + c->off_tab + sizeof td, &tf, sizeof tf, cudaMemcpyHostToDevice, s), "upload")))
         return (mr_status)rc;
+    std::vector<int> chunk_inst((size_t)c->nchunk);
+    for (int i = 0; i < n; ++i) std::fill_n(chunk_inst.begin() + dd[i].chunk0, init_chunks_of(dd[i].Jmax), i);
+    if ((rc = c->cuda(cudaMemcpyAsync(c->ws + c->off_chunk, chunk_inst.data(), sizeof(int) * chunk_inst.size(), cudaMemcpyHostToDevice, s), "upload")))
+        return (mr_status)rc;
     if ((rc = c->cuda(cudaStreamSynchronize(s), "cudaStreamSynchronize"))) return (mr_status)rc;
     c->wmax = 0;
     for (int i = 0; i < n; ++i) c->wmax = std::max(c->wmax, (int)smem_region_words(dd[i].Wtot, dd[i].OW));
@@ -678,7 +690,11 @@ mr_status mr_set_initial(mr_ctx *c, const double *m, size_t count) {
         if (rc) return (mr_status)rc;
         src = c->ws + c->off_stage;
     }
-    int rc = launch(c, PH_INIT_FULL, 0, -1, src, nullptr);
+    int rc = c->cuda((cudaError_t)mrg_init(c->fp32(), (const InstDesc *)(c->ws + c->off_desc), (const int *)(c->ws + c->off_chunk),
+                                           c->nchunk, c->ws + c->off_tab + (c->fp32() ? sizeof(Tables<double>) : 0),
+                                           (const double *)src, c->stream),
+                     "kernel launch");
+    c->launches += 2;
     if (rc) return (mr_status)rc;
     c->initialised = true;
     return MR_OK;

@@ -35,9 +35,11 @@ enum { M_I0 = 0, M_I1 = 1, M_KEEP = 2, M_REF = 3, NMASK = 4 };
 // segments by level
 enum { L_INT = 0, L_PRED = 1, L_GH = 2, L_LEAF = 3, NLIST = 4, NSEG = 3 };
 // phases of the persistent kernel
-enum { PH_INIT_FULL = 1, PH_INIT_STATE = 2, PH_ADAPT = 4, PH_STEP = 8 };
+enum { PH_INIT_STATE = 2, PH_ADAPT = 4, PH_STEP = 8 };
 // device status bits
-enum { ST_NONFINITE = 1 };
+// ST_DETAILS: KEEP and REF hold the decisions of the initial state, for the
+// first adaptation (mr_set_initial takes them over the whole GPU)
+enum { ST_NONFINITE = 1, ST_DETAILS = 2 };
 // phases timed by the profiling build (MRG_PHASE_TIMERS)
 enum {
     T_UPSWEEP_A = 0, T_DETAILS, T_ENLARGE, T_GRADE, T_GRADE_SMALL, T_CANDIDATES, T_LISTS, T_TRANSFER,
@@ -50,6 +52,8 @@ struct InstState {
     int seg[NSEG][MAXLEV + 2];    // list segments: level l >= 5 at [seg[l], seg[l+1]), the levels below it at [0, seg[5])
     int status;                   // ST_* bits
     int near_ties;                // threshold decisions within 1e-12 relative of the threshold
+    int first_ties;               // near ties among the decisions of the initial state
+    unsigned chunks;              // runs of the initial state done, while it is set
     unsigned deplev[2];           // levels holding transfer / ghost pairs that wait on the same list
     unsigned long long updates;   // sum over steps of #S(Lambda^{n+1})
     unsigned long long steps;
@@ -71,6 +75,7 @@ struct InstDesc {
     long long S;           // cells over all levels
     long long N;           // 2^Jmax
     long long m_off;       // offset of this instance's initial data in the input array
+    int chunk0;            // its first run of INIT_CELLS finest cells among those of all instances
     void *V;
     void *Phi;
     uint32_t *masks;
@@ -150,6 +155,10 @@ struct Tables {
     T pc[4][3];
 };
 
+// the initial state is set by runs of this many finest cells (2^Jmax when fewer)
+constexpr int INIT_CELLS = 512;
+MRG_HD inline int init_chunks_of(int Jmax) { return Jmax > 9 ? 1 << (Jmax - 9) : 1; }
+
 struct LaunchArgs {
     const InstDesc *descs;
     const int *order;     // instance processing order (longest first)
@@ -185,6 +194,10 @@ int mrg_launch(bool fp32, int block, int grid, const mrg::LaunchArgs &a, void *s
 int mrg_occupancy(bool fp32, int block, int kind, int mask_words, int *blocks_per_sm);
 int mrg_min_blocks(bool fp32, int block, int kind);  // residency the variant is compiled for
 size_t mrg_smem_bytes(bool fp32, int block, int mask_words);
+// initial state of n instances from their conserved moments (mr_field.cu);
+// chunk_inst: the instance of each of the nchunk runs (null: instance 0)
+int mrg_init(bool fp32, const mrg::InstDesc *descs, const int *chunk_inst, int nchunk, const void *tables, const double *mcons,
+             void *stream);
 // reconstruction of one instance (scheme variant var: D1Q2^1..3, 4 D1Q3, 5 D1Q5)
 // on its finest level, into device memory (mr_field.cu)
 int mrg_finest(bool fp32, int var, int Jmax, const mrg::InstDesc *desc, const void *tables, double *out, void *stream);

@@ -1,5 +1,6 @@
-// mr_field.cu -- whole-field kernels, spread over the GPU: the reconstruction
-// of an instance on its finest level (mr_get_finest, mr_run_static).
+// mr_field.cu -- whole-field kernels, spread over the GPU: the initial state
+// (mr_set_initial) and the reconstruction of an instance on its finest level
+// (mr_get_finest); mr_run_static uses both.
 //
 // The persistent kernel gives an instance one block, which suits a step over a
 // few hundred cells and not a pass over 2^Jmax of them.  Here a block owns a
@@ -111,6 +112,216 @@ __global__ void __launch_bounds__(256) mr_finest(const InstDesc *desc, const Tab
     }
 }
 
+// ---------------------------------------------------------------------------
+// Initial state: the full tree, populations at equilibrium, projections of every
+// level, lists, and the details' decisions for the first adaptation.
+//
+// mr_init_cells: a block takes a run of INIT_CELLS finest cells, evaluates their
+// populations and projects them in shared memory up to the one cell (or, below
+// Jmin, to level Jmin) above the run; the block that finishes an instance last
+// (a ticket, no waiting) projects the levels above the runs, folds the runs'
+// totals in their order and writes the state.  mr_init_details: a warp takes a
+// word of 32 internal cells and writes their KEEP and REF words.
+// What bounds them: FP64 operations of the equilibria and the 3 q of a detail
+// (two lanes a cycle and SM), and for small schemes the traffic, 2 q values
+// written and read per finest cell.  One block per instance took 2.6 ms for the
+// batch of 4096 (FP64) and 11 ms for a lone Euler instance of Jmax = 18 (FP32),
+// and the first adaptation 0.9 ms more for the latter.
+template <typename T, int NF>
+__device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const double *mcons, unsigned char *smem) {
+    constexpr bool DQ = NF >= 4;
+    constexpr int q = DQ ? (NF == 4 ? 3 : 5) : 2 * NF, nf = DQ ? 2 : NF;
+    const int Jmin = d.Jmin, Jmax = d.Jmax, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = 1 << Jmax, ch = min(INIT_CELLS, N), nch = init_chunks_of(Jmax), c0 = chunk * ch;
+    T *a = (T *)smem, *b = a + INIT_CELLS * q;
+    double(*red)[8] = (double(*)[8])(smem + sizeof(T) * q * (INIT_CELLS + INIT_CELLS / 2));
+    T *V = (T *)d.V - (1LL << Jmin) * q;
+    uint32_t *leaves = d.lists + d.list_off[L_LEAF], *inner = d.lists + d.list_off[L_INT] - (1 << Jmin);
+    const double dx = ldexp(d.b - d.a, -Jmax);
+    double m[3] = {0.0, 0.0, 0.0};
+    for (int t = tid; t < ch; t += 256) {
+        const int k = c0 + t;
+        double mc[3], f[q];
+        for (int j = 0; j < nf; ++j) mc[j] = mcons[(long long)j * N + k];
+        if constexpr (DQ)
+            dq_equilibrium_populations<q>(d, mc, f);
+        else
+            equilibrium_populations<NF>(d, mc, f);
+        double m0 = 0.0, m1 = 0.0;
+#pragma unroll
+        for (int j = 0; j < q; ++j) {
+            const T x = (T)f[j];
+            a[t * q + j] = x;
+            V[(size_t)(N + k) * q + j] = x;
+            if constexpr (DQ) {
+                m0 += (double)x;
+                m1 += (dq_w(j) * d.lam) * (double)x;
+            }
+        }
+        if constexpr (DQ) {
+            m[0] += dx * m0;
+            m[1] += dx * m1;
+        } else {
+#pragma unroll
+            for (int j = 0; j < nf; ++j) m[j] += dx * ((double)a[t * q + 2 * j] + (double)a[t * q + 2 * j + 1]);
+        }
+        leaves[k] = (uint32_t)(N + k);
+    }
+    // the run's totals, into the interface array (free until the first step)
+#pragma unroll
+    for (int j = 0; j < nf; ++j) {
+        for (int o = 16; o > 0; o >>= 1) m[j] += __shfl_down_sync(FULL, m[j], o);
+        if (lane == 0) red[j][warp] = m[j];
+    }
+    __syncthreads();
+    if (tid < nf) {
+        double x = 0.0;
+        for (int w = 0; w < 8; ++w) x += red[tid][w];
+        ((double *)d.Phi)[3 * chunk + tid] = x;
+    }
+    int l = Jmax - 1;
+    for (int n = ch / 2; n >= 1 && l >= Jmin; n >>= 1, --l) {
+        const uint32_t h0 = (1u << l) + (uint32_t)(c0 >> (Jmax - l));
+        for (int t = tid; t < n; t += 256) {
+#pragma unroll
+            for (int j = 0; j < q; ++j) {
+                const T x = half_of<T>(a[2 * t * q + j] + a[(2 * t + 1) * q + j]);
+                b[t * q + j] = x;
+                V[(size_t)(h0 + t) * q + j] = x;
+            }
+            inner[h0 + t] = h0 + t;
+        }
+        __syncthreads();
+        T *x = a;
+        a = b;
+        b = x;
+    }
+    // the tree: every cell above Jmax is internal; the runs share the words
+    const int W = d.Wtot, wpc = W / nch;
+    for (int w = chunk * wpc + tid; w < (chunk + 1) * wpc; w += 256)
+        d.masks[w] = w == 0 ? (Jmax >= 5 ? 0xFFFFFFFEu : (1u << (1 << Jmax)) - 2u) : FULL;
+    // the run that finishes last completes the instance
+    InstState &st = *d.st;
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&st.chunks, 1u) == (unsigned)(nch - 1);
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (l = Jmax - 10; l >= Jmin; --l) {  // the levels above the runs, from values in L2
+        for (uint32_t h = (1u << l) + tid; h < (2u << l); h += 256) {
+#pragma unroll
+            for (int j = 0; j < q; ++j)
+                V[(size_t)h * q + j] = half_of<T>(__ldcg(&V[(size_t)(2u * h) * q + j]) + __ldcg(&V[(size_t)(2u * h + 1u) * q + j]));
+            inner[h] = h;
+        }
+        __threadfence_block();
+        __syncthreads();
+    }
+    for (int j = 0; j < nf; ++j) {
+        double x = 0.0;
+        for (int c = tid; c < nch; c += 256) x += __ldcg((const double *)d.Phi + 3 * c + j);
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(FULL, x, o);
+        if (lane == 0) red[j][warp] = x;
+    }
+    for (int j = tid; j < d.OW; j += 256) {  // occupancy of the tree: no word is empty
+        uint32_t *occ = d.masks + (long long)(NMASK + 1) * W;
+        occ[j] = W >= 32 ? FULL : (1u << W) - 1u;
+    }
+    for (int k = tid; k < MAXLEV + 2; k += 256) {
+        st.seg[L_INT][k] = max(0, (1 << min(k, Jmax)) - (1 << Jmin));
+        st.seg[L_PRED][k] = st.seg[L_GH][k] = 0;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int j = 0; j < 3; ++j) {
+            double x = 0.0;
+            if (j < nf)
+                for (int w = 0; w < 8; ++w) x += red[j][w];
+            st.mass[j] = x;
+        }
+        st.cur = M_I0;
+        st.nleaf = N;
+        st.status = ST_DETAILS;
+        st.near_ties = st.first_ties = 0;
+        st.deplev[0] = st.deplev[1] = 0u;
+        st.updates = st.steps = st.passes = 0ULL;
+        st.audit = 0.0;
+        st.chunks = 0u;
+#ifdef MRG_PHASE_TIMERS
+        for (int p = 0; p < NPHASE; ++p) st.ptime[p] = 0ULL;
+#endif
+    }
+}
+
+__device__ __forceinline__ int variant_of_desc(const InstDesc &d) { return d.eq == 4 ? 4 : d.eq == 5 ? 5 : d.nf; }
+
+template <typename T>
+__global__ void __launch_bounds__(256) mr_init_cells(const InstDesc *descs, const int *chunk_inst, const double *mcons) {
+    __shared__ __align__(16) unsigned char smem[sizeof(T) * 6 * (INIT_CELLS + INIT_CELLS / 2) + 3 * 8 * sizeof(double)];
+    const int inst = chunk_inst ? chunk_inst[blockIdx.x] : 0;
+    const InstDesc &d = descs[inst];
+    const int chunk = (int)blockIdx.x - (chunk_inst ? d.chunk0 : 0);
+    const double *m = mcons + d.m_off;
+    switch (variant_of_desc(d)) {
+    case 1: init_cells<T, 1>(d, chunk, m, smem); break;
+    case 2: init_cells<T, 2>(d, chunk, m, smem); break;
+    case 3: init_cells<T, 3>(d, chunk, m, smem); break;
+    case 4: init_cells<T, 4>(d, chunk, m, smem); break;
+    default: init_cells<T, 5>(d, chunk, m, smem); break;
+    }
+}
+
+template <typename T, int q, bool WIDE>
+__device__ __forceinline__ void init_details(const InstDesc &d, int chunk, const Tables<T> &tab, const Thresholds &th) {
+    const int W = d.Wtot, wpc = W / init_chunks_of(d.Jmax), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const T *V = (const T *)d.V - (1LL << d.Jmin) * q;
+    for (int w = chunk * wpc + warp; w < (chunk + 1) * wpc; w += 8) {
+        const uint32_t p = 32u * w + lane;
+        bool keep = false, ref = false, tie = false;
+        if (p >= (1u << d.Jmin) && p < (1u << d.Jmax))
+            pair_decision<T, q, WIDE>(V, p, d.Jmax, d.bc, d.gamma, tab, th, keep, ref, tie);
+        const unsigned kb = __ballot_sync(FULL, keep), rb = __ballot_sync(FULL, ref), tb = __ballot_sync(FULL, tie);
+        if (lane == 0) {
+            d.masks[(long long)M_KEEP * W + w] = kb;
+            d.masks[(long long)M_REF * W + w] = rb;
+            if (tb) atomicAdd(&d.st->first_ties, __popc(tb));
+        }
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) mr_init_details(const InstDesc *descs, const int *chunk_inst, const Tables<T> *tabs) {
+    __shared__ Thresholds th;
+    const int inst = chunk_inst ? chunk_inst[blockIdx.x] : 0;
+    const InstDesc &d = descs[inst];
+    const int chunk = (int)blockIdx.x - (chunk_inst ? d.chunk0 : 0);
+    for (int l = threadIdx.x; l <= MAXLEV; l += 256) th.set(d, l);
+    __syncthreads();
+    const Tables<T> &tab = *tabs;
+    switch (variant_of_desc(d) + (d.gamma > 1 ? 8 : 0)) {
+    case 1: init_details<T, 2, false>(d, chunk, tab, th); break;
+    case 2: init_details<T, 4, false>(d, chunk, tab, th); break;
+    case 3: init_details<T, 6, false>(d, chunk, tab, th); break;
+    case 4: init_details<T, 3, false>(d, chunk, tab, th); break;
+    case 5: init_details<T, 5, false>(d, chunk, tab, th); break;
+    case 9: init_details<T, 2, true>(d, chunk, tab, th); break;
+    case 10: init_details<T, 4, true>(d, chunk, tab, th); break;
+    default: init_details<T, 6, true>(d, chunk, tab, th); break;
+    }
+}
+
+template <typename T>
+static cudaError_t init_of(const InstDesc *descs, const int *chunk_inst, int nchunk, const Tables<T> *tabs, const double *mcons,
+                           cudaStream_t s) {
+    mr_init_cells<T><<<nchunk, 256, 0, s>>>(descs, chunk_inst, mcons);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    mr_init_details<T><<<nchunk, 256, 0, s>>>(descs, chunk_inst, tabs);
+    return cudaGetLastError();
+}
+
 template <typename T>
 static cudaError_t finest_of(int var, int Jmax, const InstDesc *desc, const Tables<T> *tabs, double *out, cudaStream_t s) {
     const int grid = Jmax > 9 ? 1 << (Jmax - 9) : 1;
@@ -131,4 +342,11 @@ static cudaError_t finest_of(int var, int Jmax, const InstDesc *desc, const Tabl
 int mrg_finest(bool fp32, int var, int Jmax, const mrg::InstDesc *desc, const void *tables, double *out, void *stream) {
     if (fp32) return (int)mrg::finest_of<float>(var, Jmax, desc, (const mrg::Tables<float> *)tables, out, (cudaStream_t)stream);
     return (int)mrg::finest_of<double>(var, Jmax, desc, (const mrg::Tables<double> *)tables, out, (cudaStream_t)stream);
+}
+
+int mrg_init(bool fp32, const mrg::InstDesc *descs, const int *chunk_inst, int nchunk, const void *tables, const double *mcons,
+             void *stream) {
+    if (fp32)
+        return (int)mrg::init_of<float>(descs, chunk_inst, nchunk, (const mrg::Tables<float> *)tables, mcons, (cudaStream_t)stream);
+    return (int)mrg::init_of<double>(descs, chunk_inst, nchunk, (const mrg::Tables<double> *)tables, mcons, (cudaStream_t)stream);
 }

@@ -169,13 +169,27 @@ __device__ __forceinline__ uint32_t graded_parents(uint32_t x, uint32_t xl, uint
 // ---------------------------------------------------------------------------
 // shared memory: per-team state and per-block tables
 
+// eps_l = 2^{l - Jmax} eps (Prop. ErrorControl) and the Harten level
+// 2^{mu_bar + 1} eps_l, with their roundings to float
+struct Thresholds {
+    double eps_l[MAXLEV + 1], big_l[MAXLEV + 1];
+    float eps_f[MAXLEV + 1], big_f[MAXLEV + 1];
+    __device__ __forceinline__ void set(const InstDesc &d, int l) {
+        const double el = ldexp(d.eps, l - d.Jmax), bl = ldexp(el, d.mu_bar + 1);
+        eps_l[l] = el;
+        big_l[l] = bl;
+        eps_f[l] = (float)el;
+        big_f[l] = (float)bl;
+    }
+};
+
 template <typename T>
 struct TeamSmem {
     InstDesc d;
     int cw_seg[MAXLEV + 2];  // candidate words of level l >= 5: entries [cw_seg[l], cw_seg[l+1]) of their list
     int seg[NSEG][MAXLEV + 2];
-    double eps_l[MAXLEV + 1], big_l[MAXLEV + 1], dx_l[MAXLEV + 1];  // per level
-    float eps_f[MAXLEV + 1], big_f[MAXLEV + 1];
+    Thresholds th;
+    double dx_l[MAXLEV + 1];  // cell size per level
     double mass[3];
     double audit;
     unsigned long long updates, steps, passes;
@@ -366,9 +380,9 @@ __device__ __forceinline__ void equilibrium_populations(const InstDesc &d, const
     equilibria<double, NF>(d, d.eqp, mc, meq);
 #pragma unroll
     for (int i = 0; i < NF; ++i) {
-        double g = A::div(meq[i], d.lam);
-        f[2 * i] = A::mul(0.5, A::add(mc[i], g));
-        f[2 * i + 1] = A::mul(0.5, A::sub(mc[i], g));
+        const double g = d.lam_log2 != NOT_POW2 ? scale2(meq[i], -d.lam_log2) : div_lam<double>(meq[i], d);  // meq / lambda
+        f[2 * i] = half_f64(A::add(mc[i], g));
+        f[2 * i + 1] = half_f64(A::sub(mc[i], g));
     }
 }
 
@@ -464,6 +478,92 @@ __device__ __forceinline__ void decide_bits(unsigned long long Db, double el, do
     if ((de < 16384 && de > -16384) || (hasref && db < 16384 && db > -16384)) {
         const double D = __longlong_as_double((long long)Db);
         tie = fabs(D - el) <= 1e-12 * el || (hasref && fabs(D - bl) <= 1e-12 * bl);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// prediction stencils and the threshold decision of one pair
+
+// sum_a c_a (f_{p+a} - f_{p-a}) of population h with the stencil of half-width
+// g (coefficients c, in increasing a), given the gamma = 1 sum first (used as it
+// is when g = 1); V: cell x at V + x q, lo: first cell of p's level
+template <typename T, int q>
+__device__ __forceinline__ T wide_sum(const T *V, uint32_t p, uint32_t lo, int bc, int g, const T *c, int h, T first) {
+    if (g == 1) return first;
+    auto at = [&](int a) { return V[neighbour(p, a, lo, bc) * (uint32_t)q + (uint32_t)h]; };
+    T sum = c[0] * (at(1) - at(-1));
+#pragma unroll 1
+    for (int a = 2; a <= g; ++a) sum = sum + c[a - 1] * (at(a) - at(-a));
+    return sum;
+}
+
+// Keep / refine decision of the children of p (Sections 3.2, 3.4, 4.2), and
+// whether it lies within 1e-12 relative of a threshold.  FP64: the detail in
+// double.  FP32: the detail in float with a rigorous bound on its rounding
+// error; only when a threshold lies within that bound is the detail recomputed
+// in FP64 from the stored values, so every decision equals the one the exact
+// detail of the stored state gives.
+template <typename T, int q, bool WIDE>
+__device__ __forceinline__ void pair_decision(const T *V, uint32_t p, int Jmax, int bc, int g, const Tables<T> &tab,
+                                              const Thresholds &th, bool &keepit, bool &refit, bool &tie) {
+    const uint32_t lo = level_first(p);
+    const int l = level_of(p) + 1;
+    const bool hasref = l < Jmax;
+    tie = false;
+    const T *vk = V + 2u * p * (uint32_t)q, *vp = V + p * (uint32_t)q, *vl = V + neighbour(p, -1, lo, bc) * (uint32_t)q,
+            *vr = V + neighbour(p, 1, lo, bc) * (uint32_t)q;
+    const T *c = tab.pc[g];
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long Db = 0ull;
+#pragma unroll
+        for (int h = 0; h < q; ++h) {
+            double sum = C1 * (vr[h] - vl[h]);
+            if constexpr (WIDE) sum = wide_sum<T, q>(V, p, lo, bc, g, c, h, sum);
+            const unsigned long long b = abs_bits(vk[h] - (vp[h] + sum));
+            Db = b > Db ? b : Db;
+        }
+        decide_bits(Db, th.eps_l[l], th.big_l[l], hasref, keepit, refit, tie);
+    } else {
+        float D = 0.0f, B = 0.0f;
+#pragma unroll
+        for (int h = 0; h < q; ++h) {
+            const float xk = vk[h], xp = vp[h], xl = vl[h], xr = vr[h];
+            float sum = float(C1) * (xr - xl), mag = fabsf(xl) + fabsf(xr);
+            if constexpr (WIDE) {
+                sum = wide_sum<T, q>(V, p, lo, bc, g, c, h, sum);
+#pragma unroll 1
+                for (int a = 2; a <= g; ++a)
+                    mag += fabsf(V[neighbour(p, a, lo, bc) * (uint32_t)q + h]) + fabsf(V[neighbour(p, -a, lo, bc) * (uint32_t)q + h]);
+            }
+            D = fmaxf(D, fabsf(xk - (xp + sum)));
+            B = fmaxf(B, fabsf(xk) + fabsf(xp) + mag);
+        }
+        // the rounding of the detail: for gamma = 1 4 times the bound of its
+        // evaluation; (6 gamma + 2) u times the sum of |inputs| else (3 gamma + 1
+        // roundings, each at most u times that sum, with a factor 2 margin)
+        B *= WIDE && g > 1 ? (float)(6 * g + 2) * 0x1p-24f : 0x1p-21f;
+        const float el = th.eps_f[l], bl = th.big_f[l];
+        // the band also covers the rounding of the thresholds to float
+        const bool amb = fabsf(D - el) <= B + el * 0x1p-22f || (hasref && fabsf(D - bl) <= B + bl * 0x1p-22f);
+        if (amb) {
+            double Dd = 0.0;
+#pragma unroll 1
+            for (int h = 0; h < q; ++h) {
+                double sum = (WIDE ? (double)c[0] : C1) * ((double)vr[h] - (double)vl[h]);
+                if constexpr (WIDE)
+                    for (int a = 2; a <= g; ++a)
+                        sum = sum + (double)c[a - 1] * ((double)V[neighbour(p, a, lo, bc) * (uint32_t)q + h] -
+                                                        (double)V[neighbour(p, -a, lo, bc) * (uint32_t)q + h]);
+                Dd = fmax(Dd, fabs((double)vk[h] - ((double)vp[h] + sum)));
+            }
+            const double e64 = th.eps_l[l], b64 = th.big_l[l];
+            keepit = Dd >= e64;
+            refit = hasref && Dd >= b64;
+            tie = fabs(Dd - e64) <= 1e-12 * e64 || (hasref && fabs(Dd - b64) <= 1e-12 * b64);
+        } else {
+            keepit = D >= el;
+            refit = hasref && D >= bl;
+        }
     }
 }
 
@@ -885,74 +985,17 @@ struct Worker {
     }
 
     // ---- A2: details of the pairs of the tree, threshold T, Harten flags ----
-    // FP64: the detail of Section 3.2 in double.  FP32: the detail in float with
-    // a rigorous bound on its rounding error; only when a threshold lies within
-    // that bound is the detail recomputed in FP64 from the stored values, so
-    // every decision equals the one the exact detail of the stored state gives.
     // KEEP / REF bits go to the pair's parent p (both children of a kept pair
-    // are kept).  The prediction sums c_a (f_{p+a} - f_{p-a}) in increasing a.
+    // are kept)
     __device__ void details() {
         const uint32_t *lst = list(L_INT);
         const int e = sm.seg[L_INT][top()];
-        const int g = WIDE ? d.gamma : 1;
         uint32_t *keep = mask(M_KEEP), *ref = mask(M_REF);
 #pragma unroll 1
         for (int i = tid; i < e; i += TS) {
             const uint32_t p = lst[i];
-            const uint32_t lo = level_first(p);
-            const int l = level_of(p) + 1;
-            const bool hasref = l < Jmax;
-            bool keepit, refit, tie = false;
-            const T *vk = cell(2u * p), *vp = cell(p), *vl = cell(nb(p, -1, lo)), *vr = cell(nb(p, 1, lo));
-            if constexpr (sizeof(T) == 8) {
-                unsigned long long Db = 0ull;
-#pragma unroll
-                for (int h = 0; h < q; ++h) {
-                    double sum = C1 * (vr[h] - vl[h]);
-                    if constexpr (WIDE) sum = wide_sum(p, lo, h, sum);
-                    const unsigned long long b = abs_bits(vk[h] - (vp[h] + sum));
-                    Db = b > Db ? b : Db;
-                }
-                decide_bits(Db, sm.eps_l[l], sm.big_l[l], hasref, keepit, refit, tie);
-            } else {
-                float D = 0.0f, B = 0.0f;
-#pragma unroll
-                for (int h = 0; h < q; ++h) {
-                    const float xk = vk[h], xp = vp[h], xl = vl[h], xr = vr[h];
-                    float sum = float(C1) * (xr - xl), mag = fabsf(xl) + fabsf(xr);
-                    if constexpr (WIDE) {
-                        sum = wide_sum(p, lo, h, sum);
-                        mag += wide_mag(p, lo, h);
-                    }
-                    D = fmaxf(D, fabsf(xk - (xp + sum)));
-                    B = fmaxf(B, fabsf(xk) + fabsf(xp) + mag);
-                }
-                // the rounding of the detail: for gamma = 1 4 times the bound of its
-                // evaluation; (6 gamma + 2) u times the sum of |inputs| else (3 gamma + 1
-                // roundings, each at most u times that sum, with a factor 2 margin)
-                B *= WIDE && g > 1 ? (float)(6 * g + 2) * 0x1p-24f : 0x1p-21f;
-                const float el = sm.eps_f[l], bl = sm.big_f[l];
-                // the band also covers the rounding of the thresholds to float
-                const bool amb = fabsf(D - el) <= B + el * 0x1p-22f || (hasref && fabsf(D - bl) <= B + bl * 0x1p-22f);
-                if (amb) {
-                    double Dd = 0.0;
-#pragma unroll 1
-                    for (int h = 0; h < q; ++h) {
-                        double sum = (WIDE ? (double)tab.pc[g][0] : C1) * ((double)vr[h] - (double)vl[h]);
-                        if constexpr (WIDE)
-                            for (int a = 2; a <= g; ++a)
-                                sum = sum + (double)tab.pc[g][a - 1] * ((double)cell(nb(p, a, lo))[h] - (double)cell(nb(p, -a, lo))[h]);
-                        Dd = fmax(Dd, fabs((double)vk[h] - ((double)vp[h] + sum)));
-                    }
-                    const double e64 = sm.eps_l[l], b64 = sm.big_l[l];
-                    keepit = Dd >= e64;
-                    refit = hasref && Dd >= b64;
-                    tie = fabs(Dd - e64) <= 1e-12 * e64 || (hasref && fabs(Dd - b64) <= 1e-12 * b64);
-                } else {
-                    keepit = D >= el;
-                    refit = hasref && D >= bl;
-                }
-            }
+            bool keepit, refit, tie;
+            pair_decision<T, q, WIDE>(V, p, Jmax, bc, WIDE ? d.gamma : 1, tab, sm.th, keepit, refit, tie);
             if (tie) atomicAdd(&sm.near_ties, 1);
             if (keepit) {
                 const uint32_t bit = 1u << (p & 31u);
@@ -961,24 +1004,6 @@ struct Worker {
             }
         }
     }
-    // sum_a c_a (f_{p+a} - f_{p-a}) of population h with the instance's stencil,
-    // given the gamma = 1 sum first (used as it is when gamma = 1)
-    __device__ __forceinline__ T wide_sum(uint32_t p, uint32_t lo, int h, T first) const {
-        const int g = d.gamma;
-        if (g == 1) return first;
-        const T *c = tab.pc[g];
-        T sum = c[0] * (cell(nb(p, 1, lo))[h] - cell(nb(p, -1, lo))[h]);
-#pragma unroll 1
-        for (int a = 2; a <= g; ++a) sum = sum + c[a - 1] * (cell(nb(p, a, lo))[h] - cell(nb(p, -a, lo))[h]);
-        return sum;
-    }
-    __device__ __forceinline__ float wide_mag(uint32_t p, uint32_t lo, int h) const {
-        float m = 0.0f;
-#pragma unroll 1
-        for (int a = 2; a <= d.gamma; ++a) m += fabsf((float)cell(nb(p, a, lo))[h]) + fabsf((float)cell(nb(p, -a, lo))[h]);
-        return m;
-    }
-
     // ---- candidate words of the step -----------------------------------------
     // (gamma = 1.)  A cell that becomes internal is within one cell of a kept
     // one, a child of a refined one, or an ancestor that grading requires, and
@@ -1272,7 +1297,7 @@ struct Worker {
 #pragma unroll
         for (int h = 0; h < q; ++h) {
             T t = T(C1) * (vr[h] - vl[h]);  // exact: c_1 is a power of two
-            if constexpr (WIDE) t = wide_sum(p, lo, h, t);
+            if constexpr (WIDE) t = wide_sum<T, q>(V, p, lo, bc, d.gamma, tab.pc[d.gamma], h, t);
             a[h] = vp[h] + t;
             a[q + h] = vp[h] - t;
         }
@@ -1330,7 +1355,7 @@ struct Worker {
             for (int j = tid; j < d.OW; j += TS) on[j] = 0u;
         }
         tick(T_CANDIDATES);
-        details();
+        if (!(sm.status & ST_DETAILS)) details();  // else the initial state came with its decisions
         sync();
         tick(T_DETAILS);
         enlarge(In);
@@ -1354,6 +1379,10 @@ struct Worker {
         if (tid == 0) {
             sm.cur ^= 1;
             sm.updates += (unsigned long long)sm.nleaf;
+            if (sm.status & ST_DETAILS) {
+                sm.near_ties += d.st->first_ties;
+                sm.status &= ~(int)ST_DETAILS;
+            }
         }
         sync();
     }
@@ -1361,6 +1390,12 @@ struct Worker {
     // ---- one step of the adaptive scheme on the current mesh -----------------
     __device__ void lbm_step() {
         tick(NPHASE);
+        if (sm.status & ST_DETAILS) {
+            // the step moves the state that the initial decisions belong to
+            clear_masks();
+            sync();
+            if (tid == 0) sm.status &= ~(int)ST_DETAILS;
+        }
         if constexpr (WIDE) {
             if (d.collision)
                 collide_reconstructed();  // S1, eq. reconstructedCollision
@@ -1813,34 +1848,11 @@ struct Worker {
     }
 
     // ---- initial state -------------------------------------------------------
-    // full tree, populations at equilibrium of the conserved moments (staged m_cons)
-    __device__ __noinline__ void init_full(const double *mcons) {
-        clear_masks();
-        uint32_t *I = mask(M_I0);
-#pragma unroll 1
-        for (int w = tid; w < d.Wtot; w += TS) I[w] = w == 0 ? (Jmax >= 5 ? 0xFFFFFFFEu : (1u << (1 << Jmax)) - 2u) : FULL;
-        const int N = 1 << Jmax;
-#pragma unroll 1
-        for (int k = tid; k < N; k += TS) {
-            double mc[3], f[q];
-            T ft[q];
-            for (int j = 0; j < nf; ++j) mc[j] = mcons[(long long)j * N + k];
-            if constexpr (DQ)
-                dq_equilibrium_populations<q>(d, mc, f);
-            else
-                equilibrium_populations<NF>(d, mc, f);
-#pragma unroll
-            for (int h = 0; h < q; ++h) ft[h] = (T)f[h];
-            store_cell((uint32_t)(N + k), ft);
-        }
-        finish_init();
-    }
-
-    // the bit arrays but the current tree's (M_I0)
+    // KEEP and REF, and the tree buffer beside the current one
     __device__ __forceinline__ void clear_masks() {
 #pragma unroll 1
         for (int w = tid; w < d.Wtot; w += TS) {
-            mask(M_I1)[w] = 0u;
+            mask(sm.cur ^ 1)[w] = 0u;
             mask(M_KEEP)[w] = 0u;
             mask(M_REF)[w] = 0u;
         }
@@ -1848,6 +1860,8 @@ struct Worker {
 
     // arbitrary graded tree (one byte per cell) and values
     __device__ __noinline__ void init_state(const unsigned char *Rb, const double *vals) {
+        if (tid == 0) sm.cur = M_I0;
+        sync();
         clear_masks();
         uint32_t *I = mask(M_I0);
         const uint32_t off = 1u << Jmin;
@@ -1870,7 +1884,6 @@ struct Worker {
     }
 
     __device__ __noinline__ void finish_init() {
-        if (tid == 0) sm.cur = M_I0;
         if constexpr (SPM != 0) {
             // every word is a candidate of this first listing
             uint32_t *cw = cwl();
@@ -1948,13 +1961,7 @@ __device__ void load_instance(TeamSmem<T> &sm, const InstDesc &dg, int tid) {
 #endif
     }
     for (int l = tid; l <= MAXLEV; l += TS) {
-        // eps_l = 2^{l - Jmax} eps (Prop. ErrorControl), Harten level 2^{mu_bar + 1} eps_l
-        double el = ldexp(dg.eps, l - dg.Jmax);
-        double bl = ldexp(el, dg.mu_bar + 1);
-        sm.eps_l[l] = el;
-        sm.big_l[l] = bl;
-        sm.eps_f[l] = (float)el;
-        sm.big_f[l] = (float)bl;
+        sm.th.set(dg, l);
         sm.dx_l[l] = ldexp(dg.b - dg.a, -l);
     }
     for (int i = tid; i < NSEG * (MAXLEV + 2); i += TS) (&sm.seg[0][0])[i] = (&st.seg[0][0])[i];
@@ -1991,7 +1998,6 @@ template <typename T, int NF, int TS, bool WIDE, int SPM>
 __device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx, const LaunchArgs &a, int tid,
                              uint32_t *masks) {
     Worker<T, NF, TS, WIDE, SPM> w(sm, tab, bx, tid, masks);
-    if (a.phases & PH_INIT_FULL) w.init_full((const double *)a.aux0 + sm.d.m_off);
     if (a.phases & PH_INIT_STATE) w.init_state((const unsigned char *)a.aux0, (const double *)a.aux1);
 #pragma unroll 1
     for (int n = 0; n < a.nsteps; ++n) {
@@ -2002,8 +2008,9 @@ __device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &t
 
 // The bit arrays live in shared memory (smask, room for `cap` words) when the
 // instance fits: the current tree is copied in at the start and back at the
-// end; KEEP and REF are clear between two adaptations, and every adaptation
-// writes the other tree buffer.
+// end; KEEP and REF are clear between two adaptations (but for the decisions
+// that come with an initial state, ST_DETAILS), and every adaptation writes the
+// other tree buffer.
 template <typename T, int TS, bool WIDE, bool SCALAR, int SPM>
 __device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx, const LaunchArgs &a,
                          const InstDesc &dg, int tid, uint32_t *smask, int cap) {
@@ -2021,10 +2028,13 @@ __device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx
     if (local) {
         const uint32_t *gi = sm.d.masks + (long long)sm.cur * W;
         uint32_t *li = smask + sm.cur * W;
+        uint32_t *gk = sm.d.masks + (long long)M_KEEP * W, *gr = sm.d.masks + (long long)M_REF * W;
+        const bool first = (sm.status & ST_DETAILS) != 0;  // the initial state's decisions, taken once
         for (int g = tid; g < W; g += TS) {
             li[g] = gi[g];
-            smask[M_KEEP * W + g] = 0u;
-            smask[M_REF * W + g] = 0u;
+            smask[M_KEEP * W + g] = first ? gk[g] : 0u;
+            smask[M_REF * W + g] = first ? gr[g] : 0u;
+            if (first) gk[g] = gr[g] = 0u;
         }
         if constexpr (SPM != 0)
             for (int g = tid; g < OW; g += TS) smask[oo + g] = sm.d.masks[oo + g];
@@ -2047,7 +2057,7 @@ __device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx
         uint32_t *gi = sm.d.masks + (long long)sm.cur * W;
         const uint32_t *li = smask + sm.cur * W;
         for (int g = tid; g < W; g += TS) gi[g] = li[g];
-        if (a.phases & (PH_INIT_FULL | PH_INIT_STATE))  // clear there too, for a launch that keeps them there
+        if (a.phases & PH_INIT_STATE)  // clear there too, for a launch that keeps them there
             for (int g = tid; g < W; g += TS) {
                 sm.d.masks[(long long)M_KEEP * W + g] = 0u;
                 sm.d.masks[(long long)M_REF * W + g] = 0u;

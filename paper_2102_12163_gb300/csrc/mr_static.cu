@@ -208,16 +208,12 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     const long long sregion = smem_region_words(W, OW);
     a.smem_mask_words = sregion <= fit ? (int)sregion : 0;
     a.kind = d.gamma > 1 ? K_GENERAL : d.collision != 0 ? K_RECOLL : W >= CW_MIN_WORDS ? K_LARGE : K_FAST;
-    const int phases[2] = {PH_INIT_FULL, PH_ADAPT | PH_STEP};
-    const int steps[2] = {0, nsteps};
-    for (int i = 0; i < 2; ++i) {
-        if (i == 1 && nsteps == 0) continue;
-        a.phases = phases[i];
-        a.nsteps = steps[i];
-        a.aux0 = i == 0 ? (const void *)m_cons : nullptr;
-        if ((e = cudaMemsetAsync(a.queue, 0, sizeof(int), s)) != cudaSuccess)
-            return fail(MR_ERR_CUDA, "mr_run_static: queue reset failed (%lld)", (long long)e);
-        int rc = mrg_launch(fp32, block, 1, a, s, 0);
+    if (const int rc = mrg_init(fp32, a.descs, nullptr, init_chunks_of(d.Jmax), a.tables, m_cons, s))
+        return fail(MR_ERR_CUDA, "mr_run_static: kernel launch failed (%lld)", (long long)rc);
+    if (nsteps > 0) {
+        a.phases = PH_ADAPT | PH_STEP;
+        a.nsteps = nsteps;
+        const int rc = mrg_launch(fp32, block, 1, a, s, 0);
         if (rc) return fail(MR_ERR_CUDA, "mr_run_static: kernel launch failed (%lld)", (long long)rc);
     }
     if (const int rc = mrg_finest(fp32, mrg_variant(d.eq), d.Jmax, a.descs, a.tables, m_finest, s))

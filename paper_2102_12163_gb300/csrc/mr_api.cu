@@ -330,6 +330,16 @@ static void make_tables(Tables<double> &td, Tables<float> &tf) {
                 td.t1[dj][j] = td.cf[dj - 1][j];
                 td.t12[dj][j] = td.cf2[dj - 1][j];
             }
+        for (int k = 0; k < 2; ++k) {
+            // t (l0, l1, b + tt, b - tt), tt = c_1 (e - (l0 + l1) / 2): exact while the
+            // entries fit 53 bits
+            const double *t = k ? td.t12[dj] : td.t1[dj], D = -0.125 * (t[2] - t[3]);
+            double *w = k ? td.t42[dj] : td.t4[dj];
+            w[0] = t[0] - 0.5 * D;
+            w[1] = t[1] - 0.5 * D;
+            w[2] = t[2] + t[3];
+            w[3] = D;
+        }
         i128 nv[4] = {0, 0, 0, 0}, nu[2] = {0, 0}, nv2[4] = {0, 0, 0, 0}, nu2[2] = {0, 0};
         for (int r = 0; r < 4; ++r)
             for (int j = 0; j < 4; ++j) {
@@ -352,6 +362,8 @@ static void make_tables(Tables<double> &td, Tables<float> &tf) {
             tf.t1[dj][j] = (float)td.t1[dj][j];
             tf.cf2[dj][j] = (float)td.cf2[dj][j];
             tf.t12[dj][j] = (float)td.t12[dj][j];
+            tf.t4[dj][j] = (float)td.t4[dj][j];
+            tf.t42[dj][j] = (float)td.t42[dj][j];
         }
         for (int j = 0; j < 2; ++j) {
             tf.bf[dj][j] = (float)td.bf[dj][j];

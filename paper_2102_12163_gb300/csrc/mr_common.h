@@ -86,9 +86,9 @@ struct InstDesc {
     // the scheme constants rounded to float once, for the FP32 path
     float lam_f, eqp_f, s_f[3];
     float minv_f[5][5];
-    // correctly rounded reciprocal of lambda, for the FP64 division by lambda
-    // with one correction step (see the kernel's div_lam)
-    double rlam;
+    // 2 lambda and its correctly rounded reciprocal, for the FP64 division with
+    // one correction step (see the kernel's div_2lam)
+    double lam2, rlam2;
     // constant factors of the FP64 collision, rounded once exactly as the
     // per-cell expressions would round them: 1 - s[j]; Euler 1.5 - 0.5 gamma_gas,
     // gamma_gas - 1, 0.5 (1 - gamma_gas); shallow water 0.5 g
@@ -126,7 +126,8 @@ inline void fill_float_constants(InstDesc &h) {
     for (int j = 0; j < 3; ++j) h.s_f[j] = (float)h.s[j];
     for (int i = 0; i < 5; ++i)
         for (int j = 0; j < 5; ++j) h.minv_f[i][j] = (float)h.minv[i][j];
-    h.rlam = 1.0 / h.lam;  // IEEE division: correctly rounded
+    h.lam2 = 2.0 * h.lam;
+    h.rlam2 = 1.0 / h.lam2;  // IEEE division: correctly rounded
     for (int j = 0; j < 3; ++j) h.oms[j] = 1.0 - h.s[j];
     h.eu_a = 1.5 - 0.5 * h.eqp;
     h.eu_b = h.eqp - 1.0;
@@ -142,6 +143,9 @@ inline void fill_float_constants(InstDesc &h) {
 // The last finest cell uses the mirrored coefficients.
 //   cf2, t12, bf2  the same for the second finest cell from the edge (the
 //           populations with |v| = 2 lambda stream two cells per step)
+//   t4, t42  the weights t1 (t12) next to a finer neighbour with the leaf's
+//           predicted children expanded, on (2k-2, 2k-1) of the level below, the
+//           leaf k and k+1: the refined neighbour k-1 is the mean of the first two
 //   pc[g]   the prediction coefficients c_1..c_g of the stencil gamma = g
 //           (Section 3.1; gamma = 3 with c_3 = -5/1024)
 template <typename T>
@@ -152,6 +156,8 @@ struct Tables {
     T cf2[MAXDJ + 1][4];
     T t12[MAXDJ + 1][4];
     T bf2[MAXDJ + 1][2];
+    T t4[MAXDJ + 1][4];
+    T t42[MAXDJ + 1][4];
     T pc[4][3];
 };
 

@@ -242,20 +242,14 @@ __device__ __forceinline__ double scale2(double x, int k) {
 }
 __device__ __forceinline__ float scale2(float x, int k) { return x * ldexpf(1.0f, k); }
 
-// x / 2, bit for bit the product x * 0.5, on the integer units: an exponent
-// field e >= 2 loses one; for e <= 1 the magnitude bits are the value in units
-// of 2^-1074 (the implicit bit included), halved with ties to even (which also
-// carries into the smallest normal number); infinities and NaNs pass unchanged
+// x / 2, bit for bit the product x * 0.5, on the integer units where the
+// exponent field allows (a normal operand and result, four instructions; or
+// zero) and with the multiply otherwise
 __device__ __forceinline__ double half_f64(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned long long sign = b & 0x8000000000000000ull, mag = b ^ sign;
-    const unsigned e = (unsigned)(mag >> 52);
-    unsigned long long r;
-    if (e >= 2u)
-        r = e == 0x7FFu ? mag : mag - (1ull << 52);
-    else
-        r = (mag >> 1) + ((mag & 1ull) & ((mag >> 1) & 1ull));
-    return __longlong_as_double((long long)(sign | r));
+    const unsigned hi = (unsigned)__double2hiint(x);
+    if ((hi & 0x7FF00000u) - 0x00200000u < 0x7FD00000u) return __hiloint2double((int)(hi - 0x00100000u), __double2loint(x));
+    if (((hi << 1) | (unsigned)__double2loint(x)) == 0u) return x;
+    return __dmul_rn(x, 0.5);
 }
 template <typename T>
 __device__ __forceinline__ T half_of(T x) {
@@ -303,21 +297,30 @@ __device__ __forceinline__ void eq_consts(const InstDesc &d, T &a, T &b, T &c, T
     }
 }
 
-// x / lambda for a lambda that is no power of two, in FP64 bit for bit the
-// correctly rounded quotient without a division: q0 = RN(x r) with r = RN(1 / lambda) is
-// within one ulp of x / lambda, the residual x - q0 lambda is exact in one FMA,
-// and q0 + residual r rounded once is the correctly rounded quotient (P.
-// Markstein, IBM J. Res. Dev. 34(1), 1990).  Operands near the ends of the
-// exponent range, zeros and non-finite values take the division.
+// Quotients in FP64 from a reciprocal (P. Markstein, IBM J. Res. Dev. 34(1),
+// 1990): with r = RN(1 / y), q0 = RN(x r) is within one ulp of x / y, the
+// residual x - q0 y is exact in one FMA, and q0 + residual r rounded once is the
+// correctly rounded quotient, bit for bit the division.  Operands near the ends
+// of the exponent range and non-finite values take the division; a zero (a
+// state at rest has many) stays on the short path.
+__device__ __forceinline__ bool mid_range(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    return ((hi >> 20) & 0x7FFu) - 64u < 1920u || ((hi << 1) | (unsigned)__double2loint(x)) == 0u;
+}
+__device__ __forceinline__ double markstein(double x, double y, double r) {
+    const double q0 = __dmul_rn(x, r);
+    return __fma_rn(__fma_rn(-q0, y, x), r, q0);
+}
+// x / (2 lambda), half of what the collision adds to and takes from a moment,
+// for a lambda that is no power of two (halving is exact, so its halves are the
+// halves of the rounded quotient by lambda)
 template <typename T>
-__device__ __forceinline__ T div_lam(T x, const InstDesc &d) {
+__device__ __forceinline__ T div_2lam(T x, const InstDesc &d) {
     if constexpr (sizeof(T) == 8) {
-        const int e = (__double2hiint(x) >> 20) & 0x7FF;
-        if (e < 64 || e > 1983) return __ddiv_rn(x, d.lam);
-        const double q0 = __dmul_rn(x, d.rlam);
-        return __fma_rn(__fma_rn(-q0, d.lam, x), d.rlam, q0);
+        if (!mid_range(x)) return half_f64(__ddiv_rn(x, d.lam));
+        return markstein(x, d.lam2, d.rlam2);
     } else {
-        return __fdiv_rn(x, d.lam_f);  // FP32 divisions are cheap; the register budget is not
+        return 0.5f * __fdiv_rn(x, d.lam_f);  // FP32 divisions are cheap; the register budget is not
     }
 }
 
@@ -343,32 +346,57 @@ __device__ __forceinline__ void equilibria(const InstDesc &d, T eqp, const T *mc
         T gg = eqp;
         T u2 = A::mul(mc[1], mc[1]);
         meq[0] = mc[1];
+        if constexpr (sizeof(T) == 8) {
+            // the three quotients from one reciprocal: its square, refined once, is
+            // that of rho^2 (about 20 FP64 instructions instead of three divisions'
+            // 35; a lane pair of FP64 units makes them the cost of the collision)
+            const double em = A::mul(mc[2], mc[1]), u3 = A::mul(u2, mc[1]);
+            if (mc[0] != 0.0 && mid_range(mc[0]) && mid_range(u2) && mid_range(em) && mid_range(u3)) {
+                const double r = __drcp_rn(mc[0]), r2 = __dmul_rn(mc[0], mc[0]);
+                double q2 = __dmul_rn(r, r);
+                q2 = __fma_rn(__fma_rn(-r2, q2, 1.0), q2, q2);
+                meq[1] = A::add(A::mul(ca, markstein(u2, mc[0], r)), A::mul(cb, mc[2]));
+                meq[2] = A::add(A::mul(gg, markstein(em, mc[0], r)), A::mul(cc, markstein(u3, r2, q2)));
+                return;
+            }
+        }
         meq[1] = A::add(A::mul(ca, A::div(u2, mc[0])), A::mul(cb, mc[2]));
         meq[2] = A::add(A::mul(gg, A::div(A::mul(mc[2], mc[1]), mc[0])),
                         A::mul(cc, A::div(A::mul(u2, mc[1]), A::mul(mc[0], mc[0]))));
     }
 }
 
+// half of m* / lambda, an exact power-of-two scaling when lambda = 2^k (the same
+// value as the division)
+template <typename T>
+__device__ __forceinline__ T half_over_lam(T x, const InstDesc &d) {
+    return d.lam_log2 != NOT_POW2 ? scale2(x, -d.lam_log2 - 1) : div_2lam<T>(x, d);
+}
+// relaxed moment (1 - s) m + s m_eq of field i, m = lambda (f+ - f-); full
+// relaxation is m_eq itself (0 m + 1 m_eq), five FP64 operations fewer
+template <typename T>
+__device__ __forceinline__ T relaxed(const InstDesc &d, int i, T fp, T fm, T meq) {
+    using A = Ar<T>;
+    const T s = s_of<T>(d, i);
+    if constexpr (sizeof(T) == 8)
+        if (s == 1.0) return meq;
+    return A::add(A::mul(oms_of<T>(d, i), A::mul(lam_of<T>(d), A::sub(fp, fm))), A::mul(s, meq));
+}
+
 // leaves collision on the q populations of one cell: m = M f, relax, f* = M^-1 m*
 template <typename T, int NF>
 __device__ __forceinline__ void collide(const InstDesc &d, T *f) {
     using A = Ar<T>;
-    T mc[NF], mn[NF], meq[NF];
-    const T lam = lam_of<T>(d);
+    T mc[NF], meq[NF];
 #pragma unroll
-    for (int i = 0; i < NF; ++i) {
-        mc[i] = A::add(f[2 * i], f[2 * i + 1]);
-        mn[i] = A::mul(lam, A::sub(f[2 * i], f[2 * i + 1]));
-    }
+    for (int i = 0; i < NF; ++i) mc[i] = A::add(f[2 * i], f[2 * i + 1]);
     equilibria<T, NF>(d, eqp_of<T>(d), mc, meq);
 #pragma unroll
     for (int i = 0; i < NF; ++i) {
-        T s = s_of<T>(d, i);
-        T mstar = A::add(A::mul(oms_of<T>(d, i), mn[i]), A::mul(s, meq[i]));
-        // m*/lambda: an exact power-of-two scaling when lambda = 2^k (same value as the division)
-        T g = d.lam_log2 != NOT_POW2 ? scale2(mstar, -d.lam_log2) : div_lam<T>(mstar, d);
-        f[2 * i] = half_of<T>(A::add(mc[i], g));
-        f[2 * i + 1] = half_of<T>(A::sub(mc[i], g));
+        // f+- = (mc +- m* / lambda) / 2, the halves taken first (exact)
+        const T g = half_over_lam<T>(relaxed<T>(d, i, f[2 * i], f[2 * i + 1], meq[i]), d), m = half_of<T>(mc[i]);
+        f[2 * i] = A::add(m, g);
+        f[2 * i + 1] = A::sub(m, g);
     }
 }
 
@@ -380,9 +408,9 @@ __device__ __forceinline__ void equilibrium_populations(const InstDesc &d, const
     equilibria<double, NF>(d, d.eqp, mc, meq);
 #pragma unroll
     for (int i = 0; i < NF; ++i) {
-        const double g = d.lam_log2 != NOT_POW2 ? scale2(meq[i], -d.lam_log2) : div_lam<double>(meq[i], d);  // meq / lambda
-        f[2 * i] = half_f64(A::add(mc[i], g));
-        f[2 * i + 1] = half_f64(A::sub(mc[i], g));
+        const double g = half_over_lam<double>(meq[i], d), m = half_f64(mc[i]);
+        f[2 * i] = A::add(m, g);
+        f[2 * i + 1] = A::sub(m, g);
     }
 }
 
@@ -390,26 +418,52 @@ __device__ __forceinline__ void equilibrium_populations(const InstDesc &d, const
 // velocities v^h = lambda w^h, w = (0, 1, -1, 2, -2); moments m^i = sum_h (v^h)^i f^h
 __device__ __forceinline__ int dq_w(int h) { return h == 0 ? 0 : (h & 1) ? (h + 1) / 2 : -(h / 2); }
 
+// moments of the velocity set through the even and odd parts of its two velocity
+// pairs: m^i = lambda^i (p1 + 2^i p2), p the sums (i even) or differences (i odd)
+template <typename T, int Q>
+__device__ __forceinline__ void dq_moments(T lam, const T *f, T *m) {
+    const T s1 = f[1] + f[2], d1 = f[1] - f[2];
+    if constexpr (Q == 3) {
+        m[0] = f[0] + s1;
+        m[1] = lam * d1;
+        m[2] = (lam * lam) * s1;
+    } else {
+        const T s2 = f[3] + f[4], d2 = f[3] - f[4], l2 = lam * lam;
+        m[0] = f[0] + (s1 + s2);
+        m[1] = lam * (d1 + T(2) * d2);
+        m[2] = l2 * (s1 + T(4) * s2);
+        m[3] = (l2 * lam) * (d1 + T(8) * d2);
+        m[4] = (l2 * l2) * (s1 + T(16) * s2);
+    }
+}
+// f + M^{-1} dm for dm with zero conserved rows.  M^{-1} carries the same mirror
+// symmetry: the populations +-w get the even moments' part alike and the odd
+// moment's part with opposite signs.
+template <typename T, int Q>
+__device__ __forceinline__ void dq_add(const InstDesc &d, const T *dm, T *f) {
+    if constexpr (Q == 3) {
+        f[0] = f[0] + minv_of<T>(d, 0, 2) * dm[2];
+        const T a = minv_of<T>(d, 1, 2) * dm[2];
+        f[1] = f[1] + a;
+        f[2] = f[2] + a;
+    } else {
+        f[0] = f[0] + (minv_of<T>(d, 0, 2) * dm[2] + minv_of<T>(d, 0, 4) * dm[4]);
+#pragma unroll
+        for (int h = 1; h < 5; h += 2) {
+            const T a = minv_of<T>(d, h, 2) * dm[2] + minv_of<T>(d, h, 4) * dm[4], b = minv_of<T>(d, h, 3) * dm[3];
+            f[h] = f[h] + (a + b);
+            f[h + 1] = f[h + 1] + (a - b);
+        }
+    }
+}
 // collision: the relaxed moments i >= 2 move to (1 - s^i) m^i + s^i m^{i,eq}, with
 // m^{2,eq} = (hu)^2 / h + g h^2 / 2, m^{3,eq} = lambda^2 hu, m^{4,eq} = lambda^2
 // m^{2,eq}; f* = f + M^{-1} (m* - m) (the conserved rows of m* - m are zero)
 template <typename T, int Q>
 __device__ __forceinline__ void dq_collide(const InstDesc &d, T *f) {
     const T lam = lam_of<T>(d);
-    T m[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) m[i] = T(0);
-#pragma unroll
-    for (int h = 0; h < Q; ++h) {
-        const T v = (T)dq_w(h) * lam;
-        T x = f[h];
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            m[i] = m[i] + x;
-            x = x * v;
-        }
-    }
-    T meq[Q];
+    T m[Q], meq[Q], dm[Q];
+    dq_moments<T, Q>(lam, f, m);
     T ca, cb, cc, g2;
     eq_consts<T>(d, ca, cb, cc, g2);
     meq[2] = (m[1] * m[1]) / m[0] + g2 * (m[0] * m[0]);
@@ -417,16 +471,9 @@ __device__ __forceinline__ void dq_collide(const InstDesc &d, T *f) {
         meq[3] = (lam * lam) * m[1];
         meq[4] = (lam * lam) * meq[2];
     }
-    T dm[Q];
 #pragma unroll
     for (int i = 2; i < Q; ++i) dm[i] = s_of<T>(d, i - 2) * (meq[i] - m[i]);
-#pragma unroll
-    for (int h = 0; h < Q; ++h) {
-        T acc = T(0);
-#pragma unroll
-        for (int i = 2; i < Q; ++i) acc = acc + minv_of<T>(d, h, i) * dm[i];
-        f[h] = f[h] + acc;
-    }
+    dq_add<T, Q>(d, dm, f);
 }
 
 // populations at equilibrium of (h, hu), in FP64: f = M^{-1} (h, hu, m^{2,eq}, ...)
@@ -862,41 +909,19 @@ struct Worker {
 #pragma unroll
             for (int r = 0; r < NR; ++r) mavg[r] = Phi[r * stride + i];
             if constexpr (DQ) {
-                const T lam = lam_of<T>(d);
-                T m[q];
-#pragma unroll
-                for (int r = 0; r < q; ++r) m[r] = T(0);
-#pragma unroll
-                for (int h = 0; h < q; ++h) {
-                    const T v = (T)dq_w(h) * lam;
-                    T x = f[h];
-#pragma unroll
-                    for (int r = 0; r < q; ++r) {
-                        m[r] = m[r] + x;
-                        x = x * v;
-                    }
-                }
-                T dm[q];
+                T m[q], dm[q];
+                dq_moments<T, q>(lam_of<T>(d), f, m);
 #pragma unroll
                 for (int r = 2; r < q; ++r) dm[r] = s_of<T>(d, r - 2) * (mavg[r - 2] - m[r]);
-#pragma unroll
-                for (int h = 0; h < q; ++h) {
-                    T a = T(0);
-#pragma unroll
-                    for (int r = 2; r < q; ++r) a = a + minv_of<T>(d, h, r) * dm[r];
-                    f[h] = f[h] + a;
-                }
+                dq_add<T, q>(d, dm, f);
             } else {
                 using A = Ar<T>;
-                const T lam = lam_of<T>(d);
 #pragma unroll
                 for (int j = 0; j < NF; ++j) {
-                    const T mc = A::add(f[2 * j], f[2 * j + 1]), mn = A::mul(lam, A::sub(f[2 * j], f[2 * j + 1]));
-                    const T sj = s_of<T>(d, j);
-                    const T mstar = A::add(A::mul(oms_of<T>(d, j), mn), A::mul(sj, mavg[j]));
-                    const T g = d.lam_log2 != NOT_POW2 ? scale2(mstar, -d.lam_log2) : div_lam<T>(mstar, d);
-                    f[2 * j] = half_of<T>(A::add(mc, g));
-                    f[2 * j + 1] = half_of<T>(A::sub(mc, g));
+                    const T m = half_of<T>(A::add(f[2 * j], f[2 * j + 1]));
+                    const T g = half_over_lam<T>(relaxed<T>(d, j, f[2 * j], f[2 * j + 1], mavg[j]), d);
+                    f[2 * j] = A::add(m, g);
+                    f[2 * j + 1] = A::sub(m, g);
                 }
             }
             store_cell(hc, f);
@@ -1443,12 +1468,21 @@ struct Worker {
         }
     }
 
+    // weights next to a finer neighbour.  FP64: t4, on the two children of the
+    // neighbour, the leaf and its other neighbour (the leaf's predicted children
+    // and the projection of the refined neighbour folded into the weights: four
+    // FP64 operations instead of eight).  FP32: t1, on the neighbour's children and
+    // the leaf's own predicted ones (the operations are cheap there).
+    // sec 1: those of the second cell from the edge.
+    __device__ __forceinline__ const T *finer_weights(int dj, int sec = 0) const {
+        if constexpr (sizeof(T) == 8) return sec ? tab.t42[dj] : tab.t4[dj];
+        return sec ? tab.t12[dj] : tab.t1[dj];
+    }
     // S4: first / last finest-cell values of every leaf -> Phi, from the
     // per-level-gap tables.  One sum of four products for both stencils, so that
     // a warp whose leaves mix them evaluates it once: next to a finer neighbour
-    // the leaf's own children (predicted) enter with the weights t1, else the
-    // cells of the leaf's level with the weights cf; the mirrored sum for the
-    // last value.
+    // the finer weights, else the cells of the leaf's level with the weights cf;
+    // the mirrored sum for the last value.
     __device__ void reconstruct_edges() {
         const uint32_t *I = mask(sm.cur);
         const uint32_t *leaves = list(L_LEAF);
@@ -1481,7 +1515,7 @@ struct Worker {
             const T *l0 = fin_l ? cell(2u * hl) : cell(nb(h, -2, lo)), *l1 = fin_l ? cell(2u * hl + 1u) : cell(hl);
             const T *r0 = fin_r ? cell(2u * hr) : cell(hr), *r1 = fin_r ? cell(2u * hr + 1u) : cell(nb(h, 2, lo));
             const T *vm1 = cell(hl), *v0 = cell(h), *vp1 = cell(hr);
-            const T *wl = fin_l ? tab.t1[dj] : tab.cf[dj], *wr = fin_r ? tab.t1[dj] : tab.cf[dj], *bf = tab.bf[dj];
+            const T *wl = fin_l ? finer_weights(dj) : tab.cf[dj], *wr = fin_r ? finer_weights(dj) : tab.cf[dj], *bf = tab.bf[dj];
             const T wm[4] = {wr[3], wr[2], wr[1], wr[0]};
 #pragma unroll
             for (int j = 0; j < NF; ++j) {
@@ -1489,7 +1523,7 @@ struct Worker {
                     const int c = 2 * j;
                     const T a = vm1[c], b = v0[c], e = vp1[c];
                     T x0 = a, x1 = b;
-                    if (fin_r) {
+                    if (sizeof(T) == 4 && fin_r) {
                         const T tt = T(C1) * (e - a);
                         x0 = b + tt;
                         x1 = b - tt;
@@ -1501,7 +1535,7 @@ struct Worker {
                     const int c = 2 * j + 1;
                     const T a = vm1[c], b = v0[c], e = vp1[c];
                     T x2 = b, x3 = e;
-                    if (fin_l) {
+                    if (sizeof(T) == 4 && fin_l) {
                         const T tt = T(C1) * (e - a);
                         x2 = b + tt;
                         x3 = b - tt;
@@ -1625,36 +1659,41 @@ struct Worker {
                 }
                 const T vm1 = vm1p[h], v0 = v0p[h], vp1 = vp1p[h];
                 // cell `sec` (0: first / last, 1: second from that edge) next to the left or right
-                // edge: one sum of four products for both stencils (as in reconstruct_edges), next
-                // to a finer neighbour with the leaf's own (predicted) children and the weights t1
+                // edge: one sum of four products for both stencils (as in reconstruct_edges)
                 auto from_left = [&](int sec) -> T {
-                    const T *bf = sec ? tab.bf2[dj] : tab.bf[dj], *t1 = sec ? tab.t12[dj] : tab.t1[dj],
-                            *cf = sec ? tab.cf2[dj] : tab.cf[dj];
+                    const T *bf = sec ? tab.bf2[dj] : tab.bf[dj], *cf = sec ? tab.cf2[dj] : tab.cf[dj];
                     if (at_left) return bf[0] * v0 + bf[1] * vp1;
                     T x0, x1, x2, x3;
                     if (fin_l) {
-                        const T tt = T(C1) * (vp1 - vm1);
                         x0 = clp[h];
                         x1 = clp[q + h];
-                        x2 = v0 + tt;
-                        x3 = v0 - tt;
+                        x2 = v0;
+                        x3 = vp1;
+                        if constexpr (sizeof(T) == 4) {
+                            const T tt = T(C1) * (vp1 - vm1);
+                            x2 = v0 + tt;
+                            x3 = v0 - tt;
+                        }
                     } else {
                         x0 = vm2p[h];
                         x1 = vm1;
                         x2 = v0;
                         x3 = vp1;
                     }
-                    return dot4(fin_l ? t1 : cf, x0, x1, x2, x3);
+                    return dot4(fin_l ? finer_weights(dj, sec) : cf, x0, x1, x2, x3);
                 };
                 auto from_right = [&](int sec) -> T {
-                    const T *bf = sec ? tab.bf2[dj] : tab.bf[dj], *t1 = sec ? tab.t12[dj] : tab.t1[dj],
-                            *cf = sec ? tab.cf2[dj] : tab.cf[dj];
+                    const T *bf = sec ? tab.bf2[dj] : tab.bf[dj], *cf = sec ? tab.cf2[dj] : tab.cf[dj];
                     if (at_right) return bf[0] * v0 + bf[1] * vm1;
                     T x0, x1, x2, x3;
                     if (fin_r) {
-                        const T tt = T(C1) * (vp1 - vm1);
-                        x0 = v0 + tt;
-                        x1 = v0 - tt;
+                        x0 = vm1;
+                        x1 = v0;
+                        if constexpr (sizeof(T) == 4) {
+                            const T tt = T(C1) * (vp1 - vm1);
+                            x0 = v0 + tt;
+                            x1 = v0 - tt;
+                        }
                         x2 = crp[h];
                         x3 = crp[q + h];
                     } else {
@@ -1663,7 +1702,7 @@ struct Worker {
                         x2 = vp1;
                         x3 = vp2p[h];
                     }
-                    const T *wt = fin_r ? t1 : cf;
+                    const T *wt = fin_r ? finer_weights(dj, sec) : cf;
                     const T wm[4] = {wt[3], wt[2], wt[1], wt[0]};
                     return dot4(wm, x0, x1, x2, x3);
                 };

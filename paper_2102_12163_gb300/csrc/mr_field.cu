@@ -152,7 +152,6 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
         for (int j = 0; j < q; ++j) {
             const T x = (T)f[j];
             a[t * q + j] = x;
-            V[(size_t)(N + k) * q + j] = x;
             if constexpr (DQ) {
                 m0 += (double)x;
                 m1 += (dq_w(j) * d.lam) * (double)x;
@@ -167,6 +166,12 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
         }
         leaves[k] = (uint32_t)(N + k);
     }
+    // values to memory from the shared copy, whose layout is theirs: consecutive
+    // threads write consecutive bytes
+    auto put = [&](const T *from, uint32_t h, int cells) {
+        T *to = V + (size_t)h * q;
+        for (int i = tid; i < cells * q; i += 256) to[i] = from[i];
+    };
     // the run's totals, into the interface array (free until the first step)
 #pragma unroll
     for (int j = 0; j < nf; ++j) {
@@ -174,6 +179,7 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
         if (lane == 0) red[j][warp] = m[j];
     }
     __syncthreads();
+    put(a, (uint32_t)(N + c0), ch);
     if (tid < nf) {
         double x = 0.0;
         for (int w = 0; w < 8; ++w) x += red[tid][w];
@@ -187,11 +193,11 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
             for (int j = 0; j < q; ++j) {
                 const T x = half_of<T>(a[2 * t * q + j] + a[(2 * t + 1) * q + j]);
                 b[t * q + j] = x;
-                V[(size_t)(h0 + t) * q + j] = x;
             }
             inner[h0 + t] = h0 + t;
         }
         __syncthreads();
+        put(b, h0, n);
         T *x = a;
         a = b;
         b = x;

@@ -191,7 +191,7 @@ struct TeamSmem {
     Thresholds th;
     double dx_l[MAXLEV + 1];  // cell size per level
     double mass[3];
-    double audit;
+    double audit[3];  // per field
     unsigned long long updates, steps, passes;
     int cur, nleaf, status, near_ties, ncw;
     uint32_t deplev[2];  // levels holding transfer (0) / ghost (1) pairs that wait on the same list
@@ -738,35 +738,6 @@ struct Worker {
         }
     }
 
-    // The team's sum of x[j], in thread 0 (one barrier).  GB300's FP64 units
-    // take a warp-wide instruction whole whatever its active lanes, so the
-    // additions are kept off most warps: a few shuffle rounds in each warp leave
-    // 64 partial sums per field (groups of TS / 64 lanes) in shared memory, and
-    // warp 0 folds them (two per lane, then a shuffle tree).  A fixed order:
-    // deterministic.
-    __device__ __forceinline__ void team_sum(double (&x)[3]) {
-        constexpr int G = TS / 64;  // lanes per partial sum: 1, 2, 4, 8 or 16
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-            if (j < nf)
-#pragma unroll
-                for (int o = G / 2; o > 0; o >>= 1) x[j] += __shfl_down_sync(FULL, x[j], o);
-        if ((tid & (G - 1)) == 0)
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-                if (j < nf) bx.red[j][tid / G] = x[j];
-        sync();
-        if (tid < 32)
-#pragma unroll
-            for (int j = 0; j < 3; ++j)
-                if (j < nf) {
-                    double v = bx.red[j][tid] + bx.red[j][tid + 32];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
-                    x[j] = v;
-                }
-    }
-
     // float-float accumulation (hi + lo, error-free transformation TwoSum of
     // Knuth): the FP32 path keeps its mass audit off the FP64 pipe
     static __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
@@ -780,32 +751,64 @@ struct Worker {
         hi = s;
         lo = lo + (xl + e);
     }
-    // team sums of nf float-float pairs, as doubles valid in thread 0 (one barrier)
-    __device__ __forceinline__ void team_sum_ff(float (&hi)[3], float (&lo)[3], double (&out)[3]) {
+    // Partial sums of the team, field by field, in shared memory (one barrier),
+    // and the sum of field j of them by one warp: the warps TS / 32 - 1 - j fold one
+    // field each, valid in their lane 0, while the others go on.  GB300's FP64
+    // units take a warp-wide instruction whole whatever its active lanes, so
+    // additions are kept off most warps: two shuffle rounds or so leave 64
+    // partials a field (groups of TS / 64 lanes), and warps without a leaf (the
+    // first n threads have one) only write their zeros.  A fixed order:
+    // deterministic.
+    __device__ __forceinline__ void team_partials(double (&x)[3], int n) {
+        constexpr int G = TS / 64;  // lanes per partial sum: 2, 4, 8 or 16
+        if ((tid & ~31) < n)
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-            if (j < nf)
+            for (int j = 0; j < nf; ++j)
+#pragma unroll
+                for (int o = G / 2; o > 0; o >>= 1) x[j] += __shfl_down_sync(FULL, x[j], o);
+        if ((tid & (G - 1)) == 0)
+#pragma unroll
+            for (int j = 0; j < nf; ++j) bx.red[j][tid / G] = x[j];
+        sync();
+    }
+    __device__ __forceinline__ double team_fold(int j) const {
+        const int lane = tid & 31;
+        double v = bx.red[j][lane] + bx.red[j][lane + 32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
+        return v;
+    }
+    // the same in float-float: one partial per warp
+    __device__ __forceinline__ void team_partials_ff(float (&hi)[3], float (&lo)[3], int n) {
+        float2 *red = reinterpret_cast<float2 *>(&bx.red[0][0]);
+        if ((tid & ~31) < n)
+#pragma unroll
+            for (int j = 0; j < nf; ++j)
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
                     const float h2 = __shfl_down_sync(FULL, hi[j], o), l2 = __shfl_down_sync(FULL, lo[j], o);
                     ff_add(hi[j], lo[j], h2, l2);
                 }
-        float2 *red = reinterpret_cast<float2 *>(&bx.red[0][0]);
         if ((tid & 31) == 0)
 #pragma unroll
-            for (int j = 0; j < 3; ++j)
-                if (j < nf) red[j * 32 + (tid >> 5)] = make_float2(hi[j], lo[j]);
+            for (int j = 0; j < nf; ++j) red[j * 32 + (tid >> 5)] = make_float2(hi[j], lo[j]);
         sync();
-        // only thread 0 holds the sums: the other threads keep off the FP64 pipe
-        if (tid == 0)
+    }
+    __device__ __forceinline__ double team_fold_ff(int j) const {
+        const float2 *red = reinterpret_cast<const float2 *>(&bx.red[0][0]);
+        const int lane = tid & 31;
+        float2 v = lane < TS / 32 ? red[j * 32 + lane] : make_float2(0.0f, 0.0f);
 #pragma unroll
-            for (int j = 0; j < 3; ++j)
-                if (j < nf) {
-                    float h = 0.0f, l = 0.0f;
-#pragma unroll 1
-                    for (int w = 0; w < TS / 32; ++w) ff_add(h, l, red[j * 32 + w].x, red[j * 32 + w].y);
-                    out[j] = (double)h + (double)l;
-                }
+        for (int o = TS / 64; o > 0; o >>= 1) {
+            const float h2 = __shfl_down_sync(FULL, v.x, o), l2 = __shfl_down_sync(FULL, v.y, o);
+            ff_add(v.x, v.y, h2, l2);
+        }
+        return (double)v.x + (double)v.y;
+    }
+    // field that this thread's warp folds, or -1
+    __device__ __forceinline__ int fold_field() const {
+        const int j = TS / 32 - 1 - (tid >> 5);
+        return j < nf ? j : -1;
     }
 
     // ---- S1: leaves collision (eq. LeavesCollision) ---------------------------
@@ -929,36 +932,55 @@ struct Worker {
         sync();
     }
 
-    // ---- A1 / S2: projection sweep, fine to coarse (Def. Projection operator) -
-    // projection of cell h: the mean of its two children, 2q adjacent values
-    __device__ __forceinline__ void project_cell(uint32_t h) const {
-        T a[q], b[q];
-        load_cell(2u * h, a);
-        load_cell(2u * h + 1u, b);
-#pragma unroll
-        for (int j = 0; j < q; ++j) a[j] = half_of<T>(a[j] + b[j]);
-        store_cell(h, a);
+    // ---- S2: projection sweep, fine to coarse (Def. Projection operator) -------
+    // population j of cell h: the mean of its two children's
+    __device__ __forceinline__ void project_pop(uint32_t h, int j) const {
+        T *p = V + (h * (uint32_t)q + (uint32_t)j);
+        const T *c = V + (2u * h * (uint32_t)q + (uint32_t)j);
+        *p = half_of<T>(c[0] + c[q]);
     }
-    // one level per barrier; the levels of at most 32 cells by one warp, cell by
-    // lane, without block barriers.  Ends with a barrier.
+    // One level per barrier; the levels of at most 32 cells by one warp, without
+    // block barriers.  Ends with a barrier.  A thread takes one population of a
+    // cell: a level holds some ten cells, and an FP64 instruction costs its warp's
+    // quarter of the SM 64 cycles whatever its active lanes, so q cells x
+    // populations side by side take one addition's time where a loop over the
+    // populations took q.  The next level's cell is fetched before the barrier.
     __device__ void upsweep() {
         const uint32_t *li = list(L_INT);
         const int ls = Jmin > 6 ? Jmin : 6;
+        constexpr int CPB = TS / q;  // cells of a block pass
+        const int c = tid / q, j = tid - c * q;
+        int l = Jmax - 1;
+        if (l >= ls) {
+            int b = sm.seg[L_INT][l], e = sm.seg[L_INT][l + 1];
+            uint32_t h = c < CPB && b + c < e ? li[b + c] : 0u;
 #pragma unroll 1
-        for (int l = Jmax - 1; l >= ls; --l) {
-            const int b = sm.seg[L_INT][l], e = sm.seg[L_INT][l + 1];
-            if (b == e) continue;
+            for (;;) {
+                const int eb = b;
+                if (h) project_pop(h, j);
 #pragma unroll 1
-            for (int i = b + tid; i < e; i += TS) project_cell(li[i]);
-            sync();
+                for (int i = b + c + CPB; c < CPB && i < e; i += CPB) project_pop(li[i], j);
+                const bool some = b < e;
+                --l;
+                if (l >= ls) {
+                    e = eb;
+                    b = sm.seg[L_INT][l];
+                    h = c < CPB && b + c < e ? li[b + c] : 0u;
+                }
+                if (some) sync();
+                if (l < ls) break;
+            }
         }
         if (Jmin < 6) {
             if (tid < 32) {
                 const uint32_t *I = mask(sm.cur);
 #pragma unroll 1
-                for (int l = Jmax - 1 < 5 ? Jmax - 1 : 5; l >= Jmin; --l) {
-                    const uint32_t h = (1u << l) + tid;
-                    if (tid < (1 << l) && bit_of(I, h)) project_cell(h);
+                for (l = Jmax - 1 < 5 ? Jmax - 1 : 5; l >= Jmin; --l) {
+#pragma unroll 1
+                    for (int i = tid; i < (q << l); i += 32) {
+                        const uint32_t k = (uint32_t)i / (uint32_t)q, h = (1u << l) + k;
+                        if (bit_of(I, h)) project_pop(h, i - (int)k * q);
+                    }
                     __syncwarp();
                 }
             }
@@ -1764,33 +1786,7 @@ struct Worker {
         }
         if (bad) atomicOr(&sm.status, (int)ST_NONFINITE);
         project_by_flux_pass();  // A1 of the next adaptation, same pass
-        sum_audit(macc, fhi, flo);
-        if (tid == 0) {
-            // copy boundary: what leaves through x = a and x = b, sum over the
-            // populations of sigma 2^-Jmax-weighted telescoped stream terms
-            double flux[2] = {0.0, 0.0};
-            if (bc == 1) {
-                const double dxJ = sm.dx_l[Jmax];
-                for (int h = 1; h < q; ++h) {
-                    const int w = dq_w(h), a = w < 0 ? -w : w;
-                    double t = 0.0;
-                    for (int dl = 1; dl <= a; ++dl) {
-                        const int eta = w > 0 ? -dl : dl - 1;
-                        t += (double)phi(finest_at(eta))[h] - (double)phi(finest_at((1 << Jmax) + eta))[h];
-                    }
-                    t *= (w > 0 ? dxJ : -dxJ);
-                    flux[0] += t;
-                    flux[1] += (w * d.lam) * t;
-                }
-            }
-            for (int j = 0; j < 2; ++j) {
-                const double res = fabs(macc[j] - sm.mass[j] - flux[j]);
-                sm.audit = fmax(sm.audit, res);
-                sm.mass[j] = macc[j];
-            }
-            sm.steps += 1ULL;
-        }
-        sync();
+        finish_audit(macc, fhi, flo, nl);
     }
 
     // the audit's partial sums of one leaf: dx_l m_j in FP64, or, in the FP32
@@ -1801,14 +1797,13 @@ struct Worker {
         if constexpr (sizeof(T) == 8) {
             const double dx = sm.dx_l[l];
             if constexpr (DQ) {
-                double m0 = 0.0, m1 = 0.0;
-#pragma unroll
-                for (int c = 0; c < q; ++c) {
-                    m0 += (double)f[c];
-                    m1 += (dq_w(c) * d.lam) * (double)f[c];
+                double m0 = f[0] + (f[1] + f[2]), m1 = f[1] - f[2];
+                if constexpr (q == 5) {
+                    m0 += f[3] + f[4];
+                    m1 += 2.0 * (f[3] - f[4]);
                 }
                 macc[0] += dx * m0;
-                macc[1] += dx * m1;
+                macc[1] += dx * m1;  // times lambda at the end
             } else {
 #pragma unroll
                 for (int j = 0; j < nf; ++j) macc[j] += dx * ((double)f[2 * j] + (double)f[2 * j + 1]);
@@ -1834,18 +1829,50 @@ struct Worker {
             }
         }
     }
-    // the audit's totals, in thread 0 (one barrier)
-    __device__ __forceinline__ void sum_audit(double (&macc)[3], float (&fhi)[3], float (&flo)[3]) {
-        if constexpr (sizeof(T) == 8) {
-            team_sum(macc);
-        } else {
-            team_sum_ff(fhi, flo, macc);
-            if (tid == 0) {
-#pragma unroll
-                for (int j = 0; j < nf; ++j) macc[j] *= d.b - d.a;
-                if constexpr (DQ) macc[1] *= d.lam;
+    // End of a step: the totals of the conserved moments over the n leaves, and
+    // the residual of their change against what crossed a copy boundary, one
+    // field to a warp.  One barrier, after which the stream's results are there;
+    // nothing before the next step's end reads what the folding warps write but
+    // by the thread that wrote it (or after further barriers).
+    __device__ __forceinline__ void finish_audit(double (&macc)[3], float (&fhi)[3], float (&flo)[3], int n) {
+        if constexpr (sizeof(T) == 8)
+            team_partials(macc, n);
+        else
+            team_partials_ff(fhi, flo, n);
+        const int j = fold_field();
+        if (j < 0) return;
+        double total;
+        if constexpr (sizeof(T) == 8)
+            total = team_fold(j);
+        else
+            total = team_fold_ff(j);
+        if ((tid & 31) != 0) return;
+        if constexpr (sizeof(T) == 4) total *= d.b - d.a;
+        double flux = 0.0;
+        if constexpr (DQ) {
+            // copy boundary: what leaves through x = a and x = b, sum over the
+            // populations of sigma 2^-Jmax-weighted telescoped stream terms
+            if (j == 1) total *= d.lam;
+            if (bc == 1) {
+                const double dxJ = sm.dx_l[Jmax];
+                for (int h = 1; h < q; ++h) {
+                    const int w = dq_w(h), a = w < 0 ? -w : w;
+                    double t = 0.0;
+                    for (int dl = 1; dl <= a; ++dl) {
+                        const int eta = w > 0 ? -dl : dl - 1;
+                        t += (double)phi(finest_at(eta))[h] - (double)phi(finest_at((1 << Jmax) + eta))[h];
+                    }
+                    t *= (w > 0 ? dxJ : -dxJ);
+                    flux += j == 0 ? t : (w * d.lam) * t;
+                }
             }
+        } else if (bc == 1) {
+            const T *p0 = phi(0u), *pN = phi(1u << Jmax);
+            flux = sm.dx_l[Jmax] * (((double)p0[2 * j] - (double)pN[2 * j]) - ((double)p0[2 * j + 1] - (double)pN[2 * j + 1]));
         }
+        sm.audit[j] = fmax(sm.audit[j], fabs(total - sm.mass[j] - flux));
+        sm.mass[j] = total;
+        if (j == 0) sm.steps += 1ULL;
     }
 
     // S5: f^{n+1} = f* + sigma 2^-dj (Phi[first] - Phi[next]); mass audit
@@ -1868,22 +1895,7 @@ struct Worker {
         }
         if (bad) atomicOr(&sm.status, (int)ST_NONFINITE);
         project_by_flux_pass();  // A1 of the next adaptation, same pass
-        sum_audit(macc, fhi, flo);
-        if (tid == 0) {
-            const double dxJ = sm.dx_l[Jmax];
-            for (int j = 0; j < nf; ++j) {
-                double flux = 0.0;
-                if (bc == 1) {
-                    const T *p0 = phi(0u), *pN = phi(1u << Jmax);
-                    flux = dxJ * (((double)p0[2 * j] - (double)pN[2 * j]) - ((double)p0[2 * j + 1] - (double)pN[2 * j + 1]));
-                }
-                const double res = fabs(macc[j] - sm.mass[j] - flux);
-                sm.audit = fmax(sm.audit, res);
-                sm.mass[j] = macc[j];
-            }
-            sm.steps += 1ULL;
-        }
-        sync();
+        finish_audit(macc, fhi, flo, nl);
     }
 
     // ---- initial state -------------------------------------------------------
@@ -1960,15 +1972,20 @@ struct Worker {
                 for (int j = 0; j < nf; ++j) macc[j] += dx * ((double)f[2 * j] + (double)f[2 * j + 1]);
             }
         }
-        team_sum(macc);
+        team_partials(macc, nl);
+        if (const int j = fold_field(); j >= 0) {
+            const double total = team_fold(j);
+            if ((tid & 31) == 0) {
+                sm.mass[j] = total;
+                sm.audit[j] = 0.0;
+            }
+        }
         if (tid == 0) {
-            for (int j = 0; j < nf; ++j) sm.mass[j] = macc[j];
-            sm.audit = 0.0;
             sm.status = 0;
             sm.near_ties = 0;
             sm.updates = 0ULL;
-            sm.steps = 0ULL;
         }
+        if (tid == TS - 32) sm.steps = 0ULL;  // the thread that counts them
         if (tid == TS - 1) sm.passes = 0ULL;  // the thread that counts the barriers
         sync();
     }
@@ -1992,8 +2009,10 @@ __device__ void load_instance(TeamSmem<T> &sm, const InstDesc &dg, int tid) {
         sm.updates = st.updates;
         sm.steps = st.steps;
         sm.passes = st.passes;
-        sm.audit = st.audit;
-        for (int j = 0; j < 3; ++j) sm.mass[j] = st.mass[j];
+        for (int j = 0; j < 3; ++j) {
+            sm.mass[j] = st.mass[j];
+            sm.audit[j] = st.audit;
+        }
 #ifdef MRG_PHASE_TIMERS
         for (int p = 0; p < NPHASE; ++p) sm.ptime[p] = st.ptime[p];
         sm.tlast = clock64();
@@ -2022,7 +2041,7 @@ __device__ void store_instance(TeamSmem<T> &sm, int tid) {
         st.updates = sm.updates;
         st.steps = sm.steps;
         st.passes = sm.passes;
-        st.audit = sm.audit;
+        st.audit = fmax(sm.audit[0], fmax(sm.audit[1], sm.audit[2]));
         for (int j = 0; j < 3; ++j) st.mass[j] = sm.mass[j];
 #ifdef MRG_PHASE_TIMERS
         for (int p = 0; p < NPHASE; ++p) st.ptime[p] = sm.ptime[p];

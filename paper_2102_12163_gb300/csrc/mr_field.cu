@@ -127,6 +127,15 @@ __global__ void __launch_bounds__(256) mr_finest(const InstDesc *desc, const Tab
 // written and read per finest cell.  One block per instance took 2.6 ms for the
 // batch of 4096 (FP64) and 11 ms for a lone Euler instance of Jmax = 18 (FP32),
 // and the first adaptation 0.9 ms more for the latter.
+// (x + y) / 2; of two equal values below half the largest double the value
+// itself, without FP64 operations
+__device__ __forceinline__ double mean_of(double x, double y) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    if (__double_as_longlong(x) == __double_as_longlong(y) && (hi & 0x7FF00000u) < 0x7FE00000u) return x;
+    return half_f64(x + y);
+}
+__device__ __forceinline__ float mean_of(float x, float y) { return half_of<float>(x + y); }
+
 template <typename T, int NF>
 __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const double *mcons, unsigned char *smem) {
     constexpr bool DQ = NF >= 4;
@@ -135,22 +144,60 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
     const int N = 1 << Jmax, ch = min(INIT_CELLS, N), nch = init_chunks_of(Jmax), c0 = chunk * ch;
     T *a = (T *)smem, *b = a + INIT_CELLS * q;
     double(*red)[8] = (double(*)[8])(smem + sizeof(T) * q * (INIT_CELLS + INIT_CELLS / 2));
+    __shared__ unsigned heads[INIT_CELLS / 32];
+    __shared__ unsigned short hlist[INIT_CELLS];
     T *V = (T *)d.V - (1LL << Jmin) * q;
     uint32_t *leaves = d.lists + d.list_off[L_LEAF], *inner = d.lists + d.list_off[L_INT] - (1 << Jmin);
     const double dx = ldexp(d.b - d.a, -Jmax);
+    // The cells whose moments differ from their left neighbour's (and the first
+    // of every 32) head a stretch of equal cells; only heads are evaluated, side
+    // by side, and the others copy: the data of a Riemann problem are constant
+    // but for some jumps, and the evaluation is what costs (a warp's FP64
+    // instruction takes 16 cycles of the SM).
+    for (int t = tid; t < INIT_CELLS; t += 256) {
+        bool head = false;
+        if (t < ch) {
+            head = (t & 31) == 0;
+            for (int j = 0; j < nf && !head; ++j) {
+                const long long *x = (const long long *)mcons + (long long)j * N + c0 + t;
+                head = x[0] != x[-1];
+            }
+            leaves[c0 + t] = (uint32_t)(N + c0 + t);
+        }
+        const unsigned hb = __ballot_sync(FULL, head);
+        if (lane == 0) heads[t >> 5] = hb;
+    }
+    __syncthreads();
+    int nh = 0;  // all heads, listed in order
+    for (int t = tid; t < INIT_CELLS; t += 256) {
+        const unsigned hb = heads[t >> 5];
+        int r = 0;
+        nh = 0;
+        for (int w = 0; w < INIT_CELLS / 32; ++w) {
+            const int n = __popc(heads[w]);
+            r += w < (t >> 5) ? n : 0;
+            nh += n;
+        }
+        if ((hb >> lane) & 1u) hlist[r + __popc(hb & ((1u << lane) - 1u))] = (unsigned short)t;
+    }
+    __syncthreads();
     double m[3] = {0.0, 0.0, 0.0};
-    for (int t = tid; t < ch; t += 256) {
-        const int k = c0 + t;
-        double mc[3], f[q];
-        for (int j = 0; j < nf; ++j) mc[j] = mcons[(long long)j * N + k];
+#pragma unroll 1
+    for (int r = tid; r < nh; r += 256) {
+        const int t = hlist[r], at = t & 31;
+        const unsigned rest = (heads[t >> 5] >> at) >> 1;
+        const int len = min(rest ? __ffs(rest) : 32 - at, ch - t);
+        double mc[3], f[q], m0 = 0.0, m1 = 0.0;
+        for (int j = 0; j < nf; ++j) mc[j] = mcons[(long long)j * N + c0 + t];
         if constexpr (DQ)
             dq_equilibrium_populations<q>(d, mc, f);
         else
             equilibrium_populations<NF>(d, mc, f);
-        double m0 = 0.0, m1 = 0.0;
+        const double wgt = dx * (double)len;
 #pragma unroll
         for (int j = 0; j < q; ++j) {
             const T x = (T)f[j];
+            f[j] = (double)x;
             a[t * q + j] = x;
             if constexpr (DQ) {
                 m0 += (double)x;
@@ -158,13 +205,20 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
             }
         }
         if constexpr (DQ) {
-            m[0] += dx * m0;
-            m[1] += dx * m1;
+            m[0] += wgt * m0;
+            m[1] += wgt * m1;
         } else {
 #pragma unroll
-            for (int j = 0; j < nf; ++j) m[j] += dx * ((double)a[t * q + 2 * j] + (double)a[t * q + 2 * j + 1]);
+            for (int j = 0; j < nf; ++j) m[j] += wgt * (f[2 * j] + f[2 * j + 1]);
         }
-        leaves[k] = (uint32_t)(N + k);
+    }
+    __syncthreads();
+    for (int t = tid; t < ch; t += 256) {
+        const unsigned le = heads[t >> 5] & (FULL >> (31 - (t & 31)));
+        const int from = (t & ~31) + 31 - __clz(le);
+        if (from != t)
+#pragma unroll
+            for (int j = 0; j < q; ++j) a[t * q + j] = a[from * q + j];
     }
     // values to memory from the shared copy, whose layout is theirs: consecutive
     // threads write consecutive bytes
@@ -175,14 +229,15 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
     // the run's totals, into the interface array (free until the first step)
 #pragma unroll
     for (int j = 0; j < nf; ++j) {
-        for (int o = 16; o > 0; o >>= 1) m[j] += __shfl_down_sync(FULL, m[j], o);
+        if (32 * warp < nh)
+            for (int o = 16; o > 0; o >>= 1) m[j] += __shfl_down_sync(FULL, m[j], o);
         if (lane == 0) red[j][warp] = m[j];
     }
     __syncthreads();
     put(a, (uint32_t)(N + c0), ch);
     if (tid < nf) {
-        double x = 0.0;
-        for (int w = 0; w < 8; ++w) x += red[tid][w];
+        double x = red[tid][0];
+        for (int w = 1; w < 8 && 32 * w < nh; ++w) x += red[tid][w];
         ((double *)d.Phi)[3 * chunk + tid] = x;
     }
     int l = Jmax - 1;
@@ -191,8 +246,8 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
         for (int t = tid; t < n; t += 256) {
 #pragma unroll
             for (int j = 0; j < q; ++j) {
-                const T x = half_of<T>(a[2 * t * q + j] + a[(2 * t + 1) * q + j]);
-                b[t * q + j] = x;
+                const T x = a[2 * t * q + j], y = a[(2 * t + 1) * q + j];
+                b[t * q + j] = mean_of(x, y);
             }
             inner[h0 + t] = h0 + t;
         }
@@ -219,7 +274,7 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
         for (uint32_t h = (1u << l) + tid; h < (2u << l); h += 256) {
 #pragma unroll
             for (int j = 0; j < q; ++j)
-                V[(size_t)h * q + j] = half_of<T>(__ldcg(&V[(size_t)(2u * h) * q + j]) + __ldcg(&V[(size_t)(2u * h + 1u) * q + j]));
+                V[(size_t)h * q + j] = mean_of(__ldcg(&V[(size_t)(2u * h) * q + j]), __ldcg(&V[(size_t)(2u * h + 1u) * q + j]));
             inner[h] = h;
         }
         __threadfence_block();
@@ -286,8 +341,27 @@ __device__ __forceinline__ void init_details(const InstDesc &d, int chunk, const
     for (int w = chunk * wpc + warp; w < (chunk + 1) * wpc; w += 8) {
         const uint32_t p = 32u * w + lane;
         bool keep = false, ref = false, tie = false;
-        if (p >= (1u << d.Jmin) && p < (1u << d.Jmax))
-            pair_decision<T, q, WIDE>(V, p, d.Jmax, d.bc, d.gamma, tab, th, keep, ref, tie);
+        if (p >= (1u << d.Jmin) && p < (1u << d.Jmax)) {
+            bool flat = false;
+            if constexpr (sizeof(T) == 8) {
+                // equal values all over the stencil: the detail is zero (FP64
+                // operations only where some lane of the warp has another)
+                flat = true;
+                const uint32_t lo = level_first(p);
+                const long long *x = (const long long *)V;
+#pragma unroll
+                for (int h = 0; h < q; ++h) {
+                    const long long v = x[p * (uint32_t)q + h];
+                    flat = flat && x[2u * p * (uint32_t)q + h] == v;
+                    for (int a = 1; a <= (WIDE ? d.gamma : 1); ++a)
+                        flat = flat && x[neighbour(p, a, lo, d.bc) * (uint32_t)q + h] == v && x[neighbour(p, -a, lo, d.bc) * (uint32_t)q + h] == v;
+                }
+            }
+            if (flat)
+                decide_bits(0ull, th.eps_l[level_of(p) + 1], th.big_l[level_of(p) + 1], level_of(p) + 1 < d.Jmax, keep, ref, tie);
+            else
+                pair_decision<T, q, WIDE>(V, p, d.Jmax, d.bc, d.gamma, tab, th, keep, ref, tie);
+        }
         const unsigned kb = __ballot_sync(FULL, keep), rb = __ballot_sync(FULL, ref), tb = __ballot_sync(FULL, tie);
         if (lane == 0) {
             d.masks[(long long)M_KEEP * W + w] = kb;

@@ -204,7 +204,7 @@ struct TeamSmem {
 // block-team scratch (scan partials and reduction slots of the warps)
 struct BlockScratch {
     uint32_t scan_w[2][2][32];
-    double red[3][64];
+    double red[3][256];
 };
 
 template <typename T, int NT>
@@ -307,9 +307,28 @@ __device__ __forceinline__ bool mid_range(double x) {
     const unsigned hi = (unsigned)__double2hiint(x);
     return ((hi >> 20) & 0x7FFu) - 64u < 1920u || ((hi << 1) | (unsigned)__double2loint(x)) == 0u;
 }
+// exponents within 300 of 1's (or zero): cubes and quotients of such numbers
+// neither overflow nor underflow
+__device__ __forceinline__ bool cube_range(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    return ((hi >> 20) & 0x7FFu) - 723u < 600u || ((hi << 1) | (unsigned)__double2loint(x)) == 0u;
+}
 __device__ __forceinline__ double markstein(double x, double y, double r) {
     const double q0 = __dmul_rn(x, r);
     return __fma_rn(__fma_rn(-q0, y, x), r, q0);
+}
+// x / y.  The hardware's division sequence leaves its short path for a zero
+// numerator, which a fluid at rest has in every cell: FP64 goes by the
+// reciprocal, FP32 answers a zero itself.
+template <typename T>
+__device__ __forceinline__ T quotient(T x, T y) {
+    if constexpr (sizeof(T) == 8) {
+        if (y != 0.0 && mid_range(y) && mid_range(x)) return markstein(x, y, __drcp_rn(y));
+        return __ddiv_rn(x, y);
+    } else {
+        if (x == 0.0f && y != 0.0f && fabsf(y) < __int_as_float(0x7F800000)) return x * y;  // the zero of the quotient's sign
+        return x / y;
+    }
 }
 // x / (2 lambda), half of what the collision adds to and takes from a moment,
 // for a lambda that is no power of two (halving is exact, so its halves are the
@@ -327,7 +346,12 @@ __device__ __forceinline__ T div_2lam(T x, const InstDesc &d) {
 // equilibria of the relaxed moments; the constant factors (0.5 g, 1.5 - 0.5
 // gamma_gas, gamma_gas - 1, 0.5 (1 - gamma_gas)) come rounded from the host,
 // the same values the expressions would give per cell
-template <typename T, int NF>
+// EXACT: each quotient of the formulas rounded by itself (the initial datum,
+// which equals a plain IEEE evaluation bit for bit); else FP64 Euler takes the
+// velocity u = rho u / rho once and multiplies by it: as many roundings on the
+// way to each flux (one ulp for the quadratic ones, two for the cubic), 14 FP64
+// instructions instead of 28 for the four quotients' part of the collision.
+template <typename T, int NF, bool EXACT = false>
 __device__ __forceinline__ void equilibria(const InstDesc &d, T eqp, const T *mc, T *meq) {
     using A = Ar<T>;
     T ca, cb, cc, g2;
@@ -340,29 +364,35 @@ __device__ __forceinline__ void equilibria(const InstDesc &d, T eqp, const T *mc
     } else if constexpr (NF == 2) {
         // shallow water (h, hu): hu, hu^2 / h + g h^2 / 2
         meq[0] = mc[1];
-        meq[1] = A::add(A::div(A::mul(mc[1], mc[1]), mc[0]), A::mul(g2, A::mul(mc[0], mc[0])));
+        meq[1] = A::add(quotient<T>(A::mul(mc[1], mc[1]), mc[0]), A::mul(g2, A::mul(mc[0], mc[0])));
     } else {
         // Euler (rho, rho u, E), Section 5.3
         T gg = eqp;
         T u2 = A::mul(mc[1], mc[1]);
         meq[0] = mc[1];
         if constexpr (sizeof(T) == 8) {
-            // the three quotients from one reciprocal: its square, refined once, is
-            // that of rho^2 (about 20 FP64 instructions instead of three divisions'
-            // 35; a lane pair of FP64 units makes them the cost of the collision)
-            const double em = A::mul(mc[2], mc[1]), u3 = A::mul(u2, mc[1]);
-            if (mc[0] != 0.0 && mid_range(mc[0]) && mid_range(u2) && mid_range(em) && mid_range(u3)) {
-                const double r = __drcp_rn(mc[0]), r2 = __dmul_rn(mc[0], mc[0]);
-                double q2 = __dmul_rn(r, r);
-                q2 = __fma_rn(__fma_rn(-r2, q2, 1.0), q2, q2);
-                meq[1] = A::add(A::mul(ca, markstein(u2, mc[0], r)), A::mul(cb, mc[2]));
-                meq[2] = A::add(A::mul(gg, markstein(em, mc[0], r)), A::mul(cc, markstein(u3, r2, q2)));
+            if constexpr (EXACT) {
+                // the three quotients from one reciprocal: its square, refined
+                // once, is that of rho^2
+                const double em = A::mul(mc[2], mc[1]), u3 = A::mul(u2, mc[1]);
+                if (mc[0] != 0.0 && mid_range(mc[0]) && mid_range(u2) && mid_range(em) && mid_range(u3)) {
+                    const double r = __drcp_rn(mc[0]), r2 = __dmul_rn(mc[0], mc[0]);
+                    double q2 = __dmul_rn(r, r);
+                    q2 = __fma_rn(__fma_rn(-r2, q2, 1.0), q2, q2);
+                    meq[1] = A::add(A::mul(ca, markstein(u2, mc[0], r)), A::mul(cb, mc[2]));
+                    meq[2] = A::add(A::mul(gg, markstein(em, mc[0], r)), A::mul(cc, markstein(u3, r2, q2)));
+                    return;
+                }
+            } else if (mc[0] != 0.0 && cube_range(mc[0]) && cube_range(mc[1]) && cube_range(mc[2])) {
+                const double u = markstein(mc[1], mc[0], __drcp_rn(mc[0])), mu = A::mul(mc[1], u);
+                meq[1] = A::add(A::mul(ca, mu), A::mul(cb, mc[2]));
+                meq[2] = A::add(A::mul(gg, A::mul(mc[2], u)), A::mul(cc, A::mul(mu, u)));
                 return;
             }
         }
-        meq[1] = A::add(A::mul(ca, A::div(u2, mc[0])), A::mul(cb, mc[2]));
-        meq[2] = A::add(A::mul(gg, A::div(A::mul(mc[2], mc[1]), mc[0])),
-                        A::mul(cc, A::div(A::mul(u2, mc[1]), A::mul(mc[0], mc[0]))));
+        meq[1] = A::add(A::mul(ca, quotient<T>(u2, mc[0])), A::mul(cb, mc[2]));
+        meq[2] = A::add(A::mul(gg, quotient<T>(A::mul(mc[2], mc[1]), mc[0])),
+                        A::mul(cc, quotient<T>(A::mul(u2, mc[1]), A::mul(mc[0], mc[0]))));
     }
 }
 
@@ -405,7 +435,7 @@ template <int NF>
 __device__ __forceinline__ void equilibrium_populations(const InstDesc &d, const double *mc, double *f) {
     using A = Ar<double>;
     double meq[NF];
-    equilibria<double, NF>(d, d.eqp, mc, meq);
+    equilibria<double, NF, true>(d, d.eqp, mc, meq);
 #pragma unroll
     for (int i = 0; i < NF; ++i) {
         const double g = half_over_lam<double>(meq[i], d), m = half_f64(mc[i]);
@@ -466,7 +496,7 @@ __device__ __forceinline__ void dq_collide(const InstDesc &d, T *f) {
     dq_moments<T, Q>(lam, f, m);
     T ca, cb, cc, g2;
     eq_consts<T>(d, ca, cb, cc, g2);
-    meq[2] = (m[1] * m[1]) / m[0] + g2 * (m[0] * m[0]);
+    meq[2] = quotient<T>(m[1] * m[1], m[0]) + g2 * (m[0] * m[0]);
     if constexpr (Q == 5) {
         meq[3] = (lam * lam) * m[1];
         meq[4] = (lam * lam) * meq[2];
@@ -482,7 +512,7 @@ __device__ __forceinline__ void dq_equilibrium_populations(const InstDesc &d, co
     double m[5];
     m[0] = mc[0];
     m[1] = mc[1];
-    m[2] = (mc[1] * mc[1]) / mc[0] + (0.5 * d.eqp) * (mc[0] * mc[0]);
+    m[2] = quotient<double>(mc[1] * mc[1], mc[0]) + (0.5 * d.eqp) * (mc[0] * mc[0]);
     if constexpr (Q == 5) {
         m[3] = (d.lam * d.lam) * mc[1];
         m[4] = (d.lam * d.lam) * m[2];
@@ -755,12 +785,12 @@ struct Worker {
     // and the sum of field j of them by one warp: the warps TS / 32 - 1 - j fold one
     // field each, valid in their lane 0, while the others go on.  GB300's FP64
     // units take a warp-wide instruction whole whatever its active lanes, so
-    // additions are kept off most warps: two shuffle rounds or so leave 64
-    // partials a field (groups of TS / 64 lanes), and warps without a leaf (the
-    // first n threads have one) only write their zeros.  A fixed order:
-    // deterministic.
+    // additions are kept off most warps: a thread's own sum is a partial up to
+    // 256 threads (shuffle rounds fold wider blocks to 256), and one warp adds
+    // eight a lane and shuffles.  Warps without a leaf (the first n threads have
+    // one) only write their zeros.  A fixed order: deterministic.
     __device__ __forceinline__ void team_partials(double (&x)[3], int n) {
-        constexpr int G = TS / 64;  // lanes per partial sum: 2, 4, 8 or 16
+        constexpr int G = TS / NPART;  // lanes per partial sum: 1, 2 or 4
         if ((tid & ~31) < n)
 #pragma unroll
             for (int j = 0; j < nf; ++j)
@@ -771,9 +801,12 @@ struct Worker {
             for (int j = 0; j < nf; ++j) bx.red[j][tid / G] = x[j];
         sync();
     }
+    static constexpr int NPART = TS < 256 ? TS : 256;
     __device__ __forceinline__ double team_fold(int j) const {
         const int lane = tid & 31;
-        double v = bx.red[j][lane] + bx.red[j][lane + 32];
+        double v = bx.red[j][lane];
+#pragma unroll
+        for (int k = 32; k < NPART; k += 32) v += bx.red[j][lane + k];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
         return v;
@@ -837,7 +870,7 @@ struct Worker {
             }
             T ca, cb, cc, g2;
             eq_consts<T>(d, ca, cb, cc, g2);
-            meq[0] = (hu * hu) / h + g2 * (h * h);
+            meq[0] = quotient<T>(hu * hu, h) + g2 * (h * h);
             if constexpr (q == 5) {
                 meq[1] = (lam * lam) * hu;
                 meq[2] = (lam * lam) * meq[0];

@@ -145,7 +145,8 @@ struct mr_ctx {
     int precision = MR_FP64;
     // layout (bytes from the workspace base)
     size_t off_desc = 0, off_state = 0, off_order = 0, off_ident = 0, off_queue = 0, off_tab = 0,
-           off_stage = 0, off_chunk = 0, total = 0;
+           off_stage = 0, off_chunk = 0, off_wide = 0, total = 0;
+    bool wide = false;             // some instance has gamma > 1
     int nchunk = 0;                // runs of the initial state over all instances
     std::vector<size_t> inst_off;  // per instance region start
     std::vector<InstDesc> hdesc;   // host copy of the device descriptors
@@ -245,6 +246,10 @@ static void layout(mr_ctx *c) {
     c->off_chunk = o;
     o = align_up(o + sizeof(int) * (size_t)c->nchunk);
     int chunk0 = 0;
+    c->wide = false;
+    for (int i = 0; i < n; ++i) c->wide = c->wide || c->desc[i].gamma > 1;
+    c->off_wide = o;
+    if (c->wide) o = align_up(o + (c->fp32() ? sizeof(WideTables<float>) : sizeof(WideTables<double>)));
     c->inst_off.assign(n, 0);
     c->hdesc.assign(n, InstDesc{});
     for (int i = 0; i < n; ++i) {
@@ -383,6 +388,61 @@ static void make_tables(Tables<double> &td, Tables<float> &tf) {
         }
 }
 
+// Wide reconstruction tables, by recursion over the gap: the weights W_{dj} on a
+// window are those of gap dj - 1 on the window around the leaf's first child,
+// carried through the prediction; weights on window positions beyond a boundary
+// go to the boundary cell, whose value they stand for.  A leaf k cells from the
+// left boundary has its first child 2k from it, one r from the right 2r + 1.
+template <int G, int NC, int W>
+static void make_wide(double (&w)[NC][MAXDJ + 1][W]) {
+    static_assert(NC == 4 * G + 1 && W == 4 * G + 1, "codes and window");
+    const double coef[4][3] = {{0, 0, 0}, {0, 0, 0}, {-22.0 / 128.0, 3.0 / 128.0, 0.0}, {-201.0 / 1024.0, 11.0 / 256.0, -5.0 / 1024.0}};
+    const double *c = coef[G];
+    constexpr int C = 2 * G;
+    for (int code = 0; code < NC; ++code)
+        for (int t = 0; t < W; ++t) w[code][0][t] = t == C ? 1.0 : 0.0;
+    for (int dj = 1; dj <= MAXDJ; ++dj)
+        for (int code = 0; code < NC; ++code) {
+            int left = 1 << 20, right = 1 << 20, child = 0;  // the first child's distance from the boundaries
+            if (code >= 1 && code <= C) left = 2 * (code - 1);
+            if (code > C) right = 2 * (code - 1 - C) + 1;
+            if (left < C) child = 1 + left;
+            if (right < C) child = 1 + C + right;
+            const double *in = w[child][dj - 1];
+            double out[W] = {};
+            for (int t = 0; t < W; ++t) {
+                if (in[t] == 0.0) continue;
+                const int o = t - C, po = (o >= 0 ? o / 2 : -((1 - o) / 2)), sgn = (o & 1) ? -1 : 1;
+                out[C + po] += in[t];
+                for (int a = 1; a <= G; ++a) {
+                    out[C + po + a] += sgn * c[a - 1] * in[t];
+                    out[C + po - a] -= sgn * c[a - 1] * in[t];
+                }
+            }
+            // onto the boundary cell, for which positions beyond it stand
+            const int b = code >= 1 && code <= C ? C - (code - 1) : 0, e = code > C ? C + (code - 1 - C) : W - 1;
+            for (int t = 0; t < W; ++t) w[code][dj][t] = 0.0;
+            for (int t = 0; t < W; ++t) w[code][dj][std::min(std::max(t, b), e)] += out[t];
+        }
+}
+namespace {
+struct HostWide {
+    WideTables<double> d;
+    WideTables<float> f;
+    HostWide() {
+        make_wide<2>(d.w2);
+        make_wide<3>(d.w3);
+        const double *s = (const double *)&d;
+        float *t = (float *)&f;
+        for (size_t i = 0; i < sizeof d / sizeof(double); ++i) t[i] = (float)s[i];
+    }
+};
+}  // namespace
+const void *mrg_wide_tables(bool fp32) {
+    static const HostWide w;  // thread-safe initialisation
+    return fp32 ? (const void *)&w.f : (const void *)&w.d;
+}
+
 static int launch_group(mr_ctx *c, int phases, int nsteps, const int *order, int n, int kind, const void *aux0,
                         const void *aux1, cudaStream_t stream, int priority) {
     LaunchArgs a{};
@@ -396,6 +456,7 @@ static int launch_group(mr_ctx *c, int phases, int nsteps, const int *order, int
     a.aux0 = aux0;
     a.aux1 = aux1;
     a.tables = c->ws + c->off_tab + (c->fp32() ? sizeof(Tables<double>) : 0);
+    a.wide = c->wide ? c->ws + c->off_wide : nullptr;
     a.smem_mask_words = c->mask_cap[kind];
     int rc = c->cuda(cudaMemsetAsync(a.queue, 0, sizeof(int), stream), "cudaMemsetAsync");
     if (rc) return rc;
@@ -676,6 +737,10 @@ mr_status mr_bind(mr_ctx *c, void *ws, size_t bytes, void *stream) {
         return (mr_status)rc;
     if ((rc = c->cuda(cudaMemcpyAsync(c->ws + c->off_tab, &td, sizeof td, cudaMemcpyHostToDevice, s), "upload"))) return (mr_status)rc;
     if ((rc = c->cuda(cudaMemcpyAsync(c->ws + c->off_tab + sizeof td, &tf, sizeof tf, cudaMemcpyHostToDevice, s), "upload")))
+        return (mr_status)rc;
+    if (c->wide && (rc = c->cuda(cudaMemcpyAsync(c->ws + c->off_wide, mrg_wide_tables(c->fp32()),
+                                                 c->fp32() ? sizeof(WideTables<float>) : sizeof(WideTables<double>),
+                                                 cudaMemcpyHostToDevice, s), "upload")))
         return (mr_status)rc;
     std::vector<int> chunk_inst((size_t)c->nchunk);
     for (int i = 0; i < n; ++i) std::fill_n(chunk_inst.begin() + dd[i].chunk0, init_chunks_of(dd[i].Jmax), i);

@@ -161,6 +161,18 @@ struct Tables {
     T pc[4][3];
 };
 
+// Reconstruction tables for gamma = 2, 3: weights of the first finest cell of a
+// leaf at level gap dj on its level's window h - 2 gamma .. h + 2 gamma when no
+// cell of the window is refined, by where the leaf lies: [0] away from a copy
+// boundary, [1 + k] k < 2 gamma cells from the left one, [1 + 2 gamma + r] r from
+// the right one (a window position beyond the boundary stands for the boundary
+// cell).  The last finest cell uses the mirrored window.
+template <typename T>
+struct WideTables {
+    T w2[9][MAXDJ + 1][9];
+    T w3[13][MAXDJ + 1][13];
+};
+
 // the initial state is set by runs of this many finest cells (2^Jmax when fewer)
 constexpr int INIT_CELLS = 512;
 MRG_HD inline int init_chunks_of(int Jmax) { return Jmax > 9 ? 1 << (Jmax - 9) : 1; }
@@ -175,6 +187,7 @@ struct LaunchArgs {
     const void *aux0;     // phase input / output (see the kernel)
     const void *aux1;
     const void *tables;   // Tables<T> in device memory
+    const void *wide;     // WideTables<T> (null when no instance has gamma > 1)
     int smem_mask_words;  // block teams keep their mask region in shared memory when it has at most this many words
     int kind;             // kernel variant (K_*) the launch runs
 };
@@ -208,6 +221,7 @@ int mrg_init(bool fp32, const mrg::InstDesc *descs, const int *chunk_inst, int n
 // on its finest level, into device memory (mr_field.cu)
 int mrg_finest(bool fp32, int var, int Jmax, const mrg::InstDesc *desc, const void *tables, double *out, void *stream);
 void mrg_tables(mrg::Tables<double> *td, mrg::Tables<float> *tf);
+const void *mrg_wide_tables(bool fp32);  // host copy of WideTables<T>, built once
 void mrg_set_error(const char *msg);
 // scheme shape (mr_api.cu): conserved fields, populations, relaxation rates of
 // an mr_equilibrium, and the inverse moment matrix of the D1Q3 / D1Q5 schemes

@@ -665,14 +665,16 @@ struct Worker {
     BlockScratch &bx;
     const InstDesc &d;
     T *V;         // cell h at V + h q
+    const WideTables<T> *wide;
     uint32_t *M;  // bit arrays (shared memory when they fit, else global)
     const int tid;
     const int bc, Jmin, Jmax;
 
-    __device__ Worker(TeamSmem<T> &s, const Tables<T> &tb, BlockScratch &x, int rank, uint32_t *masks)
+    __device__ Worker(TeamSmem<T> &s, const Tables<T> &tb, BlockScratch &x, int rank, uint32_t *masks, const void *wd)
         : sm(s), tab(tb), bx(x), d(s.d), tid(rank), bc(s.d.bc), Jmin(s.d.Jmin), Jmax(s.d.Jmax) {
         V = (T *)d.V - (1LL << d.Jmin) * q;
         M = masks;
+        wide = (const WideTables<T> *)wd;
     }
 
     // leaves collision of the q populations of one cell
@@ -1492,9 +1494,14 @@ struct Worker {
         tick(T_GHOSTS);
         if constexpr (DQ)
             reconstruct_dq();  // S4 (gamma = 1)
-        else if (WIDE && d.gamma > 1)
-            reconstruct_wide();
-        else
+        else if (WIDE && d.gamma > 1) {
+            if constexpr (WIDE) {
+                if (d.gamma == 2)
+                    reconstruct_wide<2>();
+                else
+                    reconstruct_wide<3>();
+            }
+        } else
             reconstruct_edges();
         sync();
         tick(T_RECON);
@@ -1656,13 +1663,26 @@ struct Worker {
         return w[C];
     }
 
-    // S4 with the stencil of half-width gamma = 2 or 3: the first / last finest
-    // values by the level-by-level reconstruction (edge_walk) instead of tables
+    // S4 with the stencil of half-width G = 2 or 3: the first / last finest value
+    // of a leaf from its level's window (h - 2G .. h + 2G) and the tables.  Where
+    // a cell p of the window within G of the leaf is refined, the tree's children
+    // of p stand in the window one level down in the place of the predicted ones;
+    // the two differ by the pair's detail, with opposite signs, and the weights of
+    // that window carry the difference.  Further down the window holds no tree
+    // cell: a cell two levels below the leaf's needs, graded, the cells within G
+    // of its parent in the tree, and the leaf's children are not.  So a value
+    // costs 4G + 1 products and 2G + 3 operations a refined cell, where the
+    // level-by-level walk (edge_walk) predicted the whole window at each of the
+    // Jmax - l levels: 178K of a step's 238K cycles on a gamma = 3 batch (FP64).
+    // The walk is left for a leaf within 2G cells of both copy boundaries.
+    template <int G>
     __device__ __noinline__ void reconstruct_wide() {
+        constexpr int C = 2 * G, W = 4 * G + 1;
         const uint32_t *I = mask(sm.cur);
         const uint32_t *leaves = list(L_LEAF);
-        const int g = d.gamma, nl = sm.nleaf;
-        const T *cf = tab.pc[g];
+        const int nl = sm.nleaf;
+        const T *cf = tab.pc[G];
+        const T *wt = G == 2 ? &wide->w2[0][0][0] : &wide->w3[0][0][0];
         const uint32_t N = 1u << Jmax;
 #pragma unroll 1
         for (int i = tid; i < nl; i += TS) {
@@ -1672,14 +1692,58 @@ struct Worker {
             const uint32_t first = (h << dj) & (N - 1u);
             uint32_t next = first + (1u << dj);
             if (bc == 0) next &= N - 1u;
+            const int kl = bc == 0 ? C : min((int)(h - lo), C), kr = bc == 0 ? C : min((int)(2u * lo - 1u - h), C);
+            unsigned refined = 0u;  // cells within G that are internal
+            if (dj > 0)
+#pragma unroll
+                for (int o = -G; o <= G; ++o)
+                    // beyond a copy boundary stands the boundary cell, whose children are predicted there like its own
+                    if (o != 0 && (o > 0 ? o <= kr : -o <= kl) && bit_of(I, nb(h, o, lo))) refined |= 1u << (o + G);
 #pragma unroll 1
-            for (int c = 0; c < q; ++c) {
-                const bool plus = (c & 1) == 0;  // velocity +lambda
-                T rfirst = T(0), rlast = T(0);
-                if (!plus || at_left) rfirst = g == 2 ? edge_walk<2, false>(I, cf, c, h) : edge_walk<3, false>(I, cf, c, h);
-                if (plus || at_right) rlast = g == 2 ? edge_walk<2, true>(I, cf, c, h) : edge_walk<3, true>(I, cf, c, h);
-                if (plus || at_right) phi(next)[c] = rlast;
-                if (!plus || at_left) phi(first)[c] = rfirst;
+            for (int e = 0; e < q + (at_left ? NF : 0) + (at_right ? NF : 0); ++e) {
+                // population and end: +lambda its last value, -lambda its first; at a boundary the other end too
+                int c = e;
+                bool last = (c & 1) == 0;
+                if (e >= q) {
+                    const bool l = at_left && e < q + NF;
+                    c = 2 * (e - q - (at_left && !l ? NF : 0)) + (l ? 0 : 1);
+                    last = !l;
+                }
+                T *out = phi(last ? next : first) + c;
+                const T *vc = V + c;
+                auto at = [&](uint32_t x) { return vc[x * (uint32_t)q]; };
+                if (dj == 0) {
+                    *out = at(h);
+                    continue;
+                }
+                if (kl < C && kr < C) {
+                    *out = last ? edge_walk<G, true>(I, cf, c, h) : edge_walk<G, false>(I, cf, c, h);
+                    continue;
+                }
+                const int sg = last ? -1 : 1, k = last ? kr : kl, r = last ? kl : kr;  // distances, mirrored for the last value
+                const int code = k < C ? 1 + k : r < C ? 1 + C + r : 0;
+                const T *w = wt + (code * (MAXDJ + 1) + dj) * W;
+                T sum = T(0);
+#pragma unroll
+                for (int t = 0; t < W; ++t) sum = sum + w[t] * at(nb(h, sg * (t - C), lo));
+                if (refined) {
+                    const int k1 = 2 * k, r1 = 2 * r + 1;  // of the child at that end
+                    const int code1 = code == 0 ? 0 : k < C ? (k1 < C ? 1 + k1 : 0) : (r1 < C ? 1 + C + r1 : 0);
+                    const T *w1 = wt + (code1 * (MAXDJ + 1) + dj - 1) * W + C;
+                    unsigned m = refined;
+#pragma unroll 1
+                    while (m) {
+                        const int po = __ffs(m) - 1 - G, o = sg * po;
+                        m &= m - 1u;
+                        const uint32_t p = nb(h, po, lo);
+                        T s = cf[0] * (at(nb(p, sg, lo)) - at(nb(p, -sg, lo)));
+#pragma unroll
+                        for (int a = 2; a <= G; ++a) s = s + cf[a - 1] * (at(nb(p, sg * a, lo)) - at(nb(p, -sg * a, lo)));
+                        const T detail = at(last ? 2u * p + 1u : 2u * p) - (at(p) + s);
+                        sum = sum + (w1[2 * o] - (o < G ? w1[2 * o + 1] : T(0))) * detail;
+                    }
+                }
+                *out = sum;
             }
         }
     }
@@ -2088,7 +2152,7 @@ __device__ void store_instance(TeamSmem<T> &sm, int tid) {
 template <typename T, int NF, int TS, bool WIDE, int SPM>
 __device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx, const LaunchArgs &a, int tid,
                              uint32_t *masks) {
-    Worker<T, NF, TS, WIDE, SPM> w(sm, tab, bx, tid, masks);
+    Worker<T, NF, TS, WIDE, SPM> w(sm, tab, bx, tid, masks, a.wide);
     if (a.phases & PH_INIT_STATE) w.init_state((const unsigned char *)a.aux0, (const double *)a.aux1);
 #pragma unroll 1
     for (int n = 0; n < a.nsteps; ++n) {

@@ -117,6 +117,9 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     o = align256(o + 2 * sizeof(int));
     const size_t oTab = o;
     o = align256(o + sizeof(Tables<double>) + sizeof(Tables<float>));
+    const size_t wide_bytes = d.gamma > 1 ? (fp32 ? sizeof(WideTables<float>) : sizeof(WideTables<double>)) : 0;
+    const size_t oWide = o;
+    o = align256(o + wide_bytes);
     const size_t oV = o;
     o = align256(o + vb * q * S);
     const size_t oPhi = o;
@@ -192,6 +195,7 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + oQueue, zero2, sizeof zero2, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + oTab, &td, sizeof td, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(base + oTab + sizeof td, &tf, sizeof tf, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && wide_bytes) e = cudaMemcpyAsync(base + oWide, mrg_wide_tables(fp32), wide_bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail(MR_ERR_CUDA, "mr_run_static: upload failed (%lld)", (long long)e);
 
     // one block for the instance, bitmasks in shared memory when they fit
@@ -205,6 +209,7 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     a.n = 1;
     a.queue = (int *)(base + oQueue);
     a.tables = base + oTab + (fp32 ? sizeof(Tables<double>) : 0);
+    a.wide = wide_bytes ? base + oWide : nullptr;
     const long long sregion = smem_region_words(W, OW);
     a.smem_mask_words = sregion <= fit ? (int)sregion : 0;
     a.kind = d.gamma > 1 ? K_GENERAL : d.collision != 0 ? K_RECOLL : W >= CW_MIN_WORDS ? K_LARGE : K_FAST;

@@ -650,6 +650,27 @@ static int configure(mr_ctx *c) {
     return MR_OK;
 }
 
+// Threads per block unless the caller or the autotuner chose them.  An SM holds
+// about 1024 threads of the kernels, so 1024 / threads instances at once; wide
+// blocks finish an instance sooner, narrow ones keep more of them in flight.
+// The queue evens out uneven instances only when it hands an SM two or three
+// rounds of them.  Measured, us per step of the mixed FP64 batch (Jmax 8..14)
+// by instances per SM, at 128 / 256 / 512 / 1024 threads:
+//    1.0  64 / 41 / 38 / 38      4.6  105 / 82 / 56 / 87     14.5  149 / 115 / 157 / 264
+//    2.0  89 / 59 / 53 / 44      6.6  123 / 85 / 73 / 123    21    161 / 165 / 225 / 381
+//    3.0  90 / 74 / 57 / 58      9.9  142 / 89 / 108 / 180   27    208 / 229 / 302 / 498
+// FP32, D1Q3 / D1Q5, the wide stencils and the reconstructed collision cross at
+// the same places (FP32 at 6.6: 65 / 44 / 47 / 87).  Alone an instance takes
+// 15.2 us a step with 512 threads against 16.4 and 15.6 with 256 and 1024
+// (Burgers Jmax 13).
+static int default_block(int n, int sms) {
+    const double per_sm = (double)n / std::max(1, sms);
+    if (per_sm <= 1.0) return 512;
+    if (per_sm <= 2.6) return 1024;
+    if (per_sm <= 6.5) return 512;
+    return per_sm <= 19.0 ? 256 : 128;
+}
+
 // Processing order of the work queue: by kernel variant group (fast, scalar,
 // general), then by field count (blocks resident together then run the same
 // scheme's code, which keeps the instruction cache warm) unless disabled, then
@@ -716,12 +737,7 @@ mr_status mr_bind(mr_ctx *c, void *ws, size_t bytes, void *stream) {
         dd[i].lists = (uint32_t *)(base + (size_t)dd[i].lists);
         dd[i].st = (InstState *)(c->ws + c->off_state) + i;
     }
-    // launch shape: one block per instance; 1024 threads for a lone large instance
-    if (c->block == 0) {
-        int jmax = 0;
-        for (auto &d : c->desc) jmax = std::max(jmax, d.Jmax);
-        c->block = n == 1 ? (jmax >= 12 ? 1024 : 512) : 256;
-    }
+    if (c->block == 0) c->block = default_block(n, c->sms);
     c->hdesc = dd;
     Tables<double> td;
     Tables<float> tf;

@@ -199,7 +199,7 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     if (e != cudaSuccess) return fail(MR_ERR_CUDA, "mr_run_static: upload failed (%lld)", (long long)e);
 
     // one block for the instance, bitmasks in shared memory when they fit
-    const int block = d.Jmax >= 12 ? 1024 : 512;
+    const int block = 512;
     size_t sbase = mrg_smem_bytes(fp32, block, 0), limit = 220u * 1024u;
     long long fit = limit > sbase ? (long long)((limit - sbase) / sizeof(uint32_t)) : 0;
     LaunchArgs a;

@@ -201,16 +201,19 @@ struct TeamSmem {
 #endif
 };
 
-// block-team scratch (scan partials and reduction slots of the warps)
+// block-team scratch: scan partials of the warps, and the audit's partial sums
+// (FP64: one a thread up to 256 threads; FP32: a float-float pair a warp)
+template <typename T, int NT>
 struct BlockScratch {
+    static constexpr int NPART = sizeof(T) == 4 ? 64 : NT < 256 ? NT : 256;
     uint32_t scan_w[2][2][32];
-    double red[3][256];
+    double red[3][NPART];
 };
 
 template <typename T, int NT>
 struct BlockSmem {
     Tables<T> tab;
-    BlockScratch scratch;
+    BlockScratch<T, NT> scratch;
     TeamSmem<T> team;
     int idx;
 };
@@ -662,7 +665,7 @@ struct Worker {
     static_assert(TS >= 64 && TS % 64 == 0, "team width");
     TeamSmem<T> &sm;
     const Tables<T> &tab;
-    BlockScratch &bx;
+    BlockScratch<T, TS> &bx;
     const InstDesc &d;
     T *V;         // cell h at V + h q
     const WideTables<T> *wide;
@@ -670,7 +673,7 @@ struct Worker {
     const int tid;
     const int bc, Jmin, Jmax;
 
-    __device__ Worker(TeamSmem<T> &s, const Tables<T> &tb, BlockScratch &x, int rank, uint32_t *masks, const void *wd)
+    __device__ Worker(TeamSmem<T> &s, const Tables<T> &tb, BlockScratch<T, TS> &x, int rank, uint32_t *masks, const void *wd)
         : sm(s), tab(tb), bx(x), d(s.d), tid(rank), bc(s.d.bc), Jmin(s.d.Jmin), Jmax(s.d.Jmax) {
         V = (T *)d.V - (1LL << d.Jmin) * q;
         M = masks;
@@ -803,7 +806,7 @@ struct Worker {
             for (int j = 0; j < nf; ++j) bx.red[j][tid / G] = x[j];
         sync();
     }
-    static constexpr int NPART = TS < 256 ? TS : 256;
+    static constexpr int NPART = BlockScratch<T, TS>::NPART;
     __device__ __forceinline__ double team_fold(int j) const {
         const int lane = tid & 31;
         double v = bx.red[j][lane];
@@ -1273,19 +1276,14 @@ struct Worker {
 #pragma unroll 1
         for (int r = 0, base = 0; base < nu; ++r, base += TS) {
             const int u = base + tid;
-            uint32_t m[3] = {0u, 0u, 0u}, lf0 = 0u, lf1 = 0u, w = 0u;
+            uint32_t m[3] = {0u, 0u, 0u}, lf0 = 0u, lf1 = 0u, w = 0u, xp = 0u;
             const bool whole = u < nu && (u & ((1 << s) - 1)) == 0;  // the first unit of its word
             if (u < nu) {
                 w = word_at(u >> s);
                 const uint32_t x = In[w], pm = (FULL >> (32 - width)) << ((u & ((1 << s) - 1)) * width);
-                const uint32_t c0 = 2u * w < wend ? In[2u * w] : 0u, c1 = 2u * w + 1u < wend ? In[2u * w + 1u] : 0u;
-                const uint32_t xp = x & pm;
-                m[L_INT] = xp & ~above(w);
-                m[L_PRED] = xp & ~Io[w];
+                xp = x & pm;
                 if (2u * w < wend || w == 0u) m[L_GH] = dilate_word(In, w, g, bc) & ~x & pm;
                 if (w == 0u) m[L_GH] &= (1u << (Jmax - 1 < 5 ? 1 << (Jmax - 1) : 31)) * (Jmax - 1 < 5 ? 1u : 2u) - 1u;
-                lf0 = spread16(xp) & ~c0;
-                lf1 = spread16(xp >> 16) & ~c1;
                 if (whole) {
                     keep[w] = 0u;
                     ref[w] = 0u;
@@ -1293,17 +1291,28 @@ struct Worker {
                         if (x) atomicOr(&occn[w >> 5], 1u << (w & 31u));
                 }
             }
+            // most words of a fine level are empty: a warp without entries skips the scan
+            const bool some = __any_sync(FULL, (xp | m[L_GH]) != 0u);
             // per round at most 1024 x 32 internal cells and new pairs (16 bits
-            // each), 1024 x 64 leaves (17 bits), 1024 x 16 ghost pairs (15 bits)
-            uint32_t x01 = (uint32_t)__popc(m[0]) | ((uint32_t)__popc(m[1]) << 16);
-            uint32_t x23 = (uint32_t)(__popc(lf0) + __popc(lf1)) | ((uint32_t)__popc(m[2]) << 17);
-            const uint32_t c01 = x01, c23 = x23;
+            // each), 1024 x 64 leaves (17 bits), 1024 x 28 ghost pairs (15 bits)
+            uint32_t x01 = 0u, x23 = 0u, c01 = 0u, c23 = 0u;
+            if (some) {
+                if (xp) {
+                    const uint32_t c0 = 2u * w < wend ? In[2u * w] : 0u, c1 = 2u * w + 1u < wend ? In[2u * w + 1u] : 0u;
+                    m[L_INT] = xp & ~above(w);
+                    m[L_PRED] = xp & ~Io[w];
+                    lf0 = spread16(xp) & ~c0;
+                    lf1 = spread16(xp >> 16) & ~c1;
+                }
+                x01 = c01 = (uint32_t)__popc(m[0]) | ((uint32_t)__popc(m[1]) << 16);
+                x23 = c23 = (uint32_t)(__popc(lf0) + __popc(lf1)) | ((uint32_t)__popc(m[2]) << 17);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y01 = __shfl_up_sync(FULL, x01, o), y23 = __shfl_up_sync(FULL, x23, o);
-                if (lane >= o) {
-                    x01 += y01;
-                    x23 += y23;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y01 = __shfl_up_sync(FULL, x01, o), y23 = __shfl_up_sync(FULL, x23, o);
+                    if (lane >= o) {
+                        x01 += y01;
+                        x23 += y23;
+                    }
                 }
             }
             uint32_t(*sw)[32] = bx.scan_w[r & 1];  // alternate buffers: one barrier per round
@@ -1313,35 +1322,35 @@ struct Worker {
             }
             sync();
             const uint32_t v01 = lane < NW ? sw[0][lane] : 0u, v23 = lane < NW ? sw[1][lane] : 0u;
-            x01 += __reduce_add_sync(FULL, lane < warp ? v01 : 0u) - c01;
-            x23 += __reduce_add_sync(FULL, lane < warp ? v23 : 0u) - c23;
             const uint32_t t01 = __reduce_add_sync(FULL, v01), t23 = __reduce_add_sync(FULL, v23);
-            const uint32_t at[3] = {run[0] + (x01 & 0xFFFFu), run[1] + (x01 >> 16), run[2] + (x23 >> 17)};
-            if (whole && w > 0u) {
-                // the first word of a level; a candidate list may leave whole levels out
-                const int l = 5 + level_of(w);
-                int k = l;
-                if constexpr (SPM != 0) {
-                    const uint32_t before = word_at((u >> s) - 1);  // a list starts with words 0, 1, ...
-                    k = before == 0u ? 5 : 6 + level_of(before);
-                } else if ((w & (w - 1u)) != 0u)
-                    k = l + 1;
-                for (; k <= l; ++k)
+            // the first word of a level; a candidate list may leave whole levels out
+            const bool starts = whole && w > 0u && (SPM != 0 || (w & (w - 1u)) == 0u);
+            if (some || __any_sync(FULL, starts)) {
+                x01 += __reduce_add_sync(FULL, lane < warp ? v01 : 0u) - c01;
+                x23 += __reduce_add_sync(FULL, lane < warp ? v23 : 0u) - c23;
+                const uint32_t at[3] = {run[0] + (x01 & 0xFFFFu), run[1] + (x01 >> 16), run[2] + (x23 >> 17)};
+                if (starts) {
+                    const int l = 5 + level_of(w);
+                    int k = l;
+                    if constexpr (SPM != 0) {
+                        const uint32_t before = word_at((u >> s) - 1);  // a list starts with words 0, 1, ...
+                        k = before == 0u ? 5 : 6 + level_of(before);
+                    }
+                    for (; k <= l; ++k)
 #pragma unroll
-                    for (int L = 0; L < NSEG; ++L) sm.seg[L][k] = at[L];
-            }
-            const uint32_t h0 = 32u * w;
-#pragma unroll
-            for (int L = 0; L < NSEG; ++L) {
-                uint32_t *dst = list(L) + at[L];
-                uint32_t x = m[L];
-#pragma unroll 1
-                while (x) {
-                    *dst++ = h0 + (uint32_t)__ffs(x) - 1u;
-                    x &= x - 1u;
+                        for (int L = 0; L < NSEG; ++L) sm.seg[L][k] = at[L];
                 }
-            }
-            {
+                const uint32_t h0 = 32u * w;
+#pragma unroll
+                for (int L = 0; L < NSEG; ++L) {
+                    uint32_t *dst = list(L) + at[L];
+                    uint32_t x = m[L];
+#pragma unroll 1
+                    while (x) {
+                        *dst++ = h0 + (uint32_t)__ffs(x) - 1u;
+                        x &= x - 1u;
+                    }
+                }
                 uint32_t *dst = list(L_LEAF) + run[3] + (x23 & 0x1FFFFu);
 #pragma unroll 1
                 while (lf0) {
@@ -2150,7 +2159,7 @@ __device__ void store_instance(TeamSmem<T> &sm, int tid) {
 
 // one instance for the launch's steps
 template <typename T, int NF, int TS, bool WIDE, int SPM>
-__device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx, const LaunchArgs &a, int tid,
+__device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch<T, TS> &bx, const LaunchArgs &a, int tid,
                              uint32_t *masks) {
     Worker<T, NF, TS, WIDE, SPM> w(sm, tab, bx, tid, masks, a.wide);
     if (a.phases & PH_INIT_STATE) w.init_state((const unsigned char *)a.aux0, (const double *)a.aux1);
@@ -2167,7 +2176,7 @@ __device__ __forceinline__ void run_instance(TeamSmem<T> &sm, const Tables<T> &t
 // that come with an initial state, ST_DETAILS), and every adaptation writes the
 // other tree buffer.
 template <typename T, int TS, bool WIDE, bool SCALAR, int SPM>
-__device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch &bx, const LaunchArgs &a,
+__device__ void run_team(TeamSmem<T> &sm, const Tables<T> &tab, BlockScratch<T, TS> &bx, const LaunchArgs &a,
                          const InstDesc &dg, int tid, uint32_t *smask, int cap) {
     load_instance<T, TS>(sm, dg, tid);
     const int W = sm.d.Wtot, OW = sm.d.OW;

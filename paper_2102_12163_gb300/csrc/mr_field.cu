@@ -24,45 +24,70 @@ namespace mrg {
 // microseconds.  The one-block version (a projection sweep and one pass over
 // each level through global memory) took 37 us at Jmax 9, 100 us at Jmax 14
 // (FP64 Euler), 1.5 ms at Jmax 18.
-constexpr int FIN_CH = 512, FIN_CAP = 896;  // finest cells of a block; positions of all its windows: 512 + 22 * 14 at most
+// CH: 128 cells up to Jmax 16, so that an instance of Jmax 14 fills 128 SMs (its
+// FP64 sums would take 24 us on 32), 512 beyond, where a block's margins would
+// double its reads.  Windows: CH + 22 * 14 positions at most.
 
-template <typename T, int NF>
-__global__ void __launch_bounds__(256) mr_finest(const InstDesc *desc, const Tables<T> *tabs, double *out) {
+template <typename T, int NF, int CH>
+__global__ void __launch_bounds__(CH == 128 ? 128 : 256) mr_finest(const InstDesc *desc, const Tables<T> *tabs, double *out) {
     constexpr bool DQ = NF >= 4;
     constexpr int q = DQ ? (NF == 4 ? 3 : 5) : 2 * NF, nf = DQ ? 2 : NF;
-    __shared__ T val[FIN_CAP * q];
-    __shared__ unsigned char have[FIN_CAP];
-    __shared__ int wa[MAXLEV + 1], woff[MAXLEV + 2];  // first position of a level's window, its place in val
+    constexpr int CAP = CH + 320, NT = CH == 128 ? 128 : 256, R = CH / NT;
+    __shared__ T val[CAP * q];
+    __shared__ unsigned char have[CAP];
+    __shared__ int wa[MAXLEV + 1], woff[32];  // first position of a level's window, its place in val; woff[31]: all of them
     const InstDesc &d = *desc;
     const int Jmin = d.Jmin, Jmax = d.Jmax, bc = d.bc, g = d.gamma, tid = threadIdx.x;
     const int N = 1 << Jmax;
-    const int ch = min(FIN_CH, N), c0 = blockIdx.x * ch;
+    const int ch = min(CH, N), c0 = blockIdx.x * ch;
     const T *V = (const T *)d.V - (1LL << Jmin) * q;
     const uint32_t *I = d.masks + (long long)d.st->cur * d.Wtot;
-    if (tid == 0) {
-        int a = c0, b = c0 + ch - 1, o = 0;
-        for (int l = Jmax - 1; l >= Jmin; --l) {
-            a = (a >> 1) - g;
-            b = (b >> 1) + g;
+    // this thread's finest cells: their tree bits and values on their way while
+    // the windows are built
+    uint32_t word[R];
+    T f[R][q];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int k = min(c0 + tid + NT * r, N - 1);
+        word[r] = Jmax > Jmin ? __ldg(&I[(uint32_t)(N + k) >> 6]) : FULL;
+#pragma unroll
+        for (int j = 0; j < q; ++j) f[r][j] = __ldg(&V[(size_t)(N + k) * q + j]);
+    }
+    if (tid < 32) {
+        // Parents of [a, b] and g cells on either side, from level to level: a + 2g
+        // and b - 2g are halved.  Lane i holds level Jmax - 1 - i.
+        const int l = Jmax - 1 - tid;
+        int n = 0;
+        if (l >= Jmin) {
+            const int a = ((c0 + 2 * g) >> (tid + 1)) - 2 * g, b = ((c0 + ch - 1 - 2 * g) >> (tid + 1)) + 2 * g;
             wa[l] = a;
-            woff[l] = o;
-            o += b - a + 1;
+            n = b - a + 1;
         }
-        woff[MAXLEV + 1] = o;
+        int x = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, x, o);
+            if (tid >= o) x += y;
+        }
+        if (l >= Jmin) woff[l] = x - n;
+        if (tid == 31) woff[31] = x;
     }
     __syncthreads();
-    const int total = Jmax > Jmin ? woff[MAXLEV + 1] : 0;
+    const int total = woff[31];
     // position x of level l: wrapped, or the boundary cell beyond a copy boundary
     auto inside = [&](int x, int l) -> int { return bc == 0 ? (x & ((1 << l) - 1)) : min(max(x, 0), (1 << l) - 1); };
-    for (int i = tid; i < total; i += 256) {
+    for (int i = tid; i < total; i += NT) {
+        // the coarsest level whose window starts at or before i (the finest is first)
         int l = Jmax - 1;
-        while (l > Jmin && i >= woff[l - 1]) --l;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (l - o >= Jmin && woff[l - o] <= i) l -= o;
         const uint32_t h = (1u << l) + (uint32_t)inside(wa[l] + i - woff[l], l);
-        const uint32_t word = __ldg(&I[h >> 6]);
+        const uint32_t bits = __ldg(&I[h >> 6]);
         const T *p = V + (size_t)h * q;
 #pragma unroll
         for (int j = 0; j < q; ++j) val[i * q + j] = __ldg(&p[j]);
-        have[i] = (unsigned char)((word >> ((h >> 1) & 31u)) & 1u);
+        have[i] = (unsigned char)((bits >> ((h >> 1) & 31u)) & 1u);
     }
     __syncthreads();
     const T *c = tabs->pc[g];
@@ -75,39 +100,39 @@ __global__ void __launch_bounds__(256) mr_finest(const InstDesc *desc, const Tab
         if (g > 2) t = t + c3 * (w[3 * q] - w[-3 * q]);
         return (x & 1) ? w[0] - t : w[0] + t;
     };
+    // a thread takes one population of a cell: a level is one short chain
+    const int ci = tid / q, j = tid - ci * q;
+    constexpr int CPB = NT / q;
     for (int l = Jmin + 1; l < Jmax; ++l) {
         const int o = woff[l], n = woff[l - 1] - o;
-        for (int i = tid; i < n; i += 256)
-            if (!have[o + i]) {
-                const int x = bc == 0 ? wa[l] + i : inside(wa[l] + i, l);
-#pragma unroll
-                for (int j = 0; j < q; ++j) val[(o + i) * q + j] = predicted(x, l, j);
-            }
+        if (ci < CPB)
+            for (int i = ci; i < n; i += CPB)
+                if (!have[o + i]) {
+                    const int x = bc == 0 ? wa[l] + i : inside(wa[l] + i, l);
+                    val[(o + i) * q + j] = predicted(x, l, j);
+                }
         __syncthreads();
     }
-    for (int k = c0 + tid; k < c0 + ch; k += 256) {
-        const uint32_t h = (uint32_t)(N + k);
-        T f[q];
-        if (Jmax == Jmin || bit_of(I, h >> 1)) {
-            const T *p = V + (size_t)h * q;
 #pragma unroll
-            for (int j = 0; j < q; ++j) f[j] = p[j];
-        } else {
+    for (int r = 0; r < R; ++r) {
+        const int k = c0 + tid + NT * r;
+        if (k >= c0 + ch) break;
+        if (!((word[r] >> (((uint32_t)(N + k) >> 1) & 31u)) & 1u)) {
 #pragma unroll
-            for (int j = 0; j < q; ++j) f[j] = predicted(k, Jmax, j);
+            for (int i = 0; i < q; ++i) f[r][i] = predicted(k, Jmax, i);
         }
         if constexpr (DQ) {
             double m0 = 0.0, m1 = 0.0;
 #pragma unroll
-            for (int j = 0; j < q; ++j) {
-                m0 += (double)f[j];
-                m1 += (dq_w(j) * d.lam) * (double)f[j];
+            for (int i = 0; i < q; ++i) {
+                m0 += (double)f[r][i];
+                m1 += (dq_w(i) * d.lam) * (double)f[r][i];
             }
             out[k] = m0;
             out[(long long)N + k] = m1;
         } else {
 #pragma unroll
-            for (int j = 0; j < nf; ++j) out[(long long)j * N + k] = (double)f[2 * j] + (double)f[2 * j + 1];
+            for (int i = 0; i < nf; ++i) out[(long long)i * N + k] = (double)f[r][2 * i] + (double)f[r][2 * i + 1];
         }
     }
 }
@@ -168,16 +193,18 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
         if (lane == 0) heads[t >> 5] = hb;
     }
     __syncthreads();
-    int nh = 0;  // all heads, listed in order
+    // the heads listed in order: every warp scans the words' counts
+    const int own = lane < INIT_CELLS / 32 ? __popc(heads[lane]) : 0;
+    int upto = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, upto, o);
+        if (lane >= o) upto += y;
+    }
+    const int nh = __shfl_sync(FULL, upto, 31);
     for (int t = tid; t < INIT_CELLS; t += 256) {
         const unsigned hb = heads[t >> 5];
-        int r = 0;
-        nh = 0;
-        for (int w = 0; w < INIT_CELLS / 32; ++w) {
-            const int n = __popc(heads[w]);
-            r += w < (t >> 5) ? n : 0;
-            nh += n;
-        }
+        const int r = __shfl_sync(FULL, upto - own, t >> 5);
         if ((hb >> lane) & 1u) hlist[r + __popc(hb & ((1u << lane) - 1u))] = (unsigned short)t;
     }
     __syncthreads();
@@ -220,12 +247,6 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
 #pragma unroll
             for (int j = 0; j < q; ++j) a[t * q + j] = a[from * q + j];
     }
-    // values to memory from the shared copy, whose layout is theirs: consecutive
-    // threads write consecutive bytes
-    auto put = [&](const T *from, uint32_t h, int cells) {
-        T *to = V + (size_t)h * q;
-        for (int i = tid; i < cells * q; i += 256) to[i] = from[i];
-    };
     // the run's totals, into the interface array (free until the first step)
 #pragma unroll
     for (int j = 0; j < nf; ++j) {
@@ -234,7 +255,13 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
         if (lane == 0) red[j][warp] = m[j];
     }
     __syncthreads();
-    put(a, (uint32_t)(N + c0), ch);
+    // the values from the shared copy, whose layout is theirs, 16 bytes a thread
+    // (a run starts at a multiple of four cells)
+    {
+        uint4 *to = reinterpret_cast<uint4 *>(V + (size_t)(N + c0) * q);
+        const uint4 *from = reinterpret_cast<const uint4 *>(a);
+        for (int i = tid; i < ch * q * (int)sizeof(T) / 16; i += 256) to[i] = from[i];
+    }
     if (tid < nf) {
         double x = red[tid][0];
         for (int w = 1; w < 8 && 32 * w < nh; ++w) x += red[tid][w];
@@ -243,16 +270,14 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
     int l = Jmax - 1;
     for (int n = ch / 2; n >= 1 && l >= Jmin; n >>= 1, --l) {
         const uint32_t h0 = (1u << l) + (uint32_t)(c0 >> (Jmax - l));
-        for (int t = tid; t < n; t += 256) {
-#pragma unroll
-            for (int j = 0; j < q; ++j) {
-                const T x = a[2 * t * q + j], y = a[(2 * t + 1) * q + j];
-                b[t * q + j] = mean_of(x, y);
-            }
-            inner[h0 + t] = h0 + t;
+        for (int e = tid; e < n * q; e += 256) {
+            const int t = e / q, i = t * q + e;  // population e - t q of cell t: its first child's at 2 t q + that
+            const T x = mean_of(a[i], a[i + q]);
+            b[e] = x;
+            V[(size_t)h0 * q + e] = x;
         }
+        for (int t = tid; t < n; t += 256) inner[h0 + t] = h0 + t;
         __syncthreads();
-        put(b, h0, n);
         T *x = a;
         a = b;
         b = x;
@@ -319,7 +344,7 @@ __device__ __forceinline__ void init_cells(const InstDesc &d, int chunk, const d
 __device__ __forceinline__ int variant_of_desc(const InstDesc &d) { return d.eq == 4 ? 4 : d.eq == 5 ? 5 : d.nf; }
 
 template <typename T>
-__global__ void __launch_bounds__(256) mr_init_cells(const InstDesc *descs, const int *chunk_inst, const double *mcons) {
+__global__ void __launch_bounds__(256, 4) mr_init_cells(const InstDesc *descs, const int *chunk_inst, const double *mcons) {
     __shared__ __align__(16) unsigned char smem[sizeof(T) * 6 * (INIT_CELLS + INIT_CELLS / 2) + 3 * 8 * sizeof(double)];
     const int inst = chunk_inst ? chunk_inst[blockIdx.x] : 0;
     const InstDesc &d = descs[inst];
@@ -402,17 +427,23 @@ static cudaError_t init_of(const InstDesc *descs, const int *chunk_inst, int nch
     return cudaGetLastError();
 }
 
+template <typename T, int CH>
+static void finest_go(int var, int grid, const InstDesc *desc, const Tables<T> *tabs, double *out, cudaStream_t s) {
+    constexpr int NT = CH == 128 ? 128 : 256;
+    switch (var) {
+    case 1: mr_finest<T, 1, CH><<<grid, NT, 0, s>>>(desc, tabs, out); break;
+    case 2: mr_finest<T, 2, CH><<<grid, NT, 0, s>>>(desc, tabs, out); break;
+    case 3: mr_finest<T, 3, CH><<<grid, NT, 0, s>>>(desc, tabs, out); break;
+    case 4: mr_finest<T, 4, CH><<<grid, NT, 0, s>>>(desc, tabs, out); break;
+    default: mr_finest<T, 5, CH><<<grid, NT, 0, s>>>(desc, tabs, out); break;
+    }
+}
 template <typename T>
 static cudaError_t finest_of(int var, int Jmax, const InstDesc *desc, const Tables<T> *tabs, double *out, cudaStream_t s) {
-    const int grid = Jmax > 9 ? 1 << (Jmax - 9) : 1;
-    static_assert(FIN_CH == 1 << 9, "finest cells of a block");
-    switch (var) {
-    case 1: mr_finest<T, 1><<<grid, 256, 0, s>>>(desc, tabs, out); break;
-    case 2: mr_finest<T, 2><<<grid, 256, 0, s>>>(desc, tabs, out); break;
-    case 3: mr_finest<T, 3><<<grid, 256, 0, s>>>(desc, tabs, out); break;
-    case 4: mr_finest<T, 4><<<grid, 256, 0, s>>>(desc, tabs, out); break;
-    default: mr_finest<T, 5><<<grid, 256, 0, s>>>(desc, tabs, out); break;
-    }
+    if (Jmax <= 16)
+        finest_go<T, 128>(var, Jmax > 7 ? 1 << (Jmax - 7) : 1, desc, tabs, out, s);
+    else
+        finest_go<T, 512>(var, 1 << (Jmax - 9), desc, tabs, out, s);
     return cudaGetLastError();
 }
 

@@ -890,10 +890,9 @@ struct Worker {
     }
 
     // the populations of every finest cell by the reconstruction operator
-    // (Definition V): internal cells projected, then every cell outside the
-    // tree predicted, level by level
+    // (Definition V): the internal cells hold projections; every cell outside the
+    // tree is predicted, level by level
     __device__ void fill_finest() {
-        upsweep();
         const uint32_t *I = mask(sm.cur);
 #pragma unroll 1
         for (int l = Jmin; l < Jmax; ++l) {
@@ -906,10 +905,10 @@ struct Worker {
     }
 
     // S1 with the reconstructed collision (Section 4.5, eq. reconstructedCollision):
-    // the pre-collision populations are reconstructed on every finest cell;
-    // each warp averages, one leaf at a time, the equilibria of the relaxed
-    // moments over the leaf's 2^dj finest cells (into the interface array, free
-    // until S4); then every leaf relaxes towards those averages.
+    // the pre-collision populations are reconstructed on every finest cell; a
+    // thread (a small leaf) or a warp (a large one) averages the equilibria of the
+    // relaxed moments over the leaf's 2^dj finest cells (into the interface array,
+    // free until S4); then every leaf relaxes towards those averages.
     __device__ __noinline__ void collide_reconstructed() {
         fill_finest();
         constexpr int NR = DQ ? q - 2 : nf;  // relaxed moments
@@ -920,9 +919,28 @@ struct Worker {
         const long long stride = d.N + 1;
         const int nl = sm.nleaf;
 #pragma unroll 1
+        for (int i = tid; i < nl; i += TS) {
+            // a leaf of up to four finest cells (most leaves): one thread
+            const uint32_t hl = leaves[i];
+            const int dj = Jmax - level_of(hl);
+            if (dj > 2) continue;
+            T acc[3] = {T(0), T(0), T(0)};
+#pragma unroll 1
+            for (uint32_t c = hl << dj; c < (hl + 1u) << dj; ++c) {
+                T g[q], meq[3];
+                load_cell(c, g);
+                relaxed_equilibria(g, meq);
+#pragma unroll
+                for (int r = 0; r < NR; ++r) acc[r] = acc[r] + meq[r];
+            }
+#pragma unroll
+            for (int r = 0; r < NR; ++r) Phi[r * stride + i] = acc[r] * pow2m<T>(dj);
+        }
+#pragma unroll 1
         for (int i = warp; i < nl; i += NWARP) {
             const uint32_t hl = leaves[i];
             const int dj = Jmax - level_of(hl);
+            if (dj <= 2) break;  // the leaves are sorted, coarse first
             const uint32_t first = hl << dj, end = first + (1u << dj);
             T acc[3] = {T(0), T(0), T(0)};
 #pragma unroll 1
@@ -986,24 +1004,24 @@ struct Worker {
     __device__ void upsweep() {
         const uint32_t *li = list(L_INT);
         const int ls = Jmin > 6 ? Jmin : 6;
-        constexpr int CPB = TS / q;  // cells of a block pass
+        constexpr int cpb = TS / q;  // cells of a block pass
         const int c = tid / q, j = tid - c * q;
         int l = Jmax - 1;
         if (l >= ls) {
             int b = sm.seg[L_INT][l], e = sm.seg[L_INT][l + 1];
-            uint32_t h = c < CPB && b + c < e ? li[b + c] : 0u;
+            uint32_t h = c < cpb && b + c < e ? li[b + c] : 0u;
 #pragma unroll 1
             for (;;) {
                 const int eb = b;
                 if (h) project_pop(h, j);
 #pragma unroll 1
-                for (int i = b + c + CPB; c < CPB && i < e; i += CPB) project_pop(li[i], j);
+                for (int i = b + c + cpb; c < cpb && i < e; i += cpb) project_pop(li[i], j);
                 const bool some = b < e;
                 --l;
                 if (l >= ls) {
                     e = eb;
                     b = sm.seg[L_INT][l];
-                    h = c < CPB && b + c < e ? li[b + c] : 0u;
+                    h = c < cpb && b + c < e ? li[b + c] : 0u;
                 }
                 if (some) sync();
                 if (l < ls) break;

@@ -458,8 +458,6 @@ static int launch_group(mr_ctx *c, int phases, int nsteps, const int *order, int
     a.tables = c->ws + c->off_tab + (c->fp32() ? sizeof(Tables<double>) : 0);
     a.wide = c->wide ? c->ws + c->off_wide : nullptr;
     a.smem_mask_words = c->mask_cap[kind];
-    int rc = c->cuda(cudaMemsetAsync(a.queue, 0, sizeof(int), stream), "cudaMemsetAsync");
-    if (rc) return rc;
     int grid = std::min(a.n, c->grid[kind]);
     int e = mrg_launch(c->fp32(), c->block, std::max(grid, 1), a, stream, priority);
     ++c->launches;
@@ -746,6 +744,7 @@ mr_status mr_bind(mr_ctx *c, void *ws, size_t bytes, void *stream) {
     if ((rc = c->cuda(cudaMemcpyAsync(c->ws + c->off_desc, dd.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice, s), "upload")))
         return (mr_status)rc;
     if ((rc = c->cuda(cudaMemsetAsync(c->ws + c->off_state, 0, sizeof(InstState) * n, s), "memset"))) return (mr_status)rc;
+    if ((rc = c->cuda(cudaMemsetAsync(c->ws + c->off_queue, 0, sizeof(int) * 16 * NKIND, s), "memset"))) return (mr_status)rc;
     if ((rc = upload_order(c))) return (mr_status)rc;
     std::vector<int> ident(n);
     for (int i = 0; i < n; ++i) ident[i] = i;

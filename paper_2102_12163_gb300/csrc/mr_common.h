@@ -183,7 +183,7 @@ struct LaunchArgs {
     int n;                // instances in this launch
     int nsteps;
     int phases;           // PH_* bits
-    int *queue;           // work-queue counter, zero at launch
+    int *queue;           // work-queue counter, zero at launch and left so
     const void *aux0;     // phase input / output (see the kernel)
     const void *aux1;
     const void *tables;   // Tables<T> in device memory

@@ -175,7 +175,9 @@ struct Thresholds {
     double eps_l[MAXLEV + 1], big_l[MAXLEV + 1];
     float eps_f[MAXLEV + 1], big_f[MAXLEV + 1];
     __device__ __forceinline__ void set(const InstDesc &d, int l) {
-        const double el = ldexp(d.eps, l - d.Jmax), bl = ldexp(el, d.mu_bar + 1);
+        // the powers of two as factors (exact; 2^{l - Jmax}, |l - Jmax| <= 24)
+        const double el = d.eps * __longlong_as_double((long long)(1023 + l - d.Jmax) << 52),
+                     bl = el * __longlong_as_double((long long)(1024 + d.mu_bar) << 52);
         eps_l[l] = el;
         big_l[l] = bl;
         eps_f[l] = (float)el;
@@ -2144,7 +2146,7 @@ __device__ void load_instance(TeamSmem<T> &sm, const InstDesc &dg, int tid) {
     }
     for (int l = tid; l <= MAXLEV; l += TS) {
         sm.th.set(dg, l);
-        sm.dx_l[l] = ldexp(dg.b - dg.a, -l);
+        sm.dx_l[l] = (dg.b - dg.a) * pow2m<double>(l);
     }
     for (int i = tid; i < NSEG * (MAXLEV + 2); i += TS) (&sm.seg[0][0])[i] = (&st.seg[0][0])[i];
     __syncthreads();
@@ -2279,7 +2281,12 @@ __global__ void __launch_bounds__(NT, MINB) mr_persistent(LaunchArgs a) {
         __syncthreads();
         const int idx = bs.idx;
         __syncthreads();
-        if (idx >= a.n) return;
+        if (idx >= a.n) {
+            // every block takes one number past the instances; the last leaves the
+            // queue at zero for the next launch
+            if (threadIdx.x == 0 && idx == a.n + (int)gridDim.x - 1) *a.queue = 0;
+            return;
+        }
         run_team<T, NT, WIDE, KIND == K_SCALAR, SPM>(bs.team, bs.tab, bs.scratch, a, a.descs[a.order[idx]], threadIdx.x, smask,
                                                 a.smem_mask_words);
     }

@@ -204,10 +204,10 @@ struct TeamSmem {
 };
 
 // block-team scratch: scan partials of the warps, and the audit's partial sums
-// (FP64: one a thread up to 256 threads; FP32: a float-float pair a warp)
+// (FP64: one a thread up to 256 threads; FP32: a float-float pair a thread up to 128)
 template <typename T, int NT>
 struct BlockScratch {
-    static constexpr int NPART = sizeof(T) == 4 ? 64 : NT < 256 ? NT : 256;
+    static constexpr int NPART = sizeof(T) == 4 || NT < 256 ? 128 : 256;
     uint32_t scan_w[2][2][32];
     double red[3][NPART];
 };
@@ -818,28 +818,33 @@ struct Worker {
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(FULL, v, o);
         return v;
     }
-    // the same in float-float: one partial per warp
+    // the same in float-float, a pair in a double's room
     __device__ __forceinline__ void team_partials_ff(float (&hi)[3], float (&lo)[3], int n) {
-        float2 *red = reinterpret_cast<float2 *>(&bx.red[0][0]);
+        constexpr int G = TS / NPART;
         if ((tid & ~31) < n)
 #pragma unroll
             for (int j = 0; j < nf; ++j)
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
+                for (int o = G / 2; o > 0; o >>= 1) {
                     const float h2 = __shfl_down_sync(FULL, hi[j], o), l2 = __shfl_down_sync(FULL, lo[j], o);
                     ff_add(hi[j], lo[j], h2, l2);
                 }
-        if ((tid & 31) == 0)
+        if ((tid & (G - 1)) == 0)
 #pragma unroll
-            for (int j = 0; j < nf; ++j) red[j * 32 + (tid >> 5)] = make_float2(hi[j], lo[j]);
+            for (int j = 0; j < nf; ++j) reinterpret_cast<float2 *>(bx.red[j])[tid / G] = make_float2(hi[j], lo[j]);
         sync();
     }
     __device__ __forceinline__ double team_fold_ff(int j) const {
-        const float2 *red = reinterpret_cast<const float2 *>(&bx.red[0][0]);
+        const float2 *red = reinterpret_cast<const float2 *>(bx.red[j]);
         const int lane = tid & 31;
-        float2 v = lane < TS / 32 ? red[j * 32 + lane] : make_float2(0.0f, 0.0f);
+        float2 v = red[lane];
 #pragma unroll
-        for (int o = TS / 64; o > 0; o >>= 1) {
+        for (int k = 32; k < NPART; k += 32) {
+            const float2 y = red[lane + k];
+            ff_add(v.x, v.y, y.x, y.y);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
             const float h2 = __shfl_down_sync(FULL, v.x, o), l2 = __shfl_down_sync(FULL, v.y, o);
             ff_add(v.x, v.y, h2, l2);
         }
@@ -991,23 +996,33 @@ struct Worker {
     }
 
     // ---- S2: projection sweep, fine to coarse (Def. Projection operator) -------
-    // population j of cell h: the mean of its two children's
-    __device__ __forceinline__ void project_pop(uint32_t h, int j) const {
-        T *p = V + (h * (uint32_t)q + (uint32_t)j);
-        const T *c = V + (2u * h * (uint32_t)q + (uint32_t)j);
-        *p = half_of<T>(c[0] + c[q]);
+    // part j of cell h's populations (PP of them): the mean of its two children's
+    static constexpr int PP = sizeof(T) == 4 && q % 2 == 0 ? 2 : 1, NPARTS = q / PP;
+    __device__ __forceinline__ void project_part(uint32_t h, int j) const {
+        T *p = V + (h * (uint32_t)q + (uint32_t)(PP * j));
+        const T *c = V + (2u * h * (uint32_t)q + (uint32_t)(PP * j));
+        if constexpr (PP == 2) {
+            const auto x = *reinterpret_cast<const typename V2<T>::type *>(c), y = *reinterpret_cast<const typename V2<T>::type *>(c + q);
+            typename V2<T>::type m;
+            m.x = half_of<T>(x.x + y.x);
+            m.y = half_of<T>(x.y + y.y);
+            *reinterpret_cast<typename V2<T>::type *>(p) = m;
+        } else {
+            *p = half_of<T>(c[0] + c[q]);
+        }
     }
     // One level per barrier; the levels of at most 32 cells by one warp, without
     // block barriers.  Ends with a barrier.  A thread takes one population of a
     // cell: a level holds some ten cells, and an FP64 instruction costs its warp's
     // quarter of the SM 64 cycles whatever its active lanes, so q cells x
     // populations side by side take one addition's time where a loop over the
-    // populations took q.  The next level's cell is fetched before the barrier.
+    // populations took q.  (FP32 is short of instructions, not of FP64 units: two
+    // populations a thread.)  The next level's cell is fetched before the barrier.
     __device__ void upsweep() {
         const uint32_t *li = list(L_INT);
         const int ls = Jmin > 6 ? Jmin : 6;
-        constexpr int cpb = TS / q;  // cells of a block pass
-        const int c = tid / q, j = tid - c * q;
+        constexpr int cpb = TS / NPARTS;  // cells of a block pass
+        const int c = tid / NPARTS, j = tid - c * NPARTS;
         int l = Jmax - 1;
         if (l >= ls) {
             int b = sm.seg[L_INT][l], e = sm.seg[L_INT][l + 1];
@@ -1015,9 +1030,9 @@ struct Worker {
 #pragma unroll 1
             for (;;) {
                 const int eb = b;
-                if (h) project_pop(h, j);
+                if (h) project_part(h, j);
 #pragma unroll 1
-                for (int i = b + c + cpb; c < cpb && i < e; i += cpb) project_pop(li[i], j);
+                for (int i = b + c + cpb; c < cpb && i < e; i += cpb) project_part(li[i], j);
                 const bool some = b < e;
                 --l;
                 if (l >= ls) {
@@ -1035,9 +1050,9 @@ struct Worker {
 #pragma unroll 1
                 for (l = Jmax - 1 < 5 ? Jmax - 1 : 5; l >= Jmin; --l) {
 #pragma unroll 1
-                    for (int i = tid; i < (q << l); i += 32) {
-                        const uint32_t k = (uint32_t)i / (uint32_t)q, h = (1u << l) + k;
-                        if (bit_of(I, h)) project_pop(h, i - (int)k * q);
+                    for (int i = tid; i < (NPARTS << l); i += 32) {
+                        const uint32_t k = (uint32_t)i / (uint32_t)NPARTS, h = (1u << l) + k;
+                        if (bit_of(I, h)) project_part(h, i - (int)k * NPARTS);
                     }
                     __syncwarp();
                 }
@@ -1883,12 +1898,12 @@ struct Worker {
 #pragma unroll
         for (int h = 1; h < q; ++h) {
             const int w = dq_w(h), a = w < 0 ? -w : w;
-            T acc = T(0);
-#pragma unroll
-            for (int dl = 1; dl <= a; ++dl) {
+            auto across = [&](int dl) {
                 const int eta = w > 0 ? -dl : dl - 1;
-                acc = acc + (phi(finest_at(first + eta))[h] - phi(finest_at(next + eta))[h]);
-            }
+                return phi(finest_at(first + eta))[h] - phi(finest_at(next + eta))[h];
+            };
+            T acc = across(1);
+            if (a == 2) acc = acc + across(2);
             f[h] = f[h] + (w > 0 ? wgt : -wgt) * acc;
         }
     }

@@ -658,7 +658,10 @@ static int configure(mr_ctx *c) {
 //    2.0  89 / 59 / 53 / 44      6.6  123 / 85 / 73 / 123    21    161 / 165 / 225 / 381
 //    3.0  90 / 74 / 57 / 58      9.9  142 / 89 / 108 / 180   27    208 / 229 / 302 / 498
 // FP32, D1Q3 / D1Q5, the wide stencils and the reconstructed collision cross at
-// the same places (FP32 at 6.6: 65 / 44 / 47 / 87).  Alone an instance takes
+// the same places (FP32 at 6.6: 65 / 44 / 47 / 87).  128 threads win only while
+// trees are small: over 512..1024 steps of the batch of 4096, with twice the
+// leaves, eight instances' values an SM no longer fit L1 (FP64 562 / 403 / 444,
+// FP32 270 / 178 / 239 at 128 / 256 / 512), so the rule never takes them.  Alone an instance takes
 // 15.2 us a step with 512 threads against 16.4 and 15.6 with 256 and 1024
 // (Burgers Jmax 13).
 static int default_block(int n, int sms) {
@@ -666,7 +669,7 @@ static int default_block(int n, int sms) {
     if (per_sm <= 1.0) return 512;
     if (per_sm <= 2.6) return 1024;
     if (per_sm <= 6.5) return 512;
-    return per_sm <= 19.0 ? 256 : 128;
+    return 256;
 }
 
 // Processing order of the work queue: by kernel variant group (fast, scalar,

@@ -740,7 +740,21 @@ struct Worker {
         return Jmin > 5 && w < (1u << (Jmin - 5)) ? FULL : 0u;
     }
     __device__ __forceinline__ T *cell(uint32_t h) const { return V + h * (uint32_t)q; }
-    __device__ __forceinline__ T *phi(uint32_t x) const { return (T *)d.Phi + x * (uint32_t)q; }
+    // Interface values at interface x of the finest lattice (0 .. N).  D1Q2^n in
+    // FP32 keeps them in heap order, the interfaces between two cells of one parent
+    // level by level (x = 0 and N in the two places left): those of neighbouring
+    // leaves lie side by side, where in the order of x each had a line of L1 to
+    // itself (batch of 4096 at 256 threads 116 -> 109 us a step, 163 -> 153 over
+    // 1024 steps).  FP64 waits on its units, not on L1: the same order gave the
+    // batch 0.5 % and cost a lone instance 2.6 % in index arithmetic.  D1Q3 / D1Q5
+    // keep finest cells, in the order of x.
+    __device__ __forceinline__ T *phi(uint32_t x) const {
+        if constexpr (!DQ && sizeof(T) == 4) {
+            const uint32_t N = 1u << Jmax;
+            x = x == N ? 0u : (N + x) >> __ffs((int)x);
+        }
+        return (T *)d.Phi + x * (uint32_t)q;
+    }
     __device__ __forceinline__ uint32_t nb(uint32_t h, int a, uint32_t lo) const { return neighbour(h, a, lo, bc); }
 
     // the q populations of cell h in registers; two a load where the cells are

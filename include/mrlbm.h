@@ -250,14 +250,15 @@ mr_status mr_set_order(mr_ctx *ctx, int by_fields);
  * adaptive steps of the context's current state under each launch shape --
  * threads per block 128, 256, 512, 1024 (the cells of a level each block
  * sweeps per pass) with the queue order of mr_set_order -- and keeps the
- * fastest.  Before every trial, and once more at the end, the state is
+ * fastest; 128 threads, whose lead shrinks as the trees grow, only when they
+ * win by more than 8 %.  Before every trial, and once more at the end, the state is
  * restored from scratch: caller-owned device memory of at least
  * mr_workspace_size bytes, which receives a copy of the workspace.  The
  * results are unchanged by the launch shape (every shape computes the same
  * values), so the state after the call equals the state before it.
  * Synchronises the stream; not for use during stream capture.  best_block,
  * best_order (the order in use, as mr_set_order's by_fields) and best_ms (the
- * fastest trial in milliseconds) may be NULL. */
+ * kept shape's trial in milliseconds) may be NULL. */
 mr_status mr_autotune(mr_ctx *ctx, int nsteps, void *scratch, size_t scratch_bytes, int *best_block,
                       int *best_order, float *best_ms);
 

@@ -1133,7 +1133,7 @@ mr_status mr_autotune(mr_ctx *c, int nsteps, void *scratch, size_t scratch_bytes
     const int blocks[4] = {128, 256, 512, 1024};
     const int block0 = c->block, grid0 = c->grid_req;
     int bb = block0;
-    float bt = -1.0f;
+    float bt = -1.0f, narrow = 0.0f;
     auto restore = [&]() { return c->cuda(cudaMemcpyAsync(c->ws, scratch, c->total, cudaMemcpyDeviceToDevice, s), "restore"); };
     for (int ib = 0; ib < 4 && !rc; ++ib) {
         c->block = blocks[ib];
@@ -1147,10 +1147,19 @@ mr_status mr_autotune(mr_ctx *c, int nsteps, void *scratch, size_t scratch_bytes
         if ((rc = c->cuda(cudaEventSynchronize(e1), "cudaEventSynchronize"))) break;
         float ms = 0.0f;
         if ((rc = c->cuda(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime"))) break;
-        if (bt < 0.0f || ms < bt) {
+        if (blocks[ib] == 128) {
+            narrow = ms;
+        } else if (bt < 0.0f || ms < bt) {
             bt = ms;
             bb = c->block;
         }
+    }
+    // 128 threads put eight instances on an SM: their lead over 256 shrinks as the
+    // trees grow past L1 (FP64 batch of 4096: 10 % over the first 20 steps, 7 %
+    // over 64, 20 % behind over 1024), so a trial has to show more than 8 %
+    if (!rc && narrow < 0.92f * bt) {
+        bt = narrow;
+        bb = 128;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

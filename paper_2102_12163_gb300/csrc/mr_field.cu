@@ -147,11 +147,12 @@ __global__ void __launch_bounds__(CH == 128 ? 128 : 256) mr_finest(const InstDes
 // (a ticket, no waiting) projects the levels above the runs, folds the runs'
 // totals in their order and writes the state.  mr_init_details: a warp takes a
 // word of 32 internal cells and writes their KEEP and REF words.
-// What bounds them: FP64 operations of the equilibria and the 3 q of a detail
-// (two lanes a cycle and SM), and for small schemes the traffic, 2 q values
-// written and read per finest cell.  One block per instance took 2.6 ms for the
-// batch of 4096 (FP64) and 11 ms for a lone Euler instance of Jmax = 18 (FP32),
-// and the first adaptation 0.9 ms more for the latter.
+// What bounds them: with data of constant stretches the passes over shared memory
+// and their barriers (issue a quarter of the cycles, DRAM 17 % and 40 % busy); with
+// others the FP64 operations of the equilibria and the 3 q of a detail (two lanes a
+// cycle and SM).  One block per instance took 2.6 ms for the batch of 4096 (FP64)
+// and 11 ms for a lone Euler instance of Jmax = 18 (FP32), and the first adaptation
+// 0.9 ms more for the latter; now about 1.0 ms and 0.05 ms, first decisions included.
 // (x + y) / 2; of two equal values below half the largest double the value
 // itself, without FP64 operations
 __device__ __forceinline__ double mean_of(double x, double y) {

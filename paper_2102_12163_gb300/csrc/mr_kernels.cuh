@@ -303,12 +303,19 @@ __device__ __forceinline__ void eq_consts(const InstDesc &d, T &a, T &b, T &c, T
 // Quotients in FP64 from a reciprocal (P. Markstein, IBM J. Res. Dev. 34(1),
 // 1990): with r = RN(1 / y), q0 = RN(x r) is within one ulp of x / y, the
 // residual x - q0 y is exact in one FMA, and q0 + residual r rounded once is the
-// correctly rounded quotient, bit for bit the division.  Operands near the ends
-// of the exponent range and non-finite values take the division; a zero (a
-// state at rest has many) stays on the short path.
+// correctly rounded quotient, bit for bit the division, as long as the quotient
+// and the residual's last bit are normal numbers.  Other operands and non-finite
+// values take the division; a zero numerator (a state at rest has many) stays on
+// the short path.
+// |x| from 2^-959 to 2^961, or zero: x over a number within 2^+-18 of 1
 __device__ __forceinline__ bool mid_range(double x) {
     const unsigned hi = (unsigned)__double2hiint(x);
     return ((hi >> 20) & 0x7FFu) - 64u < 1920u || ((hi << 1) | (unsigned)__double2loint(x)) == 0u;
+}
+// |x| from 2^-480 to 2^480, or zero: x over another such number
+__device__ __forceinline__ bool half_range(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    return ((hi >> 20) & 0x7FFu) - 543u < 960u || ((hi << 1) | (unsigned)__double2loint(x)) == 0u;
 }
 // exponents within 300 of 1's (or zero): cubes and quotients of such numbers
 // neither overflow nor underflow
@@ -326,7 +333,7 @@ __device__ __forceinline__ double markstein(double x, double y, double r) {
 template <typename T>
 __device__ __forceinline__ T quotient(T x, T y) {
     if constexpr (sizeof(T) == 8) {
-        if (y != 0.0 && mid_range(y) && mid_range(x)) return markstein(x, y, __drcp_rn(y));
+        if (y != 0.0 && half_range(y) && half_range(x)) return markstein(x, y, __drcp_rn(y));
         return __ddiv_rn(x, y);
     } else {
         if (x == 0.0f && y != 0.0f && fabsf(y) < __int_as_float(0x7F800000)) return x * y;  // the zero of the quotient's sign
@@ -375,15 +382,12 @@ __device__ __forceinline__ void equilibria(const InstDesc &d, T eqp, const T *mc
         meq[0] = mc[1];
         if constexpr (sizeof(T) == 8) {
             if constexpr (EXACT) {
-                // the three quotients from one reciprocal: its square, refined
-                // once, is that of rho^2
+                // the two quotients by rho from one reciprocal
                 const double em = A::mul(mc[2], mc[1]), u3 = A::mul(u2, mc[1]);
-                if (mc[0] != 0.0 && mid_range(mc[0]) && mid_range(u2) && mid_range(em) && mid_range(u3)) {
-                    const double r = __drcp_rn(mc[0]), r2 = __dmul_rn(mc[0], mc[0]);
-                    double q2 = __dmul_rn(r, r);
-                    q2 = __fma_rn(__fma_rn(-r2, q2, 1.0), q2, q2);
+                if (mc[0] != 0.0 && half_range(mc[0]) && half_range(u2) && half_range(em)) {
+                    const double r = __drcp_rn(mc[0]);
                     meq[1] = A::add(A::mul(ca, markstein(u2, mc[0], r)), A::mul(cb, mc[2]));
-                    meq[2] = A::add(A::mul(gg, markstein(em, mc[0], r)), A::mul(cc, markstein(u3, r2, q2)));
+                    meq[2] = A::add(A::mul(gg, markstein(em, mc[0], r)), A::mul(cc, quotient<T>(u3, A::mul(mc[0], mc[0]))));
                     return;
                 }
             } else if (mc[0] != 0.0 && cube_range(mc[0]) && cube_range(mc[1]) && cube_range(mc[2])) {

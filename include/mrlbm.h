@@ -85,7 +85,7 @@ typedef enum {
 typedef struct {
     int Jmin, Jmax;   /* 2 <= Jmin <= Jmax <= 24 */
     int gamma;        /* prediction stencil half-width: 1, 2 or 3 */
-    int mu_bar;       /* Harten regularity guess, >= 0 (eq. HartenLossOfRegularity) */
+    int mu_bar;       /* Harten regularity guess, 0..30; mr_run_static: >= 0 (eq. HartenLossOfRegularity) */
     int bc;           /* mr_bc */
     int eq;           /* mr_equilibrium */
     double eps;       /* threshold epsilon (Prop. ErrorControl), >= 0 */

@@ -174,8 +174,13 @@ struct Thresholds {
     float eps_f[MAXLEV + 1], big_f[MAXLEV + 1];
     __device__ __forceinline__ void set(const InstDesc &d, int l) {
         // the powers of two as factors (exact; 2^{l - Jmax}, |l - Jmax| <= 24)
-        const double el = d.eps * __longlong_as_double((long long)(1023 + l - d.Jmax) << 52),
-                     bl = el * __longlong_as_double((long long)(1024 + d.mu_bar) << 52);
+        const double el = d.eps * __longlong_as_double((long long)(1023 + l - d.Jmax) << 52);
+        // 2^{mu_bar + 1} eps_l in factors that are numbers, for any mu_bar
+        // >= 0 (mr_run_static takes all): one factor up to 999; 2101 doublings are
+        // infinity for every positive eps_l
+        double bl = el;
+#pragma unroll 1
+        for (int k = min(d.mu_bar, 2100) + 1; k > 0; k -= 1000) bl *= __longlong_as_double((long long)(1023 + min(k, 1000)) << 52);
         eps_l[l] = el;
         big_l[l] = bl;
         eps_f[l] = (float)el;

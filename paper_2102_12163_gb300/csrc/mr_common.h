@@ -166,7 +166,9 @@ struct Tables {
 // cell of the window is refined, by where the leaf lies: [0] away from a copy
 // boundary, [1 + k] k < 2 gamma cells from the left one, [1 + 2 gamma + r] r from
 // the right one (a window position beyond the boundary stands for the boundary
-// cell).  The last finest cell uses the mirrored window.
+// cell).  The last finest cell uses the mirrored window.  The weights are applied
+// to the differences from the leaf's own value, so the entry of that value (2 gamma)
+// is read for the details of the level below alone.
 template <typename T>
 struct WideTables {
     T w2[9][MAXDJ + 1][9];

@@ -85,17 +85,18 @@ def host_cores():
     return usable, os.cpu_count() or usable
 
 
-def profiled_traffic(workload: str, precision: str, graph_steps: int):
+def profiled_traffic(workload: str, precision: str, graph_steps: int, block: int | None = None):
     """DRAM bytes per leaf update from the committed ncu record
-    (profiles/traffic.json) of a launch of the same number of steps, if it was
-    taken on the current kernel source.  The steps per launch are part of the
-    key because an instance's values stay in L2 between the steps of one launch:
-    the DRAM bytes per update fall as the launch grows."""
+    (profiles/traffic.json) of a launch of the same number of steps and threads
+    per block, if it was taken on the current kernel source.  The steps per
+    launch are part of the key because an instance's values stay in L2 between
+    the steps of one launch: the DRAM bytes per update fall as the launch grows.
+    The threads are, because they set how many instances share an SM and L2."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as fh:
             j = json.load(fh)
-        e = j[f"{workload}:{precision}:g{graph_steps}"]
+        e = j[f"{workload}:{precision}:g{graph_steps}" + (f":b{block}" if block is not None else "")]
         if e.get("source_hash") != source_hash():
             return None
         return e
@@ -655,7 +656,7 @@ def main():
 
     def roof(r, prec):
         achieved = r["bytes_alg"] / r["dt"] / 1e9
-        tr = (profiled_traffic(args.workload, prec, r["graph_steps"])
+        tr = (profiled_traffic(args.workload, prec, r["graph_steps"], r["tune"]["block"])
               if len(insts) == 4096 or args.workload != "batch" else None)
         launches = max(1, r["launches"])
         per_launch_updates = r["updates"] / launches
@@ -671,7 +672,8 @@ def main():
         if tr:
             out["dram_bytes_per_update"] = tr["dram_bytes_per_update"]
             if "fp64_pipe_active_pct" in tr:
-                # GB300's FP64 units are the other roof of this kernel (two FP64 operations per SM per cycle)
+                # GB300's FP64 units are the other roof of this kernel (two FP64 operations per SM per
+                # cycle); counted in a launch of the record's shape
                 out["fp64_pipe_active_pct"] = tr["fp64_pipe_active_pct"]
         return out
 

@@ -37,6 +37,23 @@ def test_traffic_record_is_keyed_by_steps_per_launch_and_kernel_source(tmp_path,
     assert b.profiled_traffic("batch", "fp64", 20) is None
 
 
+def test_traffic_record_belongs_to_one_block_size(tmp_path, monkeypatch):
+    b = _bench()
+    (tmp_path / "paper_2102_12163_gb300" / "csrc").mkdir(parents=True)
+    (tmp_path / "profiles").mkdir()
+    monkeypatch.setattr(b, "ROOT", str(tmp_path))
+    h = b.source_hash()
+    rec = {"batch:fp64:g20": {"dram_bytes_per_update": 1.0, "source_hash": h},
+           "batch:fp64:g20:b128": {"dram_bytes_per_update": 60.0, "source_hash": h},
+           "batch:fp64:g64:b256": {"dram_bytes_per_update": 17.0, "source_hash": h}}
+    (tmp_path / "profiles" / "traffic.json").write_text(json.dumps(rec))
+    assert b.profiled_traffic("batch", "fp64", 20, 128)["dram_bytes_per_update"] == 60.0
+    assert b.profiled_traffic("batch", "fp64", 64, 256)["dram_bytes_per_update"] == 17.0
+    # a launch of another block size has no record, whatever lies under the same steps
+    assert b.profiled_traffic("batch", "fp64", 20, 256) is None
+    assert b.profiled_traffic("batch", "fp64", 64, 128) is None
+
+
 def test_clock_summary_keeps_the_sampled_window_and_every_throttle_reason():
     b = _bench()
     c = b.ClockSampler(0)

@@ -275,11 +275,12 @@ mr_status mr_reconstruction_coefficients(int dj, int kind, double *out);
 
 /* Tracing: SM clock cycles spent by instance inst in each phase of the step,
  * accumulated since its initial state, in the order
- *   projection (adapt), details + threshold, enlargement, grading + marking,
+ *   projection (adapt), details + threshold, enlargement, grading,
  *   grading of the levels of at most 32 cells, candidate mask words, list
  *   compaction, data transfer, collision, projection (step), ghosts,
  *   reconstruction, stream + audit
- * (n >= 13 slots).  Only a library compiled with MRG_PHASE_TIMERS records
+ * (n >= 13 slots; the first and the fifth stay zero: their work is part of
+ * the stream and of the grading).  Only a library compiled with MRG_PHASE_TIMERS records
  * them; otherwise the cycles are zero and MR_ERR_STATE is returned. */
 mr_status mr_phase_times(mr_ctx *ctx, int inst, unsigned long long *cycles, int n);
 

@@ -465,10 +465,11 @@ static int launch_group(mr_ctx *c, int phases, int nsteps, const int *order, int
     return MR_OK;
 }
 
-// A launch over the instances.  The queue order holds up to three groups, each
+// A launch over the instances.  The queue order holds up to four groups, each
 // run by its own kernel variant: the general kernel (gamma = 2, 3), the
-// reconstructed-collision kernel (gamma = 1) and the fast kernel (gamma = 1,
-// leaves collision; the scalar kernel when all of them have one field).  With
+// reconstructed-collision kernel (gamma = 1), and for gamma = 1 with the leaves
+// collision the large-instance kernel (CW_MIN_WORDS words and more) and the fast
+// kernel (the scalar kernel when all of its instances have one field).  With
 // more than one group the groups alternate between the context's stream and a
 // side stream that forks from it and joins it again, so a group's kernel can
 // fill the SMs the previous one's tail leaves idle.  Launch priorities (earlier
@@ -657,8 +658,11 @@ static int configure(mr_ctx *c) {
 //    1.0  64 / 41 / 38 / 38      4.6  105 / 82 / 56 / 87     14.5  149 / 115 / 157 / 264
 //    2.0  89 / 59 / 53 / 44      6.6  123 / 85 / 73 / 123    21    161 / 165 / 225 / 381
 //    3.0  90 / 74 / 57 / 58      9.9  142 / 89 / 108 / 180   27    208 / 229 / 302 / 498
-// FP32, D1Q3 / D1Q5, the wide stencils and the reconstructed collision cross at
-// the same places (FP32 at 6.6: 65 / 44 / 47 / 87).  128 threads win only while
+// The other calls measured lie on the same side of the lines: D1Q3 / D1Q5 at 5.1
+// 91 / 74 / 66 / 111, gamma = 3 at 2.0 172 / 140 / 119 / 92, reconstructed
+// collision at 1.3 95 / 62 / 49 / 44.  From 512 to 256 threads FP32 crosses near 6
+// (at 6.6: 65 / 44 / 47 / 87) and FP64 near 8; the one line at 6.5 lies between, and
+// costs FP64 up to 16 % from there to 8.  128 threads win only while
 // trees are small: over 512..1024 steps of the batch of 4096, with twice the
 // leaves, eight instances' values an SM no longer fit L1 (FP64 562 / 403 / 444,
 // FP32 270 / 178 / 239 at 128 / 256 / 512), so the rule never takes them.  Alone an instance takes

@@ -40,7 +40,9 @@ enum { PH_INIT_STATE = 2, PH_ADAPT = 4, PH_STEP = 8 };
 // ST_DETAILS: KEEP and REF hold the decisions of the initial state, for the
 // first adaptation (mr_set_initial takes them over the whole GPU)
 enum { ST_NONFINITE = 1, ST_DETAILS = 2 };
-// phases timed by the profiling build (MRG_PHASE_TIMERS)
+// phases timed by the profiling build (MRG_PHASE_TIMERS); T_UPSWEEP_A and
+// T_GRADE_SMALL keep their places in mr_phase_times and stay zero (the stream moves
+// the projections, the grading takes every level)
 enum {
     T_UPSWEEP_A = 0, T_DETAILS, T_ENLARGE, T_GRADE, T_GRADE_SMALL, T_CANDIDATES, T_LISTS, T_TRANSFER,
     T_COLLIDE, T_UPSWEEP_S, T_GHOSTS, T_RECON, T_STREAM, NPHASE
@@ -167,8 +169,7 @@ struct Tables {
 // boundary, [1 + k] k < 2 gamma cells from the left one, [1 + 2 gamma + r] r from
 // the right one (a window position beyond the boundary stands for the boundary
 // cell).  The last finest cell uses the mirrored window.  The weights are applied
-// to the differences from the leaf's own value, so the entry of that value (2 gamma)
-// is read for the details of the level below alone.
+// to the differences from the leaf's own value, whose entry (2 gamma) is not read.
 template <typename T>
 struct WideTables {
     T w2[9][MAXDJ + 1][9];

@@ -818,7 +818,7 @@ struct Worker {
     // eight a lane and shuffles.  Warps without a leaf (the first n threads have
     // one) only write their zeros.  A fixed order: deterministic.
     __device__ __forceinline__ void team_partials(double (&x)[3], int n) {
-        constexpr int G = TS / NPART;  // lanes per partial sum: 1, 2 or 4
+        constexpr int G = TS / NPART;  // lanes per partial sum: 1, 2, 4, or 8 (FP32 at 1024 threads)
         if ((tid & ~31) < n)
 #pragma unroll
             for (int j = 0; j < nf; ++j)
@@ -936,7 +936,9 @@ struct Worker {
     // the pre-collision populations are reconstructed on every finest cell; a
     // thread (a small leaf) or a warp (a large one) averages the equilibria of the
     // relaxed moments over the leaf's 2^dj finest cells (into the interface array,
-    // free until S4); then every leaf relaxes towards those averages.
+    // free until S4); then every leaf relaxes towards those averages.  A barrier has
+    // to lie between a step and this: the end of a step's audit still reads the
+    // interface array (an adaptation has many; without one a launch holds one step).
     __device__ __noinline__ void collide_reconstructed() {
         fill_finest();
         constexpr int NR = DQ ? q - 2 : nf;  // relaxed moments

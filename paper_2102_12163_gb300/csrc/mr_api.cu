@@ -85,6 +85,7 @@ int variant_of(int eq) { return eq == MR_EQ_SW_D1Q3 ? 4 : eq == MR_EQ_SW_D1Q5 ? 
 // gamma = 1 instances with the leaves collision (fast kernel, or the scalar
 // kernel when every instance of the group has one field).
 constexpr int NGROUP = 4;
+constexpr int kGroupKind[NGROUP] = {K_GENERAL, K_RECOLL, K_LARGE, K_FAST};  // the last may run as K_SCALAR
 int group_of(const InstDesc &h) {
     return h.gamma > 1 ? 0 : h.collision != 0 ? 1 : h.Wtot >= CW_MIN_WORDS ? 2 : 3;
 }
@@ -162,7 +163,7 @@ struct mr_ctx {
     int mask_cap[NKIND] = {};  // mask-region words a block team keeps in shared memory, by variant
     int wmax = 0;              // mask-region words of the largest instance
     int n_group[NGROUP] = {};  // instances per group of the queue order (group_of)
-    int group_kind[NGROUP] = {K_GENERAL, K_RECOLL, K_LARGE, K_FAST};  // kernel variant of each group
+    int group_kind[NGROUP] = {kGroupKind[0], kGroupKind[1], kGroupKind[2], kGroupKind[3]};  // kernel variant of each group
     // The groups run as separate kernels; a second stream lets one group's
     // kernel fill the SMs that another's tail leaves idle (fork and join by events).
     cudaStream_t side = nullptr;
@@ -649,6 +650,39 @@ static int configure(mr_ctx *c) {
     return MR_OK;
 }
 
+// Relative length of a step of one instance: its levels are the dependent passes,
+// its populations their work; the reconstructed collision visits every finest cell.
+static double step_cost(const InstDesc &h) {
+    return (h.Jmax - h.Jmin + 1 + (h.collision ? std::ldexp(1.0, h.Jmax - 6) : 0.0)) * (npop_of(h.eq) + 2);
+}
+// Estimated time of a step of the instances with blocks of that many threads, in
+// the same units.  Of j m + 1 instances some of m resident blocks takes j + 1: the
+// (j m + 1)-th longest bounds the time j + 1 times; so does the mean.  Instances
+// that share an SM slow each other down by about a quarter each.
+static double wave_time(const std::vector<InstDesc> &dd, bool fp32, int block, int sms) {
+    double total = 0.0;
+    for (int g = 0; g < NGROUP; ++g) {
+        std::vector<double> cost;
+        bool scalar = true;
+        for (const InstDesc &h : dd)
+            if (group_of(h) == g) {
+                cost.push_back(step_cost(h));
+                scalar = scalar && variant_of(h.eq) == 1;
+            }
+        if (cost.empty()) continue;
+        std::sort(cost.begin(), cost.end(), [](double x, double y) { return x > y; });
+        const int kind = g == 3 && scalar ? K_SCALAR : kGroupKind[g], n = (int)cost.size();
+        const int resident = std::max(1, mrg_min_blocks(fp32, block, kind)), m = resident * sms;
+        double t = 0.0, sum = 0.0;
+        for (int i = 0; i < n; ++i) {
+            sum += cost[i];
+            if (i % m == 0) t = std::max(t, (i / m + 1) * cost[i]);
+        }
+        total += std::max(t, sum / m) * (1.0 + 0.25 * (std::min(resident, (n + sms - 1) / sms) - 1));
+    }
+    return total;
+}
+
 // Threads per block unless the caller or the autotuner chose them.  An SM holds
 // about 1024 threads of the kernels, so 1024 / threads instances at once; wide
 // blocks finish an instance sooner, narrow ones keep more of them in flight.
@@ -668,12 +702,43 @@ static int configure(mr_ctx *c) {
 // FP32 270 / 178 / 239 at 128 / 256 / 512), so the rule never takes them.  Alone an instance takes
 // 15.2 us a step with 512 threads against 16.4 and 15.6 with 256 and 1024
 // (Burgers Jmax 13).
-static int default_block(int n, int sms) {
-    const double per_sm = (double)n / std::max(1, sms);
-    if (per_sm <= 1.0) return 512;
-    if (per_sm <= 2.6) return 1024;
-    if (per_sm <= 6.5) return 512;
-    return 256;
+//
+// That holds for uneven instances.  Of even ones a second wave is as long as the
+// first: 200 to 304 of one size took twice the time with 1024 threads that they
+// take with 512, and 305 to 608 with 512 that they take with 256.  So narrower
+// blocks, down to 256 threads, replace the line's where an estimate of the waves
+// (wave_time) is shorter by a fifth.  us per step, line / now, FP64 and FP32:
+// Burgers Jmax 8 n = 200 20.4 / 10.6 and 15.5 / 8.5, n = 600 20.7 / 12.2 and
+// 16.1 / 8.6; Euler Jmax 11 n = 200 47 / 30 and 27 / 14, n = 600 58 / 45 and 29 / 17.
+// Estimates between 0.8 and 1 went both ways (0.86: 66 / 74; 0.93: 60 / 88 and 41 / 30).
+// A lone instance with eps = 0 keeps every cell: from Jmax 12 on the widest block
+// (Burgers, 512 / 1024 threads: Jmax 11 30.7 / 31.7 in FP64, 26.6 / 25.1 in FP32;
+// Jmax 12 58.7 / 55.9 and 47.4 / 44.2; Jmax 14 225 / 207 and 210 / 174).
+static int default_block(const std::vector<InstDesc> &dd, bool fp32, int sms) {
+    const int n = (int)dd.size();
+    sms = std::max(1, sms);
+    const double per_sm = (double)n / sms;
+    if (n == 1) return dd[0].eps == 0.0 && dd[0].Jmax >= 12 ? 1024 : 512;
+    if (per_sm > 6.5) return 256;
+    int b = per_sm <= 1.0 ? 512 : per_sm <= 2.6 ? 1024 : 512;
+    for (int x = b / 2; x >= 256; x /= 2)
+        if (wave_time(dd, fp32, x, sms) < 0.8 * wave_time(dd, fp32, b, sms)) b = x;
+    return b;
+}
+
+// The rule for a batch of n descriptions on a GPU of that many SMs (host only).
+extern "C" int mrg_default_block(const mr_instance_desc *desc, int n, int precision, int sms) {
+    std::vector<InstDesc> dd(n);
+    for (int i = 0; i < n; ++i) {
+        dd[i].Jmin = desc[i].Jmin;
+        dd[i].Jmax = desc[i].Jmax;
+        dd[i].gamma = desc[i].gamma;
+        dd[i].collision = desc[i].collision;
+        dd[i].eq = desc[i].eq;
+        dd[i].eps = desc[i].eps;
+        dd[i].Wtot = mask_words_of(desc[i].Jmax);
+    }
+    return default_block(dd, precision == MR_FP32_MIXED, sms);
 }
 
 // Processing order of the work queue: by kernel variant group (fast, scalar,
@@ -742,7 +807,7 @@ mr_status mr_bind(mr_ctx *c, void *ws, size_t bytes, void *stream) {
         dd[i].lists = (uint32_t *)(base + (size_t)dd[i].lists);
         dd[i].st = (InstState *)(c->ws + c->off_state) + i;
     }
-    if (c->block == 0) c->block = default_block(n, c->sms);
+    if (c->block == 0) c->block = default_block(dd, c->fp32(), c->sms);
     c->hdesc = dd;
     Tables<double> td;
     Tables<float> tf;

@@ -20,6 +20,9 @@
 #include "../../include/mrlbm.h"
 #include "mr_common.h"
 
+// threads per block unless the caller chose them (mr_api.cu)
+extern "C" int mrg_default_block(const mr_instance_desc *desc, int n, int precision, int sms);
+
 using namespace mrg;
 
 namespace {
@@ -198,8 +201,9 @@ extern "C" mr_status mr_run_static(const mr_instance_desc *desc, int precision, 
     if (e == cudaSuccess && wide_bytes) e = cudaMemcpyAsync(base + oWide, mrg_wide_tables(fp32), wide_bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail(MR_ERR_CUDA, "mr_run_static: upload failed (%lld)", (long long)e);
 
-    // one block for the instance, bitmasks in shared memory when they fit
-    const int block = 512;
+    // one block for the instance, bitmasks in shared memory when they fit; threads as
+    // for a lone instance of a context
+    const int block = mrg_default_block(&d, 1, precision, 1);
     size_t sbase = mrg_smem_bytes(fp32, block, 0), limit = 220u * 1024u;
     long long fit = limit > sbase ? (long long)((limit - sbase) / sizeof(uint32_t)) : 0;
     LaunchArgs a;

@@ -1747,10 +1747,10 @@ struct Worker {
     // the weights' rounding and the sum's count for the differences alone.  Random
     // windows in FP32, rms error in units of 2^-24 at gaps 1 / 2 / 8, gamma = 3:
     // 0.46 / 0.48 / 0.55, the walk 0.46 / 0.72 / 1.44, the weights on the values
-    // themselves 0.93 / 1.05 / 1.39.  The subtractions cost a call of 300 instances
-    // 2 % in FP64 (4.13 against 4.05 ms) and nothing in FP32; a chain of products a
-    // side of the window gained nothing.
-    // Gap 1 is the predicted child by the exact coefficients.
+    // themselves 0.93 / 1.05 / 1.39.  The subtractions cost 3 to 5 % of a gamma = 3
+    // step in FP64 (batch of 300: 87.3 -> 89.9 us), 1 to 3 % with gamma = 2 and up to
+    // 3 % in FP32; a chain of products a side of the window gained nothing.
+    // Gap 1 is the predicted child by the exact coefficients (by the tables: 95 us).
     template <int G>
     __device__ __noinline__ void reconstruct_wide() {
         constexpr int C = 2 * G, W = 4 * G + 1;

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(CH == 128 ? 128 : 256) mr_finest(const InstDes
 // totals in their order and writes the state.  mr_init_details: a warp takes a
 // word of 32 internal cells and writes their KEEP and REF words.
 // What bounds them: with data of constant stretches the passes over shared memory
-// and their barriers (issue a quarter of the cycles, DRAM 17 % and 40 % busy); with
+// and their barriers (issue a third of the cycles, DRAM 24 % and 40 % busy); with
 // others the FP64 operations of the equilibria and the 3 q of a detail (two lanes a
 // cycle and SM).  One block per instance took 2.6 ms for the batch of 4096 (FP64)
 // and 11 ms for a lone Euler instance of Jmax = 18 (FP32), and the first adaptation
